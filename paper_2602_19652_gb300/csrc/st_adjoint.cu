@@ -472,51 +472,74 @@ __global__ void k_chain_jacobians(const uint32_t* idx, const uint32_t* count, in
     }
 }
 
-// direct path: one thread per microphone, sequential over bins
-__global__ void k_direct_adjoint(const DirectAccumArgs a, const float* qhi, const float* qlo, const float2* G,
-                                 float* mic_out, float* emit_out) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= a.M) return;
-    float gx = 0.f, gy = 0.f, gz = 0.f;
-    if (a.vis[m]) {
-        const float mx = a.mics[3 * m], my = a.mics[3 * m + 1], mz = a.mics[3 * m + 2];
-        const ff r = dist_ff(mx, my, mz, a.s[0], a.s[1], a.s[2]);
-        float dLdr = 0.0f;
-        for (int k = 0; k < a.F; ++k) {
-            const double f = a.F == 1 ? a.f_lo : a.f_lo + (double)k * a.df;
-            const float alpha = (float)(a.a0 + a.a1 * (f / 1000.0));
-            const float L = log2f(a.gain) - 2.0f * log2_ff(r) - alpha * r.hi * (3.3219280948873623f / 20.0f);
-            const ff x = ff_mul(r, ff{qhi[k], qlo[k]});
-            float sn, cs;
-            sincospif(2.0f * ff_frac(x), &sn, &cs);
-            const float A = exp2f(L);
-            const float Tr = A * cs, Ti = A * sn;
-            const float2 gk = G[(int64_t)m * a.F + k];
-            const float wr = gk.x * Tr + gk.y * Ti, wi = gk.x * Ti - gk.y * Tr;
-            const float dr = -2.0f / r.hi - alpha * (2.302585092994046f / 20.0f);
-            const float di = (float)(2.0 * 3.141592653589793 * f / a.c);
-            dLdr += dr * wr - di * wi;
-        }
-        const float iv = 1.0f / r.hi;
-        gx = dLdr * (mx - a.s[0]) * iv;
-        gy = dLdr * (my - a.s[1]) * iv;
-        gz = dLdr * (mz - a.s[2]) * iv;
+// Direct path: one block per microphone, its threads over the bins, their sums added in a fixed-order tree.
+// Bound by the float64 steps of each bin (frequency, wavenumber): one thread per microphone walked all bins in
+// sequence (32 microphones x 512 bins: 443 us, the longest launch of a small backward pass after the specular
+// adjoint); spread over the threads a bin costs each of them a few float64 instructions.
+constexpr int kDirThreads = 128;
+__global__ void __launch_bounds__(kDirThreads) k_direct_adjoint(const DirectAccumArgs a, const float* qhi,
+                                                               const float* qlo, const float2* G, float* mic_out,
+                                                               float* emit_out) {
+    __shared__ float red[kDirThreads];
+    const int m = blockIdx.x;
+    const bool vis = a.vis[m] != 0;
+    const float mx = a.mics[3 * m], my = a.mics[3 * m + 1], mz = a.mics[3 * m + 2];
+    const ff r = dist_ff(mx, my, mz, a.s[0], a.s[1], a.s[2]);
+    float dLdr = 0.0f;
+    for (int k = threadIdx.x; vis && k < a.F; k += kDirThreads) {
+        const double f = a.F == 1 ? a.f_lo : a.f_lo + (double)k * a.df;
+        const float alpha = (float)(a.a0 + a.a1 * (f / 1000.0));
+        const float L = log2f(a.gain) - 2.0f * log2_ff(r) - alpha * r.hi * (3.3219280948873623f / 20.0f);
+        const ff x = ff_mul(r, ff{qhi[k], qlo[k]});
+        float sn, cs;
+        sincospif(2.0f * ff_frac(x), &sn, &cs);
+        const float A = exp2f(L);
+        const float Tr = A * cs, Ti = A * sn;
+        const float2 gk = G[(int64_t)m * a.F + k];
+        const float wr = gk.x * Tr + gk.y * Ti, wi = gk.x * Ti - gk.y * Tr;
+        const float dr = -2.0f / r.hi - alpha * (2.302585092994046f / 20.0f);
+        const float di = (float)(2.0 * 3.141592653589793 * f / a.c);
+        dLdr += dr * wr - di * wi;
     }
-    mic_out[3 * m] = gx;
-    mic_out[3 * m + 1] = gy;
-    mic_out[3 * m + 2] = gz;
-    emit_out[3 * m] = -gx;
-    emit_out[3 * m + 1] = -gy;
-    emit_out[3 * m + 2] = -gz;
+    red[threadIdx.x] = dLdr;
+    __syncthreads();
+    for (int h = kDirThreads / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x < 3) {
+        const int c = threadIdx.x;
+        float g = 0.0f;
+        if (vis) {
+            const float iv = 1.0f / r.hi;
+            g = red[0] * ((c == 0 ? mx : c == 1 ? my : mz) - a.s[c]) * iv;
+        }
+        mic_out[3 * m + c] = g;
+        emit_out[3 * m + c] = -g;
+    }
 }
 
-// V[u][k] = sum of the partial slices in order (one thread per (u, k)), written to slice 0's place
-__global__ void k_v_reduce(float* v_part, int n_slices, int F) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= kNV * F) return;
+// V[u][k] = sum of the partial slices, written to slice 0's place: a block takes 32 neighbouring (u, k), its rows
+// of threads every 16th slice each, the rows' sums added in row order (only the block itself reads those places of
+// slice 0, before it writes them).  One thread per (u, k) ran a chain of n_slices loads: 20 us at 128 bins x 304
+// slices.
+constexpr int kVRows = 16;
+__global__ void __launch_bounds__(32 * kVRows) k_v_reduce(float* v_part, int n_slices, int F) {
+    __shared__ float rows[kVRows][33];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int idx = blockIdx.x * 32 + x;
     float acc = 0.0f;
-    for (int sl = 0; sl < n_slices; ++sl) acc += v_part[(size_t)sl * kNV * F + idx];
-    v_part[idx] = acc;
+    if (idx < kNV * F) {
+#pragma unroll 4
+        for (int sl = y; sl < n_slices; sl += kVRows) acc += v_part[(size_t)sl * kNV * F + idx];
+    }
+    rows[y][x] = acc;
+    __syncthreads();
+    if (y == 0 && idx < kNV * F) {
+#pragma unroll
+        for (int r = 1; r < kVRows; ++r) acc += rows[r][x];
+        v_part[idx] = acc;
+    }
 }
 
 // dk[mat][b] = sum_k V[mat][k] w_b(k) / k(mat, f_k) over the bins whose interpolation uses band b.
@@ -619,19 +642,27 @@ __global__ void __launch_bounds__(kDkThreads) k_dbeta_contract(const float* V, i
     if (threadIdx.x == 0) dbeta[(size_t)mat * n_bands + b] = (float)red[0];
 }
 
-// positions: dmic[m] = sum of all partial slices in order; demit = sum of emitter slices in order
-__global__ void k_pos_reduce(const float* mic_parts, int n_mic_slices, const float* emit_parts, int n_emit_slices,
-                             int M, float* dmic, float* demit) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < 3 * M) {
-        float acc = 0.0f;
-        for (int sl = 0; sl < n_mic_slices; ++sl) acc += mic_parts[(size_t)sl * M * 3 + idx];
+// positions: dmic[m] = sum of all partial slices; demit = sum of the emitter slices.  One warp per output, its
+// lanes over the slices, then a fixed-order tree (one thread per output ran a chain of all the slices' loads:
+// 15 us at 32 microphones x 305 slices)
+__global__ void __launch_bounds__(128) k_pos_reduce(const float* mic_parts, int n_mic_slices, const float* emit_parts,
+                                                    int n_emit_slices, int M, float* dmic, float* demit) {
+    const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (idx >= 3 * M + 3) return;
+    const bool mic = idx < 3 * M;
+    const float* src = mic ? mic_parts + idx : emit_parts + (idx - 3 * M);
+    const size_t step = mic ? (size_t)M * 3 : 3;
+    const int n = mic ? n_mic_slices : n_emit_slices;
+    float acc = 0.0f;
+#pragma unroll 4
+    for (int sl = lane; sl < n; sl += 32) acc += src[(size_t)sl * step];
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, h);
+    if (lane != 0) return;
+    if (mic) {
         if (dmic) dmic[idx] = acc;
-    } else if (idx < 3 * M + 3) {
-        const int c = idx - 3 * M;
-        float acc = 0.0f;
-        for (int sl = 0; sl < n_emit_slices; ++sl) acc += emit_parts[(size_t)sl * 3 + c];
-        if (demit) demit[c] = acc;
+    } else if (demit) {
+        demit[idx - 3 * M] = acc;
     }
 }
 
@@ -714,7 +745,7 @@ cudaError_t adjoint_direct(const DirectAccumArgs& a, const float* qhi, const flo
                            float* mic_out, float* emit_out, cudaStream_t s) {
     if (a.M <= 0) return cudaSuccess;
     note_launch();
-    k_direct_adjoint<<<(a.M + 63) / 64, 64, 0, s>>>(a, qhi, qlo, G, mic_out, emit_out);
+    k_direct_adjoint<<<a.M, kDirThreads, 0, s>>>(a, qhi, qlo, G, mic_out, emit_out);
     return cudaGetLastError();
 }
 
@@ -726,7 +757,7 @@ cudaError_t adjoint_dk(const float* v_part, int n_slices, int F, int mat_base, i
     if (n <= 0) return cudaSuccess;
     float* v = const_cast<float*>(v_part);
     note_launch();
-    k_v_reduce<<<(kNV * F + 127) / 128, 128, 0, s>>>(v, n_slices, F);
+    k_v_reduce<<<(kNV * F + 31) / 32, 32 * kVRows, 0, s>>>(v, n_slices, F);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     note_launch();
@@ -751,7 +782,7 @@ cudaError_t adjoint_dbeta(const float* v_part, int n_slices, int F, int mat_base
     if (n <= 0) return cudaSuccess;
     float* v = const_cast<float*>(v_part);
     note_launch();
-    k_v_reduce<<<(kNV * F + 127) / 128, 128, 0, s>>>(v, n_slices, F);
+    k_v_reduce<<<(kNV * F + 31) / 32, 32 * kVRows, 0, s>>>(v, n_slices, F);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     note_launch();
@@ -762,7 +793,7 @@ cudaError_t adjoint_dbeta(const float* v_part, int n_slices, int F, int mat_base
 cudaError_t adjoint_pos(const float* mic_parts, int n_mic_slices, const float* emit_parts, int n_emit_slices, int M,
                         float* dmic, float* demit, cudaStream_t s) {
     note_launch();
-    k_pos_reduce<<<(3 * M + 3 + 127) / 128, 128, 0, s>>>(mic_parts, n_mic_slices, emit_parts, n_emit_slices, M, dmic,
+    k_pos_reduce<<<(3 * M + 3 + 3) / 4, 128, 0, s>>>(mic_parts, n_mic_slices, emit_parts, n_emit_slices, M, dmic,
                                                         demit);
     return cudaGetLastError();
 }

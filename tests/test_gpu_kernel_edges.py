@@ -1,0 +1,65 @@
+"""GPU kernels at the sizes where their tiling can go wrong (tile edges, remainders, the smallest shapes),
+against the oracle.  Tolerances: spectra 1e-4 and gradients 1e-3 relative L2, the parity tests' bars (float32
+amplitudes ~1e-6, float-float phases, at most 18 recurrence steps); path sets and flags bit for bit."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch_st():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2602_19652_gb300 as st
+    return torch, st
+
+
+def rel(a, b):
+    d = np.linalg.norm(np.ravel(b))
+    return float(np.linalg.norm(np.ravel(a) - np.ravel(b)) / (d if d > 0 else 1.0))
+
+
+def simulate_and_compare(st, wl, budget=20_000, tol=1e-4, **params):
+    import oracle
+    ctx = st.Context(0)
+    sc = st.from_workload(ctx, wl, st.curv_params(sample_budget=budget))
+    p = st.sim_params(max_bounces=wl.bounces, max_distance=wl.max_distance, **params)
+    S = ctx.simulate(sc, p).cpu().numpy()
+    ref = oracle.simulate(wl, curv=dict(budget=budget), **params)
+    g = ctx.paths(wl.bounces)
+    assert np.array_equal(g["tri"], ref["rec"]["tri"])
+    assert np.array_equal(g["los"], ref["rec"]["los"])
+    for c in range(3):
+        assert rel(S[c], ref["spectra"][c]) <= tol, (c, rel(S[c], ref["spectra"][c]))
+    return ctx, sc, S, ref
+
+
+# receiver reference point over more than one tile of 128 microphones; the partials' reduction over outputs that
+# are not a multiple of its 32 columns
+@pytest.mark.parametrize("n_mics,n_bins", [(1, 1), (127, 3), (128, 2), (129, 5), (257, 1)])
+def test_reference_point_and_reduction_tiles(torch_st, n_mics, n_bins):
+    _, st = torch_st
+    wl = synth.clutter(seed=7, target_tris=2_000, n_rays=1_500, bounces=2, n_mics=n_mics, n_bins=n_bins)
+    simulate_and_compare(st, wl)
+
+
+# the direct path's adjoint over fewer bins than its block has threads, a ragged multiple, and blocked microphones
+@pytest.mark.parametrize("n_bins", [1, 127, 129, 300])
+def test_direct_adjoint_bins(torch_st, n_bins):
+    torch, st = torch_st
+    import oracle
+    wl = synth.clutter(seed=9, target_tris=2_000, n_rays=500, bounces=1, n_mics=5, n_bins=n_bins, diffraction=False)
+    ctx, sc, S, o = simulate_and_compare(st, wl, components=st.ST_COMP_DIRECT | st.ST_COMP_SPECULAR)
+    rng = np.random.default_rng(3)
+    G = np.zeros(S.shape, np.complex64)
+    G[2] = rng.normal(size=S.shape[1:]) + 1j * rng.normal(size=S.shape[1:])
+    _, gm, ge = ctx.backward(sc, torch.as_tensor(G, device="cuda"), *wl.k_band.shape)
+    _, dmic, demit = oracle.spectra_grad(o["params"], o["rec"], wl.dirs, wl.tri_mat, G.astype(np.complex128),
+                                         None, None, None, o["direct_vis"],
+                                         tri_nrm=oracle.tri_normals(wl.verts, wl.tris))
+    assert rel(gm.cpu().numpy(), dmic) <= 1e-3
+    assert rel(ge.cpu().numpy(), demit) <= 1e-3
