@@ -61,6 +61,29 @@ __device__ __forceinline__ ff dist_ff(float ax, float ay, float az, float bx, fl
     sz.lo = fmaf(2.0f * dz.hi, dz.lo, sz.lo);
     return ff_sqrt(ff_add(ff_add(sx, sy), sz));
 }
+__device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// |a - b| as dist_ff, and *inv = 1 / |a - b| to about 2^-22: one reciprocal square root serves the square root (its
+// error, squared by the correction, leaves about 2^-43), the correction and the caller's unit vector
+__device__ __forceinline__ ff dist_inv_ff(float ax, float ay, float az, float bx, float by, float bz, float* inv) {
+    ff dx = two_sum(ax, -bx), dy = two_sum(ay, -by), dz = two_sum(az, -bz);
+    ff sx = two_prod(dx.hi, dx.hi);
+    sx.lo = fmaf(2.0f * dx.hi, dx.lo, sx.lo);
+    ff sy = two_prod(dy.hi, dy.hi);
+    sy.lo = fmaf(2.0f * dy.hi, dy.lo, sy.lo);
+    ff sz = two_prod(dz.hi, dz.hi);
+    sz.lo = fmaf(2.0f * dz.hi, dz.lo, sz.lo);
+    const ff x = ff_add(ff_add(sx, sy), sz);
+    const float y = rsqrtf(x.hi);
+    *inv = y;
+    if (!(x.hi > 0.0f)) return ff{0.0f, 0.0f};
+    const float q = x.hi * y;
+    const ff p = two_prod(q, q);
+    return fast_two_sum(q, (((x.hi - p.hi) - p.lo) + x.lo) * (0.5f * y));
+}
 // fractional part in [-0.5, 0.5] of a non-negative float-float
 __device__ __forceinline__ float ff_frac(ff x) {
     float n = rintf(x.hi);

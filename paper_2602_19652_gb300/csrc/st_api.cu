@@ -953,24 +953,21 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
         CKC(c, grow(c->keep, (size_t)K), "alloc");
         CKC(c, grow(c->los_q, (size_t)K * 4), "alloc");
     }
-    const int32_t chunks_spec =
-        accum_chunks(NB, M, F, S.n_mat, c->mic_nb, c->tune.mic_pairs_per_cta, c->tune.smem_kb, c->tune.bins_per_thread);
-    // diffraction on the tensor cores when the per-bin factor depends on material and bin only
-    bool diff_mma = false;
-    {
-        AccumArgs probe{};
-        probe.kind = 1;
-        probe.etab = c->n_theta > 0 ? ptr<float>(c->etab) : nullptr;
-        probe.mic_tab = c->mic_nb > 0 ? ptr<float>(c->mic_tab) : nullptr;
-        probe.M = M;
-        probe.F = F;
-        probe.n_mat_tab = S.n_mat;
-        diff_mma = K > 0 && diffraction_mma_applies(probe);
-    }
-    const int32_t chunks_diff =
-        diff_mma ? diffraction_mma_chunks(K, M, F, S.n_mat)
-                 : accum_chunks(K, M, F, S.n_mat, c->mic_nb, c->tune.mic_pairs_per_cta, c->tune.smem_kb,
-                                c->tune.bins_per_thread);
+    // launch shapes; diffraction on the tensor cores when the per-bin factor depends on material and bin only
+    AccumArgs probe{};
+    probe.M = M;
+    probe.F = F;
+    probe.n_mat_tab = S.n_mat;
+    probe.n_bands_tab = S.n_bands;
+    probe.etab = c->n_theta > 0 ? ptr<float>(c->etab) : nullptr;
+    probe.mic_tab = c->mic_nb > 0 ? ptr<float>(c->mic_tab) : nullptr;
+    probe.tile_tp = c->tune.mic_pairs_per_cta;
+    probe.tile_kb = c->tune.smem_kb;
+    probe.tile_kt = c->tune.bins_per_thread;
+    const int32_t chunks_spec = accum_chunks(probe, NB);
+    probe.kind = 1;
+    const bool diff_mma = K > 0 && diffraction_mma_applies(probe);
+    const int32_t chunks_diff = diff_mma ? diffraction_mma_chunks(K, M, F, S.n_mat) : accum_chunks(probe, K);
     if (diff_mma) {
         CKC(c, grow(c->mat_off, (size_t)(S.n_mat + 1) * 4), "alloc");
         CKC(c, grow(c->mat_scr, material_order_scratch(K)), "alloc");
@@ -1934,7 +1931,9 @@ void batch_release(BatchState& B) {
 // (the tile's per-microphone band tables), and jobs of a million paths or more, which fill the GPU alone
 // with their full chunk count (in the queue they would take a fraction of it).
 static bool big_job(const JobDev& d) { return d.N * (int64_t)d.B >= (1 << 20) || d.K >= (1 << 20); }
-static bool solo_accum(const JobDev& d) { return narrow_accum(d.M) || d.mic_tab != nullptr || big_job(d); }
+static bool solo_accum(const JobDev& d) {
+    return narrow_accum(d.M) || few_accum(d.M, d.F) || d.mic_tab != nullptr || big_job(d);
+}
 
 // All stages of one batch on stream s.
 // Accumulation arguments of job j's path kind (0 specular, 1 diffraction) in the batch's path lists.
@@ -2478,26 +2477,25 @@ static st_status simulate_batch_impl(st_ctx* c, int32_t n_jobs, const st_job* jo
         d.out = static_cast<float2*>(J.spectra_out);
         // chunks: the jobs of the work queue share the GPU, so each one's accumulation is split into about an
         // eighth of the chunks that would fill it alone (fewer partial spectra to sum); a job accumulated on its
-        // own (one microphone pair, receiver tables, a million paths or more) runs alone and takes them all
+        // own (one microphone pair, few bins, receiver tables, a million paths or more) runs alone and takes them all
         const int nb = solo_accum(d) ? 1 : kBatchChunkDiv;
-        const int dir_nb = J.mic_tables ? S.n_bands : 0;
-        {
-            AccumArgs probe{};
-            probe.kind = 1;
-            probe.M = d.M;
-            probe.F = d.F;
-            probe.n_mat_tab = S.n_mat;
-            probe.etab = d.etab;
-            probe.mic_tab = d.mic_tab;
-            d.diff_mma = d.K > 0 && diffraction_mma_applies(probe) ? 1 : 0;
-        }
+        AccumArgs probe{};
+        probe.M = d.M;
+        probe.F = d.F;
+        probe.n_mat_tab = S.n_mat;
+        probe.n_bands_tab = S.n_bands;
+        probe.etab = d.etab;
+        probe.mic_tab = d.mic_tab;
+        probe.tile_tp = tn.mic_pairs_per_cta;
+        probe.tile_kb = tn.smem_kb;
+        const int32_t chunks_spec = accum_chunks(probe, d.N * d.B);
+        probe.kind = 1;
+        d.diff_mma = d.K > 0 && diffraction_mma_applies(probe) ? 1 : 0;
         B.any_mma = B.any_mma || d.diff_mma;
         B.any_table_order = B.any_table_order || (d.etab != nullptr && d.K > 0 && !d.diff_mma);
-        B.chunks_spec[j] =
-            std::max(1, accum_chunks(d.N * d.B, d.M, d.F, S.n_mat, dir_nb, tn.mic_pairs_per_cta, tn.smem_kb) / nb);
+        B.chunks_spec[j] = std::max(1, chunks_spec / nb);
         B.chunks_diff[j] =
-            d.diff_mma ? std::max(1, diffraction_mma_chunks(d.K, d.M, d.F, S.n_mat) / nb)
-                       : std::max(1, accum_chunks(d.K, d.M, d.F, S.n_mat, dir_nb, tn.mic_pairs_per_cta, tn.smem_kb) / nb);
+            std::max(1, (d.diff_mma ? diffraction_mma_chunks(d.K, d.M, d.F, S.n_mat) : accum_chunks(probe, d.K)) / nb);
         if (solo_accum(d))
             narrow_part = std::max(narrow_part, (size_t)std::max(B.chunks_spec[j], B.chunks_diff[j]) * d.M * d.F * 8);
     }

@@ -364,8 +364,16 @@ cudaError_t build_accum_tables(AccumTables& T, const SceneDev& S, int32_t F, dou
                                double a0, double a1, cudaStream_t s);
 cudaError_t accumulate(const AccumArgs& a, cudaStream_t s);
 cudaError_t reduce_partials(const float2* partial, int32_t n_chunks, int64_t MF, float2* out, cudaStream_t s);
-int32_t accum_chunks(int64_t n_paths_hint, int32_t M, int32_t F, int32_t n_mat, int32_t dir_nb, int32_t tile_tp = 0,
-                     int32_t tile_kb = 0, int32_t tile_kt = 0);
+// chunks for an accumulation of at most n_paths paths; a: kind, sizes, directivity and tile set
+int32_t accum_chunks(const AccumArgs& a, int64_t n_paths);
+// Few frequency bins, omni receivers, three microphones or more (st_accum_few.cu).  Where the line lies: the general
+// accumulator shares a path's factors and anchors between 16 pairs and 16 subtiles and wins when it has that many
+// (specular accumulation of 104k paths, few-bin kernel / general, ms: 32 x 48 0.15 / 0.25, 32 x 96 0.22 / 0.24, 32 x 120
+// 0.29 / 0.24, 64 x 48 0.27 / 0.31, 64 x 64 0.39 / 0.28, 17 x 96 0.16 / 0.21, 17 x 128 0.22 / 0.21, 10 x 331 0.31 /
+// 0.34, 10 x 512 0.61 / 0.40, 6 x 512 0.29 / 0.39, 3 x 331 0.14 / 0.39, 3 x 1024 0.56 / 1.47).
+inline bool few_accum(int32_t M, int32_t F) { return M > 2 && (int64_t)M * F <= 3400 && (F <= 96 || M <= 10); }
+int32_t few_chunks(const AccumArgs& a, int64_t n_paths);
+cudaError_t accumulate_few(const AccumArgs& a, cudaStream_t s);
 // emitter ray sets (st_rays.cu): kind 0 spherical Fibonacci, 1 zonal equal-area centres
 cudaError_t ray_directions(int kind, int64_t n, float* out, DevBuf& scratch, cudaStream_t s);
 // impulse responses / received signals from accumulated spectra (st_signal.cu)

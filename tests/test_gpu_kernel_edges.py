@@ -63,3 +63,34 @@ def test_direct_adjoint_bins(torch_st, n_bins):
                                          tri_nrm=oracle.tri_normals(wl.verts, wl.tris))
     assert rel(gm.cpu().numpy(), dmic) <= 1e-3
     assert rel(ge.cpu().numpy(), demit) <= 1e-3
+
+
+# the few-bin accumulator: one run and several, every run length, path groups that do not divide the threads, microphone
+# blocks, ragged last runs, the sizes on both sides of its line, more materials than its shared rows hold
+@pytest.mark.parametrize("n_mics,n_bins", [(3, 1), (3, 14), (5, 15), (32, 14), (33, 13), (64, 14), (17, 25), (7, 37),
+                                           (35, 96), (36, 96), (10, 340), (3, 1024), (4, 851), (100, 33)])
+def test_few_bins_match_oracle(torch_st, n_mics, n_bins):
+    _, st = torch_st
+    wl = synth.clutter(seed=11, target_tris=2_500, n_rays=1_200, bounces=6, n_mics=n_mics, n_bins=n_bins)
+    simulate_and_compare(st, wl, budget=3_000)
+
+
+@pytest.mark.parametrize("mode,los", [(1, 0), (0, 1)])
+def test_few_bins_modes_match_oracle(torch_st, mode, los):
+    _, st = torch_st
+    wl = synth.clutter(seed=12, target_tris=2_500, n_rays=1_500, bounces=3, n_mics=9, n_bins=14)
+    wl.mics = (wl.mics + np.random.default_rng(5).uniform(-4, 4, wl.mics.shape) * [1, 1, 0.1]).astype(np.float32)
+    simulate_and_compare(st, wl, budget=3_000, reflection_mode=mode, los_mode=los)
+
+
+@pytest.mark.parametrize("n_mat", [1, 60])
+def test_few_bins_emitter_table_and_many_materials(torch_st, n_mat):
+    _, st = torch_st
+    rng = np.random.default_rng(8)
+    wl = synth.clutter(seed=13, target_tris=2_500, n_rays=1_500, bounces=5, n_mics=6, n_bins=33)
+    wl.tri_mat = (np.arange(wl.n_tris) % n_mat).astype(np.int32)
+    wl.k_band = synth.smooth_band_curves(rng, n_mat, 16, 0.3, 0.95)
+    wl.beta_band = np.deg2rad(synth.smooth_band_curves(rng, n_mat, 16, 5.0, 30.0)).astype(np.float32)
+    wl.diff_band = synth.smooth_band_curves(rng, n_mat, 16, 0.02, 0.08)
+    wl.emitter_table = rng.uniform(0.1, 1.0, (37, 33)).astype(np.float32)
+    simulate_and_compare(st, wl, budget=3_000)
