@@ -94,3 +94,11 @@ def test_few_bins_emitter_table_and_many_materials(torch_st, n_mat):
     wl.diff_band = synth.smooth_band_curves(rng, n_mat, 16, 0.02, 0.08)
     wl.emitter_table = rng.uniform(0.1, 1.0, (37, 33)).astype(np.float32)
     simulate_and_compare(st, wl, budget=3_000)
+
+
+# the general accumulator where its bins are spread over blocks (subtiles rounded to four, a second block of one bin)
+@pytest.mark.parametrize("n_mics,n_bins", [(32, 257), (17, 331), (24, 200), (12, 513), (40, 129)])
+def test_general_tile_bin_blocks_match_oracle(torch_st, n_mics, n_bins):
+    _, st = torch_st
+    wl = synth.clutter(seed=14, target_tris=2_500, n_rays=1_200, bounces=3, n_mics=n_mics, n_bins=n_bins)
+    simulate_and_compare(st, wl, budget=3_000)
