@@ -97,7 +97,7 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
     float* pdb = reinterpret_cast<float*>(reinterpret_cast<char*>(smem4) + 2 * g.buf_bytes);  // [2][PT][12]
     int* pvb = reinterpret_cast<int*>(pdb + 2 * PT * 12);                                       // [2][PT]
     // material tables: 16-byte aligned for the 128-bit loads of phase 1a
-    float* mt = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(pvb + 2 * PT) + 15) & ~uintptr_t(15));
+    float* mt = reinterpret_cast<float*>(align16(smem4, pvb + 2 * PT));
 
     const int mb = bx % g.n_mb, bb = bx / g.n_mb;
     const int mic0 = mb * MP, kb = bb * KB;
@@ -162,15 +162,15 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
                               pb0 + (tile + 1) * PT);
         }
         for (int p = 0; p < (cons ? PT : 0); ++p) {
-            const ulonglong2 z0 = C.za[((size_t)p * NS + s) * TP + tp];
-            const u64* w = C.wst + (size_t)p * 4 * TP + tp;  // component-major: conflict-free 64-bit loads
+            const ulonglong2 z0 = C.za[(p * NS + s) * TP + tp];
+            const u64* w = C.wst + p * 4 * TP + tp;  // component-major: conflict-free 64-bit loads
             const u64 w1r = w[0], w1i = w[TP], w2r = w[2 * TP], w2i = w[3 * TP];
             const u64 nw2i = fmul2(w2i, pk2(-1.0f, -1.0f));
-            const u64 ng = C.ngp[(size_t)p * TP + tp];
+            const u64 ng = C.ngp[p * TP + tp];
             u64 er = z0.x, ei = z0.y;  // even chain: bins 0, 2, 4, ...
             u64 orr = er, oi = ei;     // odd chain: bins 1, 3, 5, ...
             cmul2(orr, oi, w1r, w1i, fmul2(w1i, pk2(-1.0f, -1.0f)));
-            const float2* trow = reinterpret_cast<const float2*>(C.tab) + (size_t)p * KB + s;
+            const float2* trow = reinterpret_cast<const float2*>(C.tab) + p * KB + s;
             const float2 ngv = up2(ng);  // -gamma^2 of the two microphones
             // diffraction with the material table read directly: the producer left the offset of the path's
             // material row in the (otherwise unused) lobe slot
@@ -190,7 +190,7 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
                 if (DIR) {  // receiver directivity, linear between bands
                     const float2 bwv = bwt[kk * NS + s];
                     const int b0 = (int)bwv.x;
-                    const float* d1 = C.dband + ((size_t)p * MP + 2 * tp) * g.NB;
+                    const float* d1 = C.dband + (p * MP + 2 * tp) * g.NB;
                     const float* d2 = d1 + g.NB;
                     float D1 = d1[b0], D2 = d2[b0];
                     if (g.NB > 1) {

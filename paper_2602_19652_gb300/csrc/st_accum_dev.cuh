@@ -102,6 +102,15 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 
 constexpr float kNegInf = -__builtin_huge_valf();
 
+// p rounded up to 16 bytes within the shared memory that starts at base (16-byte aligned).  As an offset from base:
+// rounded through an integer the pointer loses its address space, and every access through it becomes a generic load
+// with 64-bit index arithmetic.
+template <class T>
+__device__ __forceinline__ char* align16(float4* base, T* p) {
+    char* b = reinterpret_cast<char*>(base);
+    return b + (((int)(reinterpret_cast<char*>(p) - b) + 15) & ~15);
+}
+
 // ---------------------------------------------------------------- accumulator
 // Packed FP32 pairs (fma/mul .f32x2, sm_100 and later): one 64-bit register holds the same
 // quantity for two microphones, so every inner-loop instruction advances two terms.
@@ -346,17 +355,17 @@ __device__ __forceinline__ void anchor_mic(const AccumArgs& a, const Geom& g, co
     const int TP = g.TP, KB = g.KB, MP = g.MP;
     const int pair = ml >> 1, half = ml & 1;
     const int m = mic0 + ml;
-    float* wf = reinterpret_cast<float*>(B.wst + (size_t)p * 4 * TP + pair);  // component c at wf[2 TP c]
-    float* nf = reinterpret_cast<float*>(B.ngp + (size_t)p * TP + pair);
+    float* wf = reinterpret_cast<float*>(B.wst + p * 4 * TP + pair);  // component c at wf[2 TP c]
+    float* nf = reinterpret_cast<float*>(B.ngp + p * TP + pair);
     // (per-microphone receiver test: a microphone that does not see the path gets a zero anchor)
     if (!pv[p] || m >= a.M || (a.mask && !((a.mask[pglob + p] >> m) & 1ull))) {
         *z_out = make_float2(0.0f, 0.0f);
         *wk_out = make_float2(0.0f, 0.0f);
         for (int q = 0; q < 4; ++q) wf[2 * TP * q + half] = 0.0f;
         nf[half] = 0.0f;
-        for (int b = 0; b < g.NB; ++b) B.dband[((size_t)p * MP + ml) * g.NB + b] = 0.0f;
+        for (int b = 0; b < g.NB; ++b) B.dband[(p * MP + ml) * g.NB + b] = 0.0f;
         if (ADJ) {
-            float* af = reinterpret_cast<float*>(B.adj + ((size_t)p * TP + pair) * 7);
+            float* af = reinterpret_cast<float*>(B.adj + (p * TP + pair) * 7);
             for (int q = 0; q < 7; ++q) af[2 * q + half] = 0.0f;
         }
         return;
@@ -365,12 +374,12 @@ __device__ __forceinline__ void anchor_mic(const AccumArgs& a, const Geom& g, co
     const float mx = a.mics[3 * m], my = a.mics[3 * m + 1], mz = a.mics[3 * m + 2];
     const ff dist = dist_ff(mx, my, mz, d[0], d[1], d[2]);
     const ff r = ff_add(ff{d[6], d[7]}, dist);
-    if (g.NB > 0) mic_bands(a, m, d[0] - mx, d[1] - my, d[2] - mz, B.dband + ((size_t)p * MP + ml) * g.NB, g.NB);
+    if (g.NB > 0) mic_bands(a, m, d[0] - mx, d[1] - my, d[2] - mz, B.dband + (p * MP + ml) * g.NB, g.NB);
     float gam2 = 0.0f;
     if (KIND == 0 || ADJ) {
         const float inv = __fdividef(1.0f, dist.hi);
         const float ux = (mx - d[0]) * inv, uy = (my - d[1]) * inv, uz = (mz - d[2]) * inv;
-        float* af = reinterpret_cast<float*>(B.adj + ((size_t)p * TP + pair) * 7);
+        float* af = reinterpret_cast<float*>(B.adj + (p * TP + pair) * 7);
         if (KIND == 0) {
             const float cg = d[3] * ux + d[4] * uy + d[5] * uz;
             const float cx = d[4] * uz - d[5] * uy, cy = d[5] * ux - d[3] * uz, cz = d[3] * uy - d[4] * ux;
@@ -398,7 +407,7 @@ __device__ __forceinline__ void anchor_mic(const AccumArgs& a, const Geom& g, co
         }
     }
     const float rh = r.hi;
-    if (ADJ) reinterpret_cast<float*>(B.adj + ((size_t)p * TP + pair) * 7)[12 + half] = 1.0f / rh;
+    if (ADJ) reinterpret_cast<float*>(B.adj + (p * TP + pair) * 7)[12 + half] = 1.0f / rh;
     const float L0 = -2.0f * log2_ff(r) + rh * (a.atm2_0 + a.atm2_step * (float)kb);
     const ff x0 = ff_mul(r, ff{a.qhi[min(kb, a.F - 1)], a.qlo[min(kb, a.F - 1)]});
     float s0, c0;
@@ -488,7 +497,7 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                 if (k0 + 3 * KT >= a.F) lx4.w = kNegInf;
             }
             // four 8-byte entries (32-byte aligned: i is a multiple of 4)
-            float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float2*>(B.tab) + (size_t)p * KB + i);
+            float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float2*>(B.tab) + p * KB + i);
             if (KIND == 0) {
                 dst[0] = make_float4(lx4.x, g4.x, lx4.y, g4.y);
                 dst[1] = make_float4(lx4.z, g4.z, lx4.w, g4.w);
@@ -535,10 +544,10 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                 }
             }
             if (KIND == 0) {
-                reinterpret_cast<float2*>(B.tab)[(size_t)p * KB + i] = make_float2(lx, gg);
+                reinterpret_cast<float2*>(B.tab)[p * KB + i] = make_float2(lx, gg);
             } else {
                 const float x = ex2(lx);
-                reinterpret_cast<float2*>(B.tab)[(size_t)p * KB + i] = make_float2(x, x);
+                reinterpret_cast<float2*>(B.tab)[p * KB + i] = make_float2(x, x);
             }
         }
     }
@@ -556,9 +565,9 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                                                 &wk[half]);
             u64 zr = pk2(zz[0].x, zz[1].x), zi = pk2(zz[0].y, zz[1].y);
             const u64 kr = pk2(wk[0].x, wk[1].x), ki = pk2(wk[0].y, wk[1].y), nki = pk2(-wk[0].y, -wk[1].y);
-            ulonglong2* zo = B.za + (size_t)p * NS * TP + pair;
+            ulonglong2* zo = B.za + p * NS * TP + pair;
             for (int s_ = 0; s_ < NS; ++s_) {
-                zo[(size_t)s_ * TP] = make_ulonglong2(zr, zi);
+                zo[s_ * TP] = make_ulonglong2(zr, zi);
                 cmul2(zr, zi, kr, ki, nki);
             }
         }
@@ -568,10 +577,10 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
             const int pair = ml >> 1, half = ml & 1;
             float2 z, wk;
             anchor_mic<KT, KIND, ADJ>(a, g, B, pd, pv, p, ml, mic0, kb, es, pglob, &z, &wk);
-            float* zf = reinterpret_cast<float*>(B.za + (size_t)p * NS * TP + pair);
+            float* zf = reinterpret_cast<float*>(B.za + p * NS * TP + pair);
             for (int s_ = 0; s_ < NS; ++s_) {
-                zf[(size_t)s_ * TP * 4 + half] = z.x;
-                zf[(size_t)s_ * TP * 4 + 2 + half] = z.y;
+                zf[s_ * TP * 4 + half] = z.x;
+                zf[s_ * TP * 4 + 2 + half] = z.y;
                 z = cmul(z, wk);
             }
         }

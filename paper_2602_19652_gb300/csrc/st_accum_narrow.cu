@@ -73,14 +73,14 @@ __device__ __forceinline__ void nproduce(const AccumArgs& a, const NGeom& g, con
         const int p = e / (2 * items), rem = e - p * 2 * items;
         const int half = rem / items, it = rem - half * items;
         const int m = half;
-        float* zf = reinterpret_cast<float*>(it == 0 ? B.zb + p : B.pw + (size_t)p * (g.LNS + 2) + (it - 1));
+        float* zf = reinterpret_cast<float*>(it == 0 ? B.zb + p : B.pw + p * (g.LNS + 2) + (it - 1));
         // (per-microphone receiver test: a microphone that does not see the path gets a zero anchor)
         if (!pv[p] || m >= a.M || (a.mask && !((a.mask[pglob + p] >> m) & 1ull))) {
             zf[half] = 0.0f;
             zf[2 + half] = 0.0f;
             if (it == 0) {
                 reinterpret_cast<float*>(B.ngp + p)[half] = 0.0f;
-                for (int b = 0; b < g.NB; ++b) B.dband[((size_t)p * g.NB + b) * 2 + half] = 0.0f;
+                for (int b = 0; b < g.NB; ++b) B.dband[(p * g.NB + b) * 2 + half] = 0.0f;
             }
             continue;
         }
@@ -100,7 +100,7 @@ __device__ __forceinline__ void nproduce(const AccumArgs& a, const NGeom& g, con
                 gam2 = gm * gm;
             }
             reinterpret_cast<float*>(B.ngp + p)[half] = -gam2;
-            if (g.NB > 0) mic_bands(a, m, d[0] - mx, d[1] - my, d[2] - mz, B.dband + (size_t)p * 2 * g.NB + half, g.NB, 2);
+            if (g.NB > 0) mic_bands(a, m, d[0] - mx, d[1] - my, d[2] - mz, B.dband + p * 2 * g.NB + half, g.NB, 2);
             const float L0 = -2.0f * log2_ff(r) + rh * (a.atm2_0 + a.atm2_step * (float)kb);
             const ff x0 = ff_mul(r, ff{a.qhi[min(kb, a.F - 1)], a.qlo[min(kb, a.F - 1)]});
             float s0, c0;
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(kNThreads, 2) k_accum_narrow(const AccumArgs a
     const int PT = g.PT, NS = g.NS, KB = g.KB;
     float* pdb = reinterpret_cast<float*>(base + 2 * g.buf_bytes);  // [3][PT][12]
     int* pvb = reinterpret_cast<int*>(pdb + 3 * PT * 12);            // [3][PT]
-    float* mt = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(pvb + 3 * PT) + 15) & ~uintptr_t(15));
+    float* mt = reinterpret_cast<float*>(align16(smem4, pvb + 3 * PT));
     const int nm = a.n_mat_tab;
     // material rows of the CTA's bins: lk, g2 (specular) or lid (diffraction), [n_mat][KB] each; then
     // the per-bin band interpolation (directional receivers)
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kNThreads, 2) k_accum_narrow(const AccumArgs a
             // this thread's first phasor: z(kb) times the bin step to the power s (bits of s)
             const ulonglong2 z0 = C.zb[p];
             u64 er = z0.x, ei = z0.y;
-            const ulonglong2* pw = C.pw + (size_t)p * (g.LNS + 2);
+            const ulonglong2* pw = C.pw + p * (g.LNS + 2);
             for (int e = 0; e < g.LNS; ++e) {
                 const ulonglong2 w = pw[e];
                 const bool on = (s >> e) & 1;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kNThreads, 2) k_accum_narrow(const AccumArgs a
                 ew = x - (float)itn;
                 e0 = a.etab + (int64_t)itn * a.F;
             }
-            const u64* dp = reinterpret_cast<const u64*>(C.dband) + (size_t)p * g.NB;
+            const u64* dp = reinterpret_cast<const u64*>(C.dband) + p * g.NB;
             // the term loop, specialised on the emitter table (its loads then carry no condition)
             auto terms = [&](auto has_e) {
                 constexpr bool HE = decltype(has_e)::value;

@@ -85,13 +85,12 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
     float* pdb = reinterpret_cast<float*>(reinterpret_cast<char*>(smem4) + 2 * g.buf_bytes);
     int* pvb = reinterpret_cast<int*>(pdb + 3 * PT * 12);
     // (16-byte aligned: each path's 12 floats are read as three float4)
-    float* pjb = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(pvb + 3 * PT) + 15) & ~uintptr_t(15));
+    float* pjb = reinterpret_cast<float*>(align16(smem4, pvb + 3 * PT));
     // (specular) per path of a tile: how often each of the launch's kNV materials occurs in its reflection chain
     float4* pcb = reinterpret_cast<float4*>(pjb + (EMIT ? 3 * PT * 12 : 0));
     // (specular) and one integer signature of those counts per path (-1: no path), compared between neighbours
     int* psg = reinterpret_cast<int*>(pcb + (KIND == 0 ? 3 * PT : 0));
-    float* mt = reinterpret_cast<float*>(
-        (reinterpret_cast<uintptr_t>(psg + (KIND == 0 ? 3 * PT : 0)) + 15) & ~uintptr_t(15));
+    float* mt = reinterpret_cast<float*>(align16(smem4, psg + (KIND == 0 ? 3 * PT : 0)));
 
     const int mb = blockIdx.x % g.n_mb, bb = blockIdx.x / g.n_mb;
     const int mic0 = mb * g.MP, kb = bb * KB;
@@ -238,17 +237,17 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
 #pragma unroll
         for (int kk = 0; kk < KT; ++kk) Y[kk] = 0.0f;
         for (int p = 0; p < PT; ++p) {
-            const ulonglong2 z0 = C.za[((size_t)p * NS + s) * TP + tp];
-            const u64* w = C.wst + (size_t)p * 4 * TP + tp;  // component-major: conflict-free 64-bit loads
+            const ulonglong2 z0 = C.za[(p * NS + s) * TP + tp];
+            const u64* w = C.wst + p * 4 * TP + tp;  // component-major: conflict-free 64-bit loads
             const u64 w1r = w[0], w1i = w[TP], w2r = w[2 * TP], w2i = w[3 * TP];
             const u64 nw2i = fmul2(w2i, pk2(-1.0f, -1.0f));
-            const u64 ng = C.ngp[(size_t)p * TP + tp];
+            const u64 ng = C.ngp[p * TP + tp];
             u64 er = z0.x, ei = z0.y, orr = er, oi = ei;
             cmul2(orr, oi, w1r, w1i, fmul2(w1i, pk2(-1.0f, -1.0f)));
             u64 c0r = 0ull, c0i = 0ull, qr = 0ull, qi = 0ull, cg = 0ull;
             u64 c1r = 0ull, c1i = 0ull;  // diffraction: C1 = sum_kk kk conj(G) T directly
             const float2 ngv = up2(ng);  // -gamma^2 of the two microphones (lobe sums)
-            const float2* trow = reinterpret_cast<const float2*>(C.tab) + (size_t)p * KB + s;
+            const float2* trow = reinterpret_cast<const float2*>(C.tab) + p * KB + s;
             // diffraction with the material table read directly: row offset left by the producer in ngp
             const u64* mrow = reinterpret_cast<const u64*>(mt) + s;
             if (KIND == 1 && g.mat_direct) mrow += (int)(uint32_t)ng;
@@ -300,7 +299,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
                 }
             }
             if (do_pos) {
-                const u64* ad = C.adj + ((size_t)p * TP + tp) * 7;
+                const u64* ad = C.adj + (p * TP + tp) * 7;
                 // C1 relative to the subtile's first bin
                 const u64 q1r = KIND == 1 ? c1r : fsub2(fmul2(pk2((float)KT, (float)KT), c0r), qr);
                 const u64 q1i = KIND == 1 ? c1i : fsub2(fmul2(pk2((float)KT, (float)KT), c0i), qi);
