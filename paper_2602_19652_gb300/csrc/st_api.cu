@@ -77,7 +77,6 @@ struct st_ctx {
     int64_t N = 0;
     DevBuf dirs, etab, perm, ord_keys, ord_scr;
     DevBuf th_keys, th_scr;          // emitter-table row order of the specular path list
-    DevBuf vs_keys, vs_scr;          // hit-point Morton order of the visibility queries
     int32_t n_theta = 0;
     float fov_half = 4.0f;
     // receivers
@@ -120,7 +119,7 @@ struct st_ctx {
     DevBuf sig_e, sig_g;             // impulse responses: call spectrum [F], combined spectra [rows][F]
     DevBuf ray_tab;                  // zone table of the zonal ray set
     DevBuf adj_jac;                  // backward: chain jacobians of the specular paths [paths][12]
-    DevBuf hit_tri, hit_t, vis_q, los_q, trav_cnt;
+    DevBuf vis_q, los_q, trav_cnt;
     DevBuf rec_mask;                 // per-microphone receiver test: visible microphones of each record  // lane-refill traversal: closest hits, query queues, counters
     cudaEvent_t ev[10] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     // stage overlap: the diffraction stage and the direct path of a simulate run on a side stream while
@@ -294,9 +293,8 @@ cudaMemcpyKind kind_out(int32_t mem) { return mem == ST_MEM_DEVICE ? cudaMemcpyD
 // of a million paths or more takes them all: it is accumulated on its own)
 constexpr int kBatchChunkDiv = 8;
 
-// triangle count from which the visibility queries of a simulate are sorted by hit point (the 4-wide
-// hierarchy and the triangles then take well over half of L2)
-constexpr int64_t kVisSortTris = 1000000;
+// traversal counters: 64 bytes of the diffraction stage's, then the trace's queue lengths and claim counters by bounce
+constexpr size_t kTravCounts = 64 + (kMaxBounces + 1) * 16;
 
 uint64_t g_scene_version = 1;
 
@@ -386,7 +384,7 @@ st_status st_destroy(st_ctx* c) {
     cudaStreamSynchronize(c->stream);
     if (c->side) cudaStreamSynchronize(c->side);
     for (DevBuf* b : {&c->mic_q, &c->mic_tab, &c->tables.bw}) release(*b);
-    for (DevBuf* b : {&c->dirs, &c->etab, &c->perm, &c->ord_keys, &c->ord_scr, &c->th_keys, &c->th_scr, &c->vs_keys, &c->vs_scr, &c->mics, &c->st_o[0], &c->st_o[1], &c->st_o[2], &c->st_d[0], &c->st_d[1],
+    for (DevBuf* b : {&c->dirs, &c->etab, &c->perm, &c->ord_keys, &c->ord_scr, &c->th_keys, &c->th_scr, &c->mics, &c->st_o[0], &c->st_o[1], &c->st_o[2], &c->st_d[0], &c->st_d[1],
                       &c->st_d[2], &c->st_r, &c->st_prev, &c->q0, &c->q1, &c->counts, &c->queries, &c->flags, &c->R, &c->rec_tri,
                       &c->rec_p, &c->rec_d, &c->rec_r, &c->rec_los, &c->sflags, &c->sscan, &c->sidx, &c->scratch,
                       &c->cand_tri, &c->cand_p, &c->keep, &c->dvis, &c->partial, &c->host_out, &c->mat_off, &c->mat_scr, &c->tables.lk,
@@ -398,7 +396,7 @@ st_status st_destroy(st_ctx* c) {
             release(*b);
     for (DevBuf* b : {&c->adj_v, &c->adj_mic, &c->adj_emit, &c->tables.band, &c->tables.kband, &c->tables.bband,
                       &c->sig_e, &c->sig_g,
-                      &c->ray_tab, &c->adj_jac, &c->hit_tri, &c->hit_t, &c->vis_q, &c->los_q, &c->trav_cnt,
+                      &c->ray_tab, &c->adj_jac, &c->vis_q, &c->los_q, &c->trav_cnt,
                       &c->rec_mask})
         release(*b);
     for (auto& e : c->ev)
@@ -909,15 +907,14 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
     CKC(c, grow(c->queries, 64), "alloc");
     CKC(c, grow(c->flags, 16), "alloc");
     CKC(c, grow(c->R, 16), "alloc");
-    CKC(c, grow(c->hit_tri, (size_t)std::max<int64_t>(N, 1) * 4), "alloc");
-    CKC(c, grow(c->hit_t, (size_t)std::max<int64_t>(N, 1) * 4), "alloc");
     const bool per_mic = p.los_mode == ST_LOS_PER_MIC;
-    CKC(c, grow(c->vis_q, (size_t)std::max<int64_t>(N, 1) * (per_mic ? (size_t)M : 1) * 4), "alloc");
+    const size_t n_visq = (size_t)std::max<int64_t>(N, 1) * (per_mic ? (size_t)M : 1);
+    CKC(c, grow(c->vis_q, 2 * n_visq * 4), "alloc");
     if (per_mic) {
         CKC(c, grow(c->rec_mask, (size_t)std::max<int64_t>(NB, 1) * 8), "alloc");
         CKC(c, grow(c->paths.mask, (size_t)std::max<int64_t>(NB, 1) * 8), "alloc");
     }
-    CKC(c, grow(c->trav_cnt, 64), "alloc");
+    CKC(c, grow(c->trav_cnt, kTravCounts), "alloc");
     CKC(c, grow(c->rec_tri, (size_t)std::max<int64_t>(NB, 1) * 4), "alloc");
     CKC(c, grow(c->rec_p, (size_t)std::max<int64_t>(NB, 1) * 12), "alloc");
     CKC(c, grow(c->rec_d, (size_t)std::max<int64_t>(NB, 1) * 12), "alloc");
@@ -927,14 +924,7 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
     CKC(c, grow(c->sscan, (size_t)nflag * 4), "alloc");
     CKC(c, grow(c->sidx, (size_t)nflag * 4), "alloc");
     CKC(c, grow(c->scratch, scan_scratch_bytes(nflag)), "alloc");
-    // Scenes whose hierarchy and triangles are well beyond L2 trace their visibility queries in the Morton
-    // order of the hit points (all go to one point, so neighbours in that order share most nodes)
-    const bool vsort = S.n_tris >= kVisSortTris && N > 1 && !per_mic;
-    if (vsort) {
-        CKC(c, grow(c->vs_keys, (size_t)N * 8), "alloc");
-        CKC(c, grow(c->vs_scr, sort_scratch_bytes(N)), "alloc");
-    }
-    if (K > 1) {  // the line-of-sight queue of the diffraction candidates is sorted likewise (own buffers)
+    if (K > 1) {  // the line-of-sight queue of the diffraction candidates is sorted by Morton code
         CKC(c, grow(c->los_keys, (size_t)K * 8), "alloc");
         CKC(c, grow(c->los_scr, sort_scratch_bytes(K)), "alloc");
     }
@@ -986,6 +976,7 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
     CKC(c, cudaMemsetAsync(out, 0, (size_t)3 * MF * 8, s), "memset out");
     CKC(c, cudaMemsetAsync(c->flags.p, 0, 16, s), "memset");
     CKC(c, cudaMemsetAsync(c->counts.p, 0, 64, s), "memset");
+    CKC(c, cudaMemsetAsync(c->trav_cnt.p, 0, kTravCounts, s), "memset");
     CKC(c, cudaMemsetAsync(c->queries.p, 0, 64, s), "memset");
     unsigned long long* qctr = ptr<unsigned long long>(c->queries);
     CKC(c, cudaMemsetAsync(c->rec_tri.p, 0xff, (size_t)std::max<int64_t>(NB, 1) * 4, s), "memset");
@@ -1074,10 +1065,8 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
             ta.dz = ptr<float>(c->st_d[2]);
             ta.racc = ptr<double>(c->st_r);
             ta.prev = ptr<int32_t>(c->st_prev);
-            ta.q_in = ptr<uint32_t>(c->q0);
-            ta.q_out = ptr<uint32_t>(c->q1);
-            ta.n_in = cnt + 0;
-            ta.n_out = cnt + 1;
+            ta.live_q[0] = ptr<uint32_t>(c->q0);
+            ta.live_q[1] = ptr<uint32_t>(c->q1);
             ta.rec_tri = ptr<int32_t>(c->rec_tri);
             ta.rec_p = ptr<float>(c->rec_p);
             ta.rec_d = ptr<float>(c->rec_d);
@@ -1085,21 +1074,15 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
             ta.rec_los = ptr<uint8_t>(c->rec_los);
             ta.flags = ptr<uint32_t>(c->flags);
             ta.queries = qctr;
-            ta.hit_tri = ptr<int32_t>(c->hit_tri);
-            ta.hit_t = ptr<float>(c->hit_t);
-            ta.vis_q = ptr<uint32_t>(c->vis_q);
-            ta.vis_n = ptr<uint32_t>(c->trav_cnt);
-            ta.ctr = reinterpret_cast<unsigned long long*>(ptr<char>(c->trav_cnt) + 16);
+            ta.vis_q[0] = ptr<uint32_t>(c->vis_q);
+            ta.vis_q[1] = ta.vis_q[0] + n_visq;
+            char* tc = ptr<char>(c->trav_cnt) + 64;
+            ta.ctr = reinterpret_cast<unsigned long long*>(tc);
+            ta.n_live = reinterpret_cast<uint32_t*>(tc + (kMaxBounces + 1) * 8);
+            ta.n_vis = ta.n_live + kMaxBounces + 1;
             ta.rec_mask = per_mic ? ptr<uint64_t>(c->rec_mask) : nullptr;
             ta.mics = ptr<float>(c->mics);
             ta.M = M;
-            ta.sort_keys = vsort ? ptr<uint64_t>(c->vs_keys) : nullptr;
-            ta.sort_scr = vsort ? c->vs_scr.p : nullptr;
-            for (int k = 0; k < 3; ++k) {
-                const float ext = S.bounds_hi[k] - S.bounds_lo[k];
-                ta.blo[k] = S.bounds_lo[k];
-                ta.bscale[k] = ext > 0.0f ? 1024.0f / ext : 0.0f;
-            }
             CKC(c, trace_rays(ta, s, c->tune.rays_per_block > 0 ? c->tune.rays_per_block : 128), "trace");
         }
         return ST_OK;

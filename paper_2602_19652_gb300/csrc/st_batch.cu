@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kTravBlock, 8) k_closest_batch(const BatchArgs
         const unsigned nd0 = __ballot_sync(full, !live && !exhausted);
         if (lv0 == 0u && nd0 == 0u) break;
         while (true) {
-            if (live && trav_step<false>(T, S, stack, a.flags)) {
+            if (live && trav_step<kClosest>(T, S, stack, a.flags)) {
                 a.hit_tri[g] = S.best;
                 a.hit_t[g] = S.tb;
                 live = false;
@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(kTravBlock, 8) k_visible_batch(const BatchArgs
         const unsigned nd0 = __ballot_sync(full, !live && !exhausted);
         if (lv0 == 0u && nd0 == 0u) break;
         while (true) {
-            if (live && trav_step<true>(T, S, stack, a.flags)) {
+            if (live && trav_step<kAny>(T, S, stack, a.flags)) {
                 out[id] = S.best < 0 ? 1 : 0;
                 live = false;
             }
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kTravBlock, 8) k_visible_mics_batch(const Batc
         const unsigned nd0 = __ballot_sync(full, !live && !exhausted);
         if (lv0 == 0u && nd0 == 0u) break;
         while (true) {
-            if (live && trav_step<true>(T, S, stack, a.flags)) {
+            if (live && trav_step<kAny>(T, S, stack, a.flags)) {
                 if (S.best < 0) {
                     atomicOr(reinterpret_cast<unsigned long long*>(&a.rec_mask[id]), 1ull << m);
                     a.rec_los[id] = 1;

@@ -199,18 +199,13 @@ struct TraceArgs {
     float* dx; float* dy; float* dz;
     double* racc;
     int32_t* prev;
-    // queues
-    uint32_t* q_in; uint32_t* q_out;
-    uint32_t* n_in; uint32_t* n_out;
-    // closest hits of the current bounce [N], the visibility queue (record ids) and the lane-refill
-    // counters (three per bounce)
-    int32_t* hit_tri; float* hit_t;
-    uint32_t* vis_q; uint32_t* vis_n;
-    unsigned long long* ctr;
-    // optional: visibility queue sorted by the Morton code of the hit points (scene bounds lo, 1024 / extent)
-    // before it is traced, so that neighbouring lanes share nodes; keys [N] and sort scratch, or null
-    uint64_t* sort_keys; void* sort_scr;
-    float blo[3], bscale[3];
+    // live-ray queues and visibility queues (record ids, or record * M + microphone), of even and odd bounces; their
+    // lengths and the claim counters by bounce, zeroed by the caller
+    uint32_t* live_q[2];
+    uint32_t* vis_q[2];
+    uint32_t* n_live;         // [kMaxBounces + 1] (entry 0 unused: the first bounce takes all rays)
+    uint32_t* n_vis;          // [kMaxBounces + 1]
+    unsigned long long* ctr;  // [kMaxBounces + 1]
     // per-microphone receiver test (ST_LOS_PER_MIC): M queries per record (query = record id * M + m), the
     // record's bit m of rec_mask set when microphone m is visible; null rec_mask: one query per record
     uint64_t* rec_mask; const float* mics; int32_t M;

@@ -7,15 +7,13 @@
 // distance, so a box is never rejected when the float32 triangle test would hit inside it; the closest
 // hit is the smallest (t, triangle index), which makes the result independent of the tree's shape.
 //
-// Bounces run as a wavefront over a compacted queue of live rays, three launches per bounce: closest
-// hits, shading (reflection, float64 path length, the record [ray][bounce], the next queue and the
-// visibility queue), and the visibility rays (to the receiver reference point, or one per microphone
-// with the per-microphone receiver test).  The traversal kernels are persistent with lane refill: a
-// query advances one wide node or one leaf triangle per step, and a lane whose query has finished takes
-// the next one from a warp-aggregated atomic counter while the other lanes of its warp continue.  In
-// large scenes the visibility queue is sorted by the Morton code of the hit points first.  Results do not
-// depend on the order: closest hits are the smallest (t, triangle index), visibility is the absence of
-// any hit in the segment.
+// Bounces run as a wavefront, one launch per bounce and one more: launch j traces the closest hits of bounce j's live
+// rays and, beside them, the visibility rays of bounce j - 1's records (to the receiver reference point, or one per
+// microphone), and shades its hits itself (reflection, float64 path length, the record [ray][bounce], the next live
+// queue and the next launch's visibility queue).  The kernel is persistent with lane refill: a query advances one wide
+// node or one leaf triangle per step, and a lane whose query has finished takes the next one from a warp-aggregated
+// atomic counter while the other lanes of its warp continue.  Results do not depend on the order: closest hits are the
+// smallest (t, triangle index), visibility is the absence of any hit in the segment.
 // Compiled with -fmad=false (see st_geom.cuh).
 #include <algorithm>
 
@@ -45,128 +43,156 @@ __host__ __device__ __forceinline__ Trav trav_of(const A& a) {
 // (the object-space ray and the instance state take more registers)
 #define ST_TRAV_BOUNDS __launch_bounds__(kTravBlock, TL ? 6 : 8)
 
-// Closest hits of one bounce: item idx of the live-ray queue (the first bounce in direction order).
+// One bounce: closest hits of its live rays (the first bounce: all rays, in direction order), shaded when a lane is
+// refilled, and the visibility queries of the bounce before.  Closest hits are claimed first.
+// Bound by instruction issue over divergent lanes, and in small calls by the longest query: separate launches for closest
+// hits, shading and visibility waited for their slowest query twice a bounce and ran the tail of each alone.  10k rays x
+// 3 in the empty room 226 -> 182 us a call, 60k x 4 in light clutter 577 -> 439 us, 100k x 3 in a forest 4726 -> 3598 us,
+// 1M x 4 among 1M leaf triangles 15.8 -> 14.6 ms.  (Sorting the visibility queue of large scenes by hit point is gone with
+// it: the sort saved 4 % of their tracing and cost as much in launches.)
 template <bool TL>
-__global__ void ST_TRAV_BOUNDS k_closest(const TraceArgs a, int j, int64_t n_first) {
+__global__ void ST_TRAV_BOUNDS k_bounce(const TraceArgs a, int j, int lanes) {
     const Trav T = trav_of(a);
-    const int64_t n = (j == 0) ? n_first : (int64_t)*a.n_in;
+    const int64_t n_closest = j == 0 ? a.N : (j < a.B ? (int64_t)a.n_live[j] : 0);
+    const int64_t n_all = n_closest + (j > 0 ? (int64_t)a.n_vis[j - 1] : 0);
+    const uint32_t* vis_in = a.vis_q[(j & 1) ^ 1];
     const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int refill = min(T.refill > 0 ? T.refill : kRefillClosest, max(1, lanes / 2));
     int2 stack[kStack];
     typename TravStateOf<TL>::type S;
-    int64_t ray = -1;
-    bool live = false, exhausted = false;
+    uint32_t id = 0;  // ray of a closest-hit query, record of a visibility query
+    int m = 0;
+    bool live = false, hit = false, exhausted = lane >= lanes;
     while (true) {
+        if (hit) {  // Algorithm 1's steps after the hit: record, visibility queue, next queue
+            hit = false;
+            const int32_t tri = S.best;
+            const float t = S.tb;
+            f3 o, d;
+            double r;
+            if (j == 0) {
+                o = f3{a.s[0], a.s[1], a.s[2]};
+                d = rotate(a.q, f3{a.dirs[3 * (size_t)id], a.dirs[3 * (size_t)id + 1], a.dirs[3 * (size_t)id + 2]});
+                r = 0.0;
+            } else {
+                o = f3{a.ox[id], a.oy[id], a.oz[id]};
+                d = f3{a.dx[id], a.dy[id], a.dz[id]};
+                r = a.racc[id];
+            }
+            const float tdx = t * d.x, tdy = t * d.y, tdz = t * d.z;
+            const f3 P{o.x + tdx, o.y + tdy, o.z + tdz};
+            const f3 nv{a.nrm[3 * (size_t)tri], a.nrm[3 * (size_t)tri + 1], a.nrm[3 * (size_t)tri + 2]};
+            const float dn = dot(d, nv);
+            const float k2 = 2.0f * dn;
+            const float knx = k2 * nv.x, kny = k2 * nv.y, knz = k2 * nv.z;
+            float len;
+            const f3 dr = normalize(f3{d.x - knx, d.y - kny, d.z - knz}, &len);
+            r = r + (double)t;
+            const size_t rec = (size_t)id * a.B + j;
+            a.rec_tri[rec] = tri;
+            a.rec_los[rec] = 0;
+            a.rec_r[rec] = r;
+            a.rec_p[3 * rec] = P.x;
+            a.rec_p[3 * rec + 1] = P.y;
+            a.rec_p[3 * rec + 2] = P.z;
+            a.rec_d[3 * rec] = dr.x;
+            a.rec_d[3 * rec + 1] = dr.y;
+            a.rec_d[3 * rec + 2] = dr.z;
+            // warp-aggregated appends: the record's visibility queries (M with the per-microphone test) ...
+            const unsigned active = __activemask();
+            const int leader = __ffs(active) - 1, before = __popc(active & ((1u << lane) - 1u));
+            const uint32_t per = a.rec_mask ? (uint32_t)a.M : 1u;
+            uint32_t base = 0;
+            if (lane == leader) base = atomicAdd(a.n_vis + j, (uint32_t)__popc(active) * per);
+            base = __shfl_sync(active, base, leader) + (uint32_t)before * per;
+            uint32_t* vis_out = a.vis_q[j & 1];
+            if (a.rec_mask) {
+                a.rec_mask[rec] = 0ull;
+                for (uint32_t q = 0; q < per; ++q) vis_out[base + q] = (uint32_t)rec * per + q;
+            } else {
+                vis_out[base] = (uint32_t)rec;
+            }
+            if (r < a.r_max && j + 1 < a.B) {  // ... and the live ray
+                a.ox[id] = P.x;
+                a.oy[id] = P.y;
+                a.oz[id] = P.z;
+                a.dx[id] = dr.x;
+                a.dy[id] = dr.y;
+                a.dz[id] = dr.z;
+                a.racc[id] = r;
+                a.prev[id] = tri;
+                const unsigned act = __activemask();
+                const int lead = __ffs(act) - 1;
+                uint32_t at = 0;
+                if (lane == lead) at = atomicAdd(a.n_live + j + 1, (uint32_t)__popc(act));
+                at = __shfl_sync(act, at, lead);
+                a.live_q[(j + 1) & 1][at + __popc(act & ((1u << lane) - 1u))] = id;
+            }
+        }
+        __syncwarp();
         const bool need = !live && !exhausted;
-        const int64_t idx = claim(a.ctr + 0, need);
+        const int64_t idx = claim(a.ctr + j, need);
         if (need) {
-            if (idx < n) {
-                ray = (j == 0) ? (a.perm ? (int64_t)a.perm[idx] : idx) : (int64_t)a.q_in[idx];
+            if (idx < n_closest) {
+                id = j == 0 ? (a.perm ? a.perm[idx] : (uint32_t)idx) : a.live_q[j & 1][idx];
+                warp_count(a.queries + 0);
                 f3 o, d;
                 int32_t prev;
                 if (j == 0) {
                     o = f3{a.s[0], a.s[1], a.s[2]};
-                    d = rotate(a.q, f3{a.dirs[3 * ray], a.dirs[3 * ray + 1], a.dirs[3 * ray + 2]});
+                    d = rotate(a.q, f3{a.dirs[3 * (size_t)id], a.dirs[3 * (size_t)id + 1], a.dirs[3 * (size_t)id + 2]});
                     prev = -1;
                 } else {
-                    o = f3{a.ox[ray], a.oy[ray], a.oz[ray]};
-                    d = f3{a.dx[ray], a.dy[ray], a.dz[ray]};
-                    prev = a.prev[ray];
+                    o = f3{a.ox[id], a.oy[id], a.oz[id]};
+                    d = f3{a.dx[id], a.dy[id], a.dz[id]};
+                    prev = a.prev[id];
                 }
                 trav_init(S, T, o, d, prev, a.t_min, __int_as_float(0x7f800000));
                 live = true;
+            } else if (idx < n_all) {
+                id = vis_in[idx - n_closest];
+                const float* to = a.R;
+                if (a.rec_mask) {  // the entry is record * M + microphone
+                    m = (int)(id % (uint32_t)a.M);
+                    id /= (uint32_t)a.M;
+                    to = a.mics + 3 * m;
+                }
+                warp_count(a.queries + 1);
+                const f3 o{a.rec_p[3 * (size_t)id], a.rec_p[3 * (size_t)id + 1], a.rec_p[3 * (size_t)id + 2]};
+                float L;
+                const f3 u = normalize(sub(f3{to[0], to[1], to[2]}, o), &L);
+                const float tmax = L - a.los_eps;
+                if (!(tmax > a.t_min)) {
+                    if (a.rec_mask) atomicOr(reinterpret_cast<unsigned long long*>(&a.rec_mask[id]), 1ull << m);
+                    a.rec_los[id] = 1;
+                } else {
+                    trav_init(S, T, o, u, a.rec_tri[id], a.t_min, tmax);
+                    S.any = true;
+                    live = true;
+                }
             } else {
                 exhausted = true;
             }
         }
-        if (__ballot_sync(full, live) == 0u) break;
+        const unsigned lv0 = __ballot_sync(full, live);
+        const unsigned nd0 = __ballot_sync(full, !live && !exhausted);
+        if (lv0 == 0u && nd0 == 0u) break;
         while (true) {
-            if (live && trav_step<false>(T, S, stack, a.flags)) {
-                trav_count<false>(T, S);
-                a.hit_tri[ray] = S.best;
-                a.hit_t[ray] = S.tb;
+            if (live && trav_step<kMixed>(T, S, stack, a.flags)) {
+                trav_count_mixed(T, S);
                 live = false;
+                if (!S.any) {
+                    hit = S.best >= 0;
+                    ST_CHECK_OR(S.best < a.chk[5], a.flags, hit = false);
+                } else if (S.best < 0) {
+                    if (a.rec_mask) atomicOr(reinterpret_cast<unsigned long long*>(&a.rec_mask[id]), 1ull << m);
+                    a.rec_los[id] = 1;
+                }
             }
             const unsigned lv = __ballot_sync(full, live);
             const unsigned nd = __ballot_sync(full, !live && !exhausted);
-            if (lv == 0u || __popc(nd) >= (T.refill > 0 ? T.refill : kRefillClosest)) break;
-        }
-    }
-}
-
-// Shading of one bounce: record, next queue, visibility queue (Algorithm 1's steps after the hit).
-__global__ void k_shade(const TraceArgs a, int j, int64_t n_first) {
-    const int64_t n_live = (j == 0) ? n_first : (int64_t)*a.n_in;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n_live; idx += stride) {
-        const int64_t ray = (j == 0) ? (a.perm ? (int64_t)a.perm[idx] : idx) : (int64_t)a.q_in[idx];
-        warp_count(a.queries + 0);
-        const int32_t tri = a.hit_tri[ray];
-        if (tri < 0) continue;
-        ST_CHECK_OR(tri < a.chk[5], a.flags, continue);
-        const float t = a.hit_t[ray];
-        f3 o, d;
-        double r;
-        if (j == 0) {
-            o = f3{a.s[0], a.s[1], a.s[2]};
-            d = rotate(a.q, f3{a.dirs[3 * ray], a.dirs[3 * ray + 1], a.dirs[3 * ray + 2]});
-            r = 0.0;
-        } else {
-            o = f3{a.ox[ray], a.oy[ray], a.oz[ray]};
-            d = f3{a.dx[ray], a.dy[ray], a.dz[ray]};
-            r = a.racc[ray];
-        }
-        const float tdx = t * d.x, tdy = t * d.y, tdz = t * d.z;
-        const f3 P{o.x + tdx, o.y + tdy, o.z + tdz};
-        const f3 nv{a.nrm[3 * tri], a.nrm[3 * tri + 1], a.nrm[3 * tri + 2]};
-        const float dn = dot(d, nv);
-        const float k2 = 2.0f * dn;
-        const float knx = k2 * nv.x, kny = k2 * nv.y, knz = k2 * nv.z;
-        float len;
-        const f3 dr = normalize(f3{d.x - knx, d.y - kny, d.z - knz}, &len);
-        r = r + (double)t;
-        const int64_t id = ray * a.B + j;
-        a.rec_tri[id] = tri;
-        a.rec_los[id] = 0;
-        a.rec_r[id] = r;
-        a.rec_p[3 * id] = P.x;
-        a.rec_p[3 * id + 1] = P.y;
-        a.rec_p[3 * id + 2] = P.z;
-        a.rec_d[3 * id] = dr.x;
-        a.rec_d[3 * id + 1] = dr.y;
-        a.rec_d[3 * id + 2] = dr.z;
-        const int lane = threadIdx.x & 31;
-        if (a.rec_mask) {  // one visibility query per microphone (warp-aggregated append of M entries a lane)
-            a.rec_mask[id] = 0ull;
-            const unsigned active = __activemask();
-            const int leader = __ffs(active) - 1;
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(a.vis_n, (uint32_t)__popc(active) * (uint32_t)a.M);
-            base = __shfl_sync(active, base, leader);
-            const uint32_t q0 = base + (uint32_t)__popc(active & ((1u << lane) - 1u)) * (uint32_t)a.M;
-            for (int m = 0; m < a.M; ++m) a.vis_q[q0 + m] = (uint32_t)id * (uint32_t)a.M + (uint32_t)m;
-        } else {  // visibility query of this record (warp-aggregated append)
-            const unsigned active = __activemask();
-            const int leader = __ffs(active) - 1;
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(a.vis_n, (uint32_t)__popc(active));
-            base = __shfl_sync(active, base, leader);
-            a.vis_q[base + __popc(active & ((1u << lane) - 1u))] = (uint32_t)id;
-        }
-        if (r < a.r_max && j + 1 < a.B) {
-            a.ox[ray] = P.x;
-            a.oy[ray] = P.y;
-            a.oz[ray] = P.z;
-            a.dx[ray] = dr.x;
-            a.dy[ray] = dr.y;
-            a.dz[ray] = dr.z;
-            a.racc[ray] = r;
-            a.prev[ray] = tri;
-            const unsigned active = __activemask();
-            const int leader = __ffs(active) - 1;
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(a.n_out, (uint32_t)__popc(active));
-            base = __shfl_sync(active, base, leader);
-            a.q_out[base + __popc(active & ((1u << lane) - 1u))] = (uint32_t)ray;
+            if (lv == 0u || __popc(nd) >= refill) break;
         }
     }
 }
@@ -180,14 +206,15 @@ __global__ void ST_TRAV_BOUNDS k_visible(const Trav T, const uint32_t* queue, co
                                                            const float* tgt_dev, float tx, float ty, float tz,
                                                            float t_min, float eps, uint8_t* out,
                                                            unsigned long long* ctr, uint32_t* flags,
-                                                           unsigned long long* queries) {
+                                                           unsigned long long* queries, int lanes) {
     const int64_t n = *count;
     const unsigned full = 0xffffffffu;
     const f3 target = tgt_dev ? f3{tgt_dev[0], tgt_dev[1], tgt_dev[2]} : f3{tx, ty, tz};
     int2 stack[kStack];
     typename TravStateOf<TL>::type S;
     int64_t id = -1;
-    bool live = false, exhausted = false;
+    bool live = false, exhausted = (int)(threadIdx.x & 31) >= lanes;
+    const int refill = min(T.refill > 0 ? T.refill : kRefillAny, max(1, lanes - 4));
     while (true) {
         const bool need = !live && !exhausted;
         const int64_t idx = claim(ctr, need);
@@ -213,70 +240,14 @@ __global__ void ST_TRAV_BOUNDS k_visible(const Trav T, const uint32_t* queue, co
         const unsigned nd0 = __ballot_sync(full, !live && !exhausted);
         if (lv0 == 0u && nd0 == 0u) break;
         while (true) {
-            if (live && trav_step<true>(T, S, stack, flags)) {
+            if (live && trav_step<kAny>(T, S, stack, flags)) {
                 trav_count<true>(T, S);
                 out[id] = S.best < 0 ? 1 : 0;
                 live = false;
             }
             const unsigned lv = __ballot_sync(full, live);
             const unsigned nd = __ballot_sync(full, !live && !exhausted);
-            if (lv == 0u || __popc(nd) >= (T.refill > 0 ? T.refill : kRefillAny)) break;
-        }
-    }
-}
-
-// Per-microphone receiver test: query q of the queue is record q / M and microphone q % M; a visible
-// microphone sets its bit of the record's mask (and the record's flag: some microphone sees it).
-template <bool TL>
-__global__ void ST_TRAV_BOUNDS k_visible_mics(const TraceArgs a, unsigned long long* ctr) {
-    const Trav T = trav_of(a);
-    const int64_t n = *a.vis_n;
-    const unsigned full = 0xffffffffu;
-    int2 stack[kStack];
-    typename TravStateOf<TL>::type S;
-    int64_t id = -1;
-    int m = 0;
-    bool live = false, exhausted = false;
-    while (true) {
-        const bool need = !live && !exhausted;
-        const int64_t idx = claim(ctr, need);
-        if (need) {
-            if (idx < n) {
-                const uint32_t q = a.vis_q[idx];
-                id = (int64_t)(q / (uint32_t)a.M);
-                m = (int)(q - (uint32_t)id * (uint32_t)a.M);
-                warp_count(a.queries + 1);
-                const f3 o{a.rec_p[3 * id], a.rec_p[3 * id + 1], a.rec_p[3 * id + 2]};
-                const f3 target{a.mics[3 * m], a.mics[3 * m + 1], a.mics[3 * m + 2]};
-                float L;
-                const f3 u = normalize(sub(target, o), &L);
-                const float tmax = L - a.los_eps;
-                if (!(tmax > a.t_min)) {
-                    atomicOr(reinterpret_cast<unsigned long long*>(&a.rec_mask[id]), 1ull << m);
-                    a.rec_los[id] = 1;
-                } else {
-                    trav_init(S, T, o, u, a.rec_tri[id], a.t_min, tmax);
-                    live = true;
-                }
-            } else {
-                exhausted = true;
-            }
-        }
-        const unsigned lv0 = __ballot_sync(full, live);
-        const unsigned nd0 = __ballot_sync(full, !live && !exhausted);
-        if (lv0 == 0u && nd0 == 0u) break;
-        while (true) {
-            if (live && trav_step<true>(T, S, stack, a.flags)) {
-                trav_count<true>(T, S);
-                if (S.best < 0) {
-                    atomicOr(reinterpret_cast<unsigned long long*>(&a.rec_mask[id]), 1ull << m);
-                    a.rec_los[id] = 1;
-                }
-                live = false;
-            }
-            const unsigned lv = __ballot_sync(full, live);
-            const unsigned nd = __ballot_sync(full, !live && !exhausted);
-            if (lv == 0u || __popc(nd) >= (T.refill > 0 ? T.refill : kRefillAny)) break;
+            if (lv == 0u || __popc(nd) >= refill) break;
         }
     }
 }
@@ -399,28 +370,6 @@ __device__ __forceinline__ uint32_t spread10(uint32_t x) {
     return x;
 }
 
-// Morton code (kVisBits per axis) of the hit point of every queued visibility query, 2^(3 kVisBits) past the
-// count (10 bits measured faster than 5 or 7 on the vegetation workload, the sort included)
-constexpr int kVisBits = 10;
-__global__ void k_vis_keys(const TraceArgs a, uint64_t* keys) {
-    const int64_t n = *a.vis_n;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < a.N; c += stride) {
-        uint64_t key = 1ull << (3 * kVisBits);
-        if (c < n) {
-            const int64_t id = a.vis_q[c];
-            const float cells = (float)(1 << kVisBits);
-            uint32_t m = 0;
-            for (int k = 0; k < 3; ++k) {
-                const float u = (a.rec_p[3 * id + k] - a.blo[k]) * a.bscale[k] * (cells * (1.0f / 1024.0f));
-                m |= spread10((uint32_t)fminf(fmaxf(u, 0.0f), cells - 1.0f)) << (2 - k);
-            }
-            key = m;
-        }
-        keys[c] = key;
-    }
-}
-
 // Morton code (kLosBits per axis) of the candidate point of every queued line-of-sight query
 constexpr int kLosBits = 10;  // swept 0, 5, 10 bits: 10 fastest on the clutter workload (5 on vegetation)
 __global__ void k_los_keys(const DiffArgs a, uint64_t* keys) {
@@ -484,55 +433,33 @@ cudaError_t direction_order(const float* dirs, int64_t n, uint64_t* keys, uint32
     return radix_sort_u64(keys, perm, n, 32, scratch, s);
 }
 
-// persistent traversal grid: one CTA per resident slot (eight per SM on flat scenes, six on two-level ones)
-static unsigned trav_grid(int64_t n, bool tl) {
-    const int64_t full = 152 * (tl ? 6 : 8);
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(full, (n + kTravBlock - 1) / kTravBlock));
+// Persistent traversal grid for at most n queries: one CTA per resident slot (eight per SM on flat scenes, six on
+// two-level ones).  Below one query per lane of that grid the queries are spread over all its warps, a few lanes each
+// (at least four): a warp's step then serialises fewer different paths, and the launch ends when its longest query does.
+struct TravGrid {
+    unsigned ctas;
+    int lanes;
+};
+static TravGrid trav_grid(int64_t n, bool tl, int block = kTravBlock) {
+    const int64_t full = 152 * (tl ? 6 : 8) * (kTravBlock / block), warps = full * (block / 32);
+    const int lanes = (int)std::min<int64_t>(32, std::max<int64_t>(4, (n + warps - 1) / warps));
+    const int64_t per = (int64_t)lanes * (block / 32);
+    return TravGrid{(unsigned)std::max<int64_t>(1, std::min<int64_t>(full, (n + per - 1) / per)), lanes};
 }
 
 cudaError_t trace_rays(TraceArgs& a, cudaStream_t s, int block) {
-    const unsigned grid = grid_for(a.N, block, 152 * 16);
-    const Trav T = trav_of(a);
     const bool tl = a.inst != nullptr;
-    for (int j = 0; j < a.B; ++j) {
-        if (j > 0) {
-            uint32_t* t = a.q_in;
-            a.q_in = a.q_out;
-            a.q_out = t;
-            uint32_t* c = a.n_in;
-            a.n_in = a.n_out;
-            a.n_out = c;
-        }
-        cudaError_t e = cudaMemsetAsync(a.n_out, 0, sizeof(uint32_t), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(a.vis_n, 0, sizeof(uint32_t), s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(a.ctr, 0, 2 * sizeof(unsigned long long), s);
-        if (e != cudaSuccess) return e;
+    const int threads = std::min(block, kTravBlock);
+    for (int j = 0; j <= a.B; ++j) {
+        const int64_t most = (j < a.B ? a.N : 0) + (j > 0 ? a.N * (a.rec_mask ? a.M : 1) : 0);
+        const TravGrid g = trav_grid(most, tl, threads);
         note_launch();
         if (tl)
-            k_closest<true><<<trav_grid(a.N, true), kTravBlock, 0, s>>>(a, j, a.N);
+            k_bounce<true><<<g.ctas, threads, 0, s>>>(a, j, g.lanes);
         else
-            k_closest<false><<<trav_grid(a.N, false), kTravBlock, 0, s>>>(a, j, a.N);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        note_launch();
-        k_shade<<<grid, block, 0, s>>>(a, j, a.N);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (a.sort_keys) {  // stable sort: equal codes keep the queue order
-            note_launch();
-            k_vis_keys<<<grid_for(a.N, 256), 256, 0, s>>>(a, a.sort_keys);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if ((e = radix_sort_u64(a.sort_keys, a.vis_q, a.N, 3 * kVisBits + 1, a.sort_scr, s)) != cudaSuccess)
-                return e;
-        }
-        note_launch();
-        if (a.rec_mask && tl)
-            k_visible_mics<true><<<trav_grid(a.N * a.M, true), kTravBlock, 0, s>>>(a, a.ctr + 1);
-        else if (a.rec_mask)
-            k_visible_mics<false><<<trav_grid(a.N * a.M, false), kTravBlock, 0, s>>>(a, a.ctr + 1);
-        else
-            (tl ? k_visible<true> : k_visible<false>)<<<trav_grid(a.N, tl), kTravBlock, 0, s>>>(
-                T, a.vis_q, a.vis_n, a.rec_p, a.rec_tri, a.R, 0.0f, 0.0f, 0.0f, a.t_min, a.los_eps, a.rec_los,
-                a.ctr + 1, a.flags, a.queries);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            k_bounce<false><<<g.ctas, threads, 0, s>>>(a, j, g.lanes);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -554,9 +481,10 @@ cudaError_t diffraction_sample(DiffArgs& a, cudaStream_t s) {
     const Trav T = trav_of(a);
     const bool tl = a.inst != nullptr;
     note_launch();
-    (tl ? k_visible<true> : k_visible<false>)<<<trav_grid(a.K, tl), kTravBlock, 0, s>>>(
+    const TravGrid g = trav_grid(a.K, tl);
+    (tl ? k_visible<true> : k_visible<false>)<<<g.ctas, kTravBlock, 0, s>>>(
         T, a.los_q, a.los_n, a.cand_p, a.cand_tri, nullptr, a.s[0], a.s[1], a.s[2], a.t_min, a.los_eps, a.keep, a.ctr,
-        a.flags, a.queries);
+        a.flags, a.queries, g.lanes);
     return cudaGetLastError();
 }
 

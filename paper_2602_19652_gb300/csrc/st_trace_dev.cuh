@@ -56,11 +56,16 @@ __device__ __forceinline__ bool slab(float lx, float ly, float lz, float hx, flo
 
 // Resumable traversal: the state of one query, advanced by one wide node or one leaf triangle per step, so that
 // a kernel can give a finished lane a new query while the other lanes of its warp continue.
+// What a query looks for: the closest hit, any hit, or (kMixed) whichever its `any` says, in a kernel whose lanes hold
+// queries of both kinds
+constexpr int kClosest = 0, kAny = 1, kMixed = 2;
+
 struct TravState {
     WRay wr;
     f3 o, inv;
     int32_t exclude;
     float t_min, t_max, tb;  // closest: tb = best t so far (+inf at first); any-hit: segment end (exclusive)
+    bool any;                // kMixed: an any-hit query
     int32_t best, ref;
     int sp, guard, n_nodes, n_tris;
 };
@@ -77,6 +82,7 @@ __device__ __forceinline__ void trav_init(TravState& S, const Trav& T, f3 o, f3 
     S.best = -1;
     S.ref = T.root;
     S.sp = 0;
+    S.any = false;
     // every node of a proper tree is visited at most once: more iterations than nodes means a
     // malformed hierarchy, reported through the flags instead of looping
     S.guard = T.max_iter;
@@ -86,7 +92,7 @@ __device__ __forceinline__ void trav_init(TravState& S, const Trav& T, f3 o, f3 
 
 // one triangle of a leaf (leaf code: first triangle << 3 | triangles left after it); true when an any-hit
 // query has found its hit.  S.ref becomes the code of the next triangle, or `after` when the leaf is done.
-template <bool AnyHit>
+template <int Hit>
 __device__ __forceinline__ bool leaf_step(const Trav& T, TravState& S, int32_t after) {
     const int32_t code = ~S.ref;
     const int i = code >> 3, rest = code & 7;
@@ -98,8 +104,8 @@ __device__ __forceinline__ bool leaf_step(const Trav& T, TravState& S, int32_t a
         ++S.n_tris;
         float th;
         if (wt_hit(S.wr, f3{v0.x, v0.y, v0.z}, f3{v1.x, v1.y, v1.z}, f3{v2.x, v2.y, v2.z}, &th) && th > S.t_min) {
-            if (AnyHit) {
-                if (th < S.t_max) {
+            if (Hit == kMixed ? S.any : Hit == kAny) {
+                if (th < S.tb) {  // (an any-hit query's tb is the segment's end until its hit)
                     S.tb = th;
                     S.best = id;
                     return true;
@@ -115,7 +121,7 @@ __device__ __forceinline__ bool leaf_step(const Trav& T, TravState& S, int32_t a
 }
 
 // one node or one leaf triangle; true when the query has finished (S.best = hit triangle or -1, S.tb = its t)
-template <bool AnyHit>
+template <int Hit>
 __device__ __forceinline__ bool trav_step(const Trav& T, TravState& S, int2* stack, uint32_t* flags) {
     if (--S.guard < 0) {
         atomicOr(flags, kFlagBadTree);
@@ -203,7 +209,7 @@ __device__ __forceinline__ bool trav_step(const Trav& T, TravState& S, int2* sta
         // one triangle of a leaf per step, so lanes in leaves and lanes in inner nodes of the same warp stay
         // in step
         ST_CHECK_OR((int64_t)((~S.ref) >> 3) + ((~S.ref) & 7) < T.chk[1], flags, return true);
-        if (leaf_step<AnyHit>(T, S, 1)) return true;
+        if (leaf_step<Hit>(T, S, 1)) return true;
         if (S.ref < 0) return false;
         if (S.sp < 0) {  // restart walk: back to the node that holds the leaf
             S.ref = stack[0].x;
@@ -313,7 +319,7 @@ __device__ __forceinline__ void tl_restart(const Trav& T, TravStateTL& S, int2* 
 }
 
 // one triangle of a prototype leaf, tested in world space
-template <bool AnyHit>
+template <int Hit>
 __device__ __forceinline__ bool leaf_step_tl(const Trav& T, TravStateTL& S, int32_t after) {
     const int32_t code = ~S.ref;
     const int i = code >> 3, rest = code & 7;
@@ -330,8 +336,8 @@ __device__ __forceinline__ bool leaf_step_tl(const Trav& T, TravStateTL& S, int3
         const f3 w2{affine_row(f0, v2.x, v2.y, v2.z), affine_row(f1, v2.x, v2.y, v2.z), affine_row(f2, v2.x, v2.y, v2.z)};
         float th;
         if (wt_hit(S.wr, w0, w1, w2, &th) && th > S.t_min) {
-            if (AnyHit) {
-                if (th < S.t_max) {
+            if (Hit == kMixed ? S.any : Hit == kAny) {
+                if (th < S.tb) {  // (an any-hit query's tb is the segment's end until its hit)
                     S.tb = th;
                     S.best = id;
                     return true;
@@ -347,7 +353,7 @@ __device__ __forceinline__ bool leaf_step_tl(const Trav& T, TravStateTL& S, int3
 }
 
 // one node (either level), one instance of a top-level leaf or one prototype triangle; true when finished
-template <bool AnyHit>
+template <int Hit>
 __device__ __forceinline__ bool trav_step(const Trav& T, TravStateTL& S, int2* stack, uint32_t* flags) {
     if (--S.guard < 0) {
         atomicOr(flags, kFlagBadTree);
@@ -421,7 +427,7 @@ __device__ __forceinline__ bool trav_step(const Trav& T, TravStateTL& S, int2* s
         }
     } else if (in) {
         ST_CHECK_OR((int64_t)((~S.ref) >> 3) + ((~S.ref) & 7) < T.chk[3], flags, return true);
-        if (leaf_step_tl<AnyHit>(T, S, 1)) return true;
+        if (leaf_step_tl<Hit>(T, S, 1)) return true;
         if (S.ref < 0) return false;
         if (S.sp < 0) {
             if (S.broot < 0) tl_exit_stackless(S, stack);  // the prototype's BVH is this one leaf
@@ -504,11 +510,16 @@ __device__ __forceinline__ int32_t traverse(const Trav& T, f3 o, f3 d, int32_t e
     typename TravStateOf<TL>::type S;
     int2 stack[kStack];
     trav_init(S, T, o, d, exclude, t_min, t_max);
-    while (!trav_step<AnyHit>(T, S, stack, flags)) {
+    while (!trav_step<AnyHit ? kAny : kClosest>(T, S, stack, flags)) {
     }
     trav_count<AnyHit>(T, S);
     *t_out = S.tb;
     return S.best;
+}
+
+// as above for a query of either kind
+__device__ __forceinline__ void trav_count_mixed(const Trav& T, const TravState& S) {
+    if (S.any) trav_count<true>(T, S); else trav_count<false>(T, S);
 }
 
 // Lane refill (persistent traversal kernels): the lanes that need a query claim consecutive indices

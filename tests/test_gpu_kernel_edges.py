@@ -102,3 +102,19 @@ def test_general_tile_bin_blocks_match_oracle(torch_st, n_mics, n_bins):
     _, st = torch_st
     wl = synth.clutter(seed=14, target_tris=2_500, n_rays=1_200, bounces=3, n_mics=n_mics, n_bins=n_bins)
     simulate_and_compare(st, wl, budget=3_000)
+
+
+# fused bounce launches: one ray, fewer queries than warps, a few lanes a warp, full warps; the last launch (visibility
+# only) after a single bounce and after the most; both receiver tests
+@pytest.mark.parametrize("n_rays,bounces,los", [(1, 1, 0), (33, 8, 0), (20_001, 2, 0), (60_007, 3, 0), (170_003, 2, 0),
+                                                (3_001, 3, 1), (9_001, 1, 1)])
+def test_bounce_queues_match_oracle(torch_st, n_rays, bounces, los):
+    _, st = torch_st
+    wl = synth.clutter(seed=21, target_tris=3_000, n_rays=n_rays, bounces=bounces, n_mics=5, n_bins=9, diffraction=False)
+    wl.mics = (wl.mics + np.random.default_rng(6).uniform(-5, 5, wl.mics.shape) * [1, 1, 0.1]).astype(np.float32)
+    ctx, _, _, ref = simulate_and_compare(st, wl, los_mode=los, components=st.ST_COMP_SPECULAR | st.ST_COMP_DIRECT)
+    g = ctx.paths(bounces)
+    for k in ("p", "d", "r"):
+        assert np.array_equal(g[k][ref["rec"]["tri"] >= 0], ref["rec"][k][ref["rec"]["tri"] >= 0]), k
+    if los:
+        assert np.array_equal(ctx.receiver_masks(bounces), ref["rec"]["mask"])
