@@ -662,16 +662,16 @@ __global__ void __launch_bounds__(kMmaMics * 32, 2) k_adjoint_diff_mma(const Acc
     }
 }
 
-// material key of every compacted diffraction candidate (past the count: a key above every material)
-__global__ void k_mat_keys(const uint32_t* idx, const uint32_t* count, int64_t cap, const int32_t* cand_tri,
-                           const int32_t* tri_mat, uint64_t* keys) {
+// material key of every compacted diffraction candidate
+__global__ void k_mat_keys(const uint32_t* idx, const uint32_t* count, const int32_t* cand_tri, const int32_t* tri_mat,
+                           uint32_t* keys) {
     const int64_t n = *count;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < cap; c += (int64_t)gridDim.x * blockDim.x)
-        keys[c] = c < n ? (uint64_t)((uint32_t)tri_mat[cand_tri[idx[c]]] & 255u) : 256ull;
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += (int64_t)gridDim.x * blockDim.x)
+        keys[c] = (uint32_t)tri_mat[cand_tri[idx[c]]] & 255u;
 }
 
 // first position of each material in the sorted keys, and the count at the end
-__global__ void k_mat_offsets(const uint64_t* keys, const uint32_t* count, int n_mat, uint32_t* off) {
+__global__ void k_mat_offsets(const uint32_t* keys, const uint32_t* count, int n_mat, uint32_t* off) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q > n_mat) return;
     const int64_t n = *count;
@@ -682,7 +682,7 @@ __global__ void k_mat_offsets(const uint64_t* keys, const uint32_t* count, int n
     int64_t lo = 0, hi = n;  // lower bound of key q
     while (lo < hi) {
         const int64_t mid = (lo + hi) >> 1;
-        if (keys[mid] < (uint64_t)q) lo = mid + 1;
+        if (keys[mid] < (uint32_t)q) lo = mid + 1;
         else hi = mid;
     }
     off[q] = (uint32_t)lo;
@@ -757,13 +757,13 @@ size_t material_order_scratch(int64_t cap) { return (size_t)std::max<int64_t>(ca
 cudaError_t material_order(const uint32_t* count, int64_t cap, const int32_t* cand_tri, const int32_t* tri_mat,
                            int n_mat, uint32_t* idx, uint32_t* mat_off, void* scratch, cudaStream_t s) {
     if (cap <= 0) return cudaSuccess;
-    uint64_t* keys = static_cast<uint64_t*>(scratch);
+    uint32_t* keys = static_cast<uint32_t*>(scratch);
     void* sort_scr = static_cast<char*>(scratch) + (size_t)cap * 8;
     note_launch();
-    k_mat_keys<<<grid_for(cap, 256), 256, 0, s>>>(idx, count, cap, cand_tri, tri_mat, keys);
+    k_mat_keys<<<grid_for(cap, 256), 256, 0, s>>>(idx, count, cand_tri, tri_mat, keys);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if ((e = radix_sort_u64(keys, idx, cap, 9, sort_scr, s)) != cudaSuccess) return e;  // stable
+    if ((e = radix_sort_u32(keys, idx, cap, 0, 8, sort_scr, s, count)) != cudaSuccess) return e;  // stable
     note_launch();
     k_mat_offsets<<<(n_mat + 1 + 127) / 128, 128, 0, s>>>(keys, count, n_mat, mat_off);
     return cudaGetLastError();

@@ -96,7 +96,7 @@ struct st_ctx {
     double tables_key[5] = {0, 0, 0, 0, 0};
     // work buffers
     DevBuf st_o[3], st_d[3], st_r, st_prev, q0, q1, counts, queries, flags, R, rec_tri, rec_p, rec_d, rec_r, rec_los;
-    DevBuf sflags, sscan, sidx, scratch;
+    DevBuf sidx, scratch;
     PathList paths, paths_diff;  // gathered specular / diffraction paths of the last simulate
     DevBuf cand_tri, cand_p, keep, dvis, partial;
     DevBuf host_out;
@@ -127,7 +127,7 @@ struct st_ctx {
     bool overlap = true;
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    DevBuf los_keys, los_scr, dflags, dscan, didx, dscratch, dpartial;
+    DevBuf los_keys, los_scr, didx, dscratch, dpartial;
     // backward: the specular path list of the last simulate put in chain order (keys and sort scratch)
     bool paths_chain_order = false;
     DevBuf ck_keys, ck_scr;
@@ -386,7 +386,7 @@ st_status st_destroy(st_ctx* c) {
     for (DevBuf* b : {&c->mic_q, &c->mic_tab, &c->tables.bw}) release(*b);
     for (DevBuf* b : {&c->dirs, &c->etab, &c->perm, &c->ord_keys, &c->ord_scr, &c->th_keys, &c->th_scr, &c->mics, &c->st_o[0], &c->st_o[1], &c->st_o[2], &c->st_d[0], &c->st_d[1],
                       &c->st_d[2], &c->st_r, &c->st_prev, &c->q0, &c->q1, &c->counts, &c->queries, &c->flags, &c->R, &c->rec_tri,
-                      &c->rec_p, &c->rec_d, &c->rec_r, &c->rec_los, &c->sflags, &c->sscan, &c->sidx, &c->scratch,
+                      &c->rec_p, &c->rec_d, &c->rec_r, &c->rec_los, &c->sidx, &c->scratch,
                       &c->cand_tri, &c->cand_p, &c->keep, &c->dvis, &c->partial, &c->host_out, &c->mat_off, &c->mat_scr, &c->tables.lk,
                       &c->tables.g2, &c->tables.lid, &c->tables.qhi, &c->tables.qlo})
         release(*b);
@@ -401,7 +401,7 @@ st_status st_destroy(st_ctx* c) {
         release(*b);
     for (auto& e : c->ev)
         if (e) cudaEventDestroy(e);
-    for (DevBuf* b : {&c->los_keys, &c->los_scr, &c->dflags, &c->dscan, &c->didx, &c->dscratch, &c->dpartial,
+    for (DevBuf* b : {&c->los_keys, &c->los_scr, &c->didx, &c->dscratch, &c->dpartial,
                       &c->ck_keys, &c->ck_scr})
         release(*b);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -764,7 +764,7 @@ st_status st_set_emitter(st_ctx* c, const float pos[3], const float quat[4], int
         CKC(c, grow(c->perm, (size_t)n_rays * 4), "set_emitter alloc");
         CKC(c, grow(c->ord_keys, (size_t)n_rays * 8), "set_emitter alloc");
         CKC(c, grow(c->ord_scr, sort_scratch_bytes(n_rays)), "set_emitter alloc");
-        CKC(c, direction_order(ptr<float>(c->dirs), n_rays, ptr<uint64_t>(c->ord_keys), ptr<uint32_t>(c->perm),
+        CKC(c, direction_order(ptr<float>(c->dirs), n_rays, ptr<uint32_t>(c->ord_keys), ptr<uint32_t>(c->perm),
                                c->ord_scr.p, c->stream),
             "set_emitter order");
     }
@@ -894,7 +894,6 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
 
     // ---- buffers
     const int64_t K = (p.components & ST_COMP_DIFFRACTION) ? S.total_samples : 0;
-    const int64_t nflag = std::max<int64_t>(std::max<int64_t>(NB, K), 1);
     for (int k = 0; k < 3; ++k) {
         CKC(c, grow(c->st_o[k], (size_t)std::max<int64_t>(N, 1) * 4), "alloc");
         CKC(c, grow(c->st_d[k], (size_t)std::max<int64_t>(N, 1) * 4), "alloc");
@@ -919,11 +918,9 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
     CKC(c, grow(c->rec_p, (size_t)std::max<int64_t>(NB, 1) * 12), "alloc");
     CKC(c, grow(c->rec_d, (size_t)std::max<int64_t>(NB, 1) * 12), "alloc");
     CKC(c, grow(c->rec_r, (size_t)std::max<int64_t>(NB, 1) * 8), "alloc");
-    CKC(c, grow(c->rec_los, (size_t)std::max<int64_t>(NB, 1)), "alloc");
-    CKC(c, grow(c->sflags, (size_t)nflag * 4), "alloc");
-    CKC(c, grow(c->sscan, (size_t)nflag * 4), "alloc");
-    CKC(c, grow(c->sidx, (size_t)nflag * 4), "alloc");
-    CKC(c, grow(c->scratch, scan_scratch_bytes(nflag)), "alloc");
+    CKC(c, grow(c->rec_los, (size_t)std::max<int64_t>(NB, 1) + 3), "alloc");  // (whole words are cleared)
+    CKC(c, grow(c->sidx, (size_t)std::max<int64_t>(NB, 1) * 4), "alloc");
+    CKC(c, grow(c->scratch, compact_scratch_bytes(NB)), "alloc");
     if (K > 1) {  // the line-of-sight queue of the diffraction candidates is sorted by Morton code
         CKC(c, grow(c->los_keys, (size_t)K * 8), "alloc");
         CKC(c, grow(c->los_scr, sort_scratch_bytes(K)), "alloc");
@@ -964,28 +961,30 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
     }
     CKC(c, grow(c->partial, (size_t)chunks_spec * M * F * 8), "alloc");
     if (K > 0) {  // the diffraction stage's compaction and partial spectra (it may run beside the specular one)
-        CKC(c, grow(c->dflags, (size_t)K * 4), "alloc");
-        CKC(c, grow(c->dscan, (size_t)K * 4), "alloc");
         CKC(c, grow(c->didx, (size_t)K * 4), "alloc");
-        CKC(c, grow(c->dscratch, scan_scratch_bytes(K)), "alloc");
+        CKC(c, grow(c->dscratch, compact_scratch_bytes(K)), "alloc");
         CKC(c, grow(c->dpartial, (size_t)chunks_diff * M * F * 8), "alloc");
     }
 
     float2* out = static_cast<float2*>(spectra_out);
     const int64_t MF = (int64_t)M * F;
-    CKC(c, cudaMemsetAsync(out, 0, (size_t)3 * MF * 8, s), "memset out");
-    CKC(c, cudaMemsetAsync(c->flags.p, 0, 16, s), "memset");
-    CKC(c, cudaMemsetAsync(c->counts.p, 0, 64, s), "memset");
-    CKC(c, cudaMemsetAsync(c->trav_cnt.p, 0, kTravCounts, s), "memset");
-    CKC(c, cudaMemsetAsync(c->queries.p, 0, 64, s), "memset");
+    {  // one launch for all of a call's initial values (eleven memsets cost a small call a tenth of its time)
+        const size_t nb = (size_t)std::max<int64_t>(NB, 1);
+        const Fill f[] = {{out, (size_t)3 * MF * 8, 0u},
+                          {c->flags.p, 16, 0u},
+                          {c->counts.p, 64, 0u},
+                          {c->trav_cnt.p, kTravCounts, 0u},
+                          {c->queries.p, 64, 0u},
+                          {c->rec_tri.p, nb * 4, 0xffffffffu},
+                          {c->rec_los.p, (nb + 3) & ~size_t(3), 0u},
+                          {c->rec_mask.p, per_mic ? nb * 8 : 0, 0u},
+                          {c->rec_r.p, nb * 8, 0u},
+                          {c->rec_p.p, nb * 12, 0u},
+                          {c->rec_d.p, nb * 12, 0u}};
+        CKC(c, fill_many(f, (int)(sizeof(f) / sizeof(f[0])), s), "initial values");
+    }
     unsigned long long* qctr = ptr<unsigned long long>(c->queries);
-    CKC(c, cudaMemsetAsync(c->rec_tri.p, 0xff, (size_t)std::max<int64_t>(NB, 1) * 4, s), "memset");
-    CKC(c, cudaMemsetAsync(c->rec_los.p, 0, (size_t)std::max<int64_t>(NB, 1), s), "memset");
-    if (per_mic) CKC(c, cudaMemsetAsync(c->rec_mask.p, 0, (size_t)std::max<int64_t>(NB, 1) * 8, s), "memset");
-    CKC(c, cudaMemsetAsync(c->rec_r.p, 0, (size_t)std::max<int64_t>(NB, 1) * 8, s), "memset");
-    CKC(c, cudaMemsetAsync(c->rec_p.p, 0, (size_t)std::max<int64_t>(NB, 1) * 12, s), "memset");
-    CKC(c, cudaMemsetAsync(c->rec_d.p, 0, (size_t)std::max<int64_t>(NB, 1) * 12, s), "memset");
-    uint32_t* cnt = ptr<uint32_t>(c->counts);  // [0],[1] queue counts, [2] visible records, [3] kept candidates
+    uint32_t* cnt = ptr<uint32_t>(c->counts);  // [2] visible records, [3] kept candidates
     mic_centroid_host_order(ptr<float>(c->mics), M, ptr<float>(c->R), s);
     CKC(c, cudaGetLastError(), "centroid");
 
@@ -1122,7 +1121,7 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
             da.los_q = ptr<uint32_t>(c->los_q);
             da.los_n = ptr<uint32_t>(c->trav_cnt) + 1;
             da.ctr = reinterpret_cast<unsigned long long*>(ptr<char>(c->trav_cnt) + 32);
-            da.sort_keys = K > 1 ? ptr<uint64_t>(c->los_keys) : nullptr;
+            da.sort_keys = K > 1 ? ptr<uint32_t>(c->los_keys) : nullptr;
             da.sort_scr = K > 1 ? c->los_scr.p : nullptr;
             for (int k = 0; k < 3; ++k) {
                 const float ext = S.bounds_hi[k] - S.bounds_lo[k];
@@ -1214,16 +1213,11 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
         // ---- specular accumulation (Eq. 2-4)
         if (p.components & ST_COMP_SPECULAR && NB > 0) {
             NvtxRange range("st_simulate: specular accumulation");
-            CKC(c, flags_visible_records(ptr<int32_t>(c->rec_tri), ptr<uint8_t>(c->rec_los), NB, ptr<uint32_t>(c->sflags), s),
-                "flags");
-            CKC(c, exclusive_scan_u32(ptr<uint32_t>(c->sflags), ptr<uint32_t>(c->sscan), NB, cnt + 2, c->scratch.p, s),
-                "scan");
-            CKC(c, compact_indices(ptr<uint32_t>(c->sflags), ptr<uint32_t>(c->sscan), NB, ptr<uint32_t>(c->sidx), s),
-                "compact");
+            CKC(c, compact_flags(ptr<uint8_t>(c->rec_los), NB, ptr<uint32_t>(c->sidx), cnt + 2, c->scratch.p, s), "compact");
             ga.count = cnt + 2;
             ga.out = &c->paths;
             if (ga.has_etab && NB > 1) {  // paths in emitter-table row order: a tile's paths share table rows
-                CKC(c, theta_order(ga, NB, ptr<uint32_t>(c->sidx), ptr<uint64_t>(c->th_keys), c->th_scr.p, s), "order");
+                CKC(c, theta_order(ga, NB, ptr<uint32_t>(c->sidx), ptr<uint32_t>(c->th_keys), c->th_scr.p, s), "order");
             }
             CKC(c, gather_specular(ga, s), "gather");
             AccumArgs x = aa;
@@ -1251,11 +1245,7 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
         // ---- diffraction accumulation (Eq. 7-8)
         if (K > 0) {
             NvtxRange range("st_simulate: diffraction accumulation");
-            CKC(c, flags_from_u8(ptr<uint8_t>(c->keep), K, ptr<uint32_t>(c->dflags), s2), "flags");
-            CKC(c, exclusive_scan_u32(ptr<uint32_t>(c->dflags), ptr<uint32_t>(c->dscan), K, cnt + 3, c->dscratch.p, s2),
-                "scan");
-            CKC(c, compact_indices(ptr<uint32_t>(c->dflags), ptr<uint32_t>(c->dscan), K, ptr<uint32_t>(c->didx), s2),
-                "compact");
+            CKC(c, compact_flags(ptr<uint8_t>(c->keep), K, ptr<uint32_t>(c->didx), cnt + 3, c->dscratch.p, s2), "compact");
             GatherArgs gd = ga;
             gd.idx = ptr<uint32_t>(c->didx);
             gd.count = cnt + 3;
@@ -1591,12 +1581,16 @@ static st_status backward_impl(st_ctx* c, st_scene* sc, const void* grad_spectra
     CKC(c, grow(c->adj_v, (size_t)chunks * g.n_mb * 4 * F * 4), "alloc");
     CKC(c, grow(c->adj_mic, (size_t)mic_slices * M * 3 * 4), "alloc");
     CKC(c, grow(c->adj_emit, (size_t)emit_slices * 3 * 4), "alloc");
-    CKC(c, cudaMemsetAsync(c->adj_mic.p, 0, (size_t)mic_slices * M * 3 * 4, s), "memset");
-    CKC(c, cudaMemsetAsync(c->adj_emit.p, 0, (size_t)emit_slices * 3 * 4, s), "memset");
     float* micp = ptr<float>(c->adj_mic);
     float* emitp = ptr<float>(c->adj_emit);
-    if (grad_k) CKC(c, cudaMemsetAsync(grad_k, 0, (size_t)S.n_mat * S.n_bands * 4, s), "memset");
-    if (grad_beta) CKC(c, cudaMemsetAsync(grad_beta, 0, (size_t)S.n_mat * S.n_bands * 4, s), "memset");
+    {
+        const size_t bands = (size_t)S.n_mat * S.n_bands * 4;
+        const Fill f[] = {{c->adj_mic.p, (size_t)mic_slices * M * 3 * 4, 0u},
+                          {c->adj_emit.p, (size_t)emit_slices * 3 * 4, 0u},
+                          {grad_k, grad_k ? bands : 0, 0u},
+                          {grad_beta, grad_beta ? bands : 0, 0u}};
+        CKC(c, fill_many(f, 4, s), "initial values");
+    }
 
     auto set_paths = [&](AccumArgs& x, PathList& PL) {
         x.px = ptr<float>(PL.px);
@@ -1693,13 +1687,7 @@ static st_status backward_impl(st_ctx* c, st_scene* sc, const void* grad_spectra
         const int64_t NB = c->last_N * c->last_B;
         if (!c->paths_chain_order || grad_emitter) {
             // the compaction of the last simulate, repeated: the visible records in the order of its path list
-            CKC(c, flags_visible_records(ptr<int32_t>(c->rec_tri), ptr<uint8_t>(c->rec_los), NB,
-                                         ptr<uint32_t>(c->sflags), s),
-                "flags");
-            CKC(c, exclusive_scan_u32(ptr<uint32_t>(c->sflags), ptr<uint32_t>(c->sscan), NB, cnt + 2, c->scratch.p, s),
-                "scan");
-            CKC(c, compact_indices(ptr<uint32_t>(c->sflags), ptr<uint32_t>(c->sscan), NB, ptr<uint32_t>(c->sidx), s),
-                "compact");
+            CKC(c, compact_flags(ptr<uint8_t>(c->rec_los), NB, ptr<uint32_t>(c->sidx), cnt + 2, c->scratch.p, s), "compact");
         }
         if (c->n_theta == 0 && NB > 1) {
             // chain order (omni emitter; with an emitter table the list keeps its table-row order): paths with
@@ -1729,7 +1717,7 @@ static st_status backward_impl(st_ctx* c, st_scene* sc, const void* grad_spectra
                 CKC(c, grow(c->ck_keys, (size_t)NB * 8), "alloc");
                 CKC(c, grow(c->ck_scr, sort_scratch_bytes(NB)), "alloc");
                 CKC(c, chain_order(ga, NB, p.reflection_mode == 1 ? 1 : 0, ptr<uint32_t>(c->sidx),
-                                   ptr<uint64_t>(c->ck_keys), c->ck_scr.p, s),
+                                   ptr<uint32_t>(c->ck_keys), c->ck_scr.p, s),
                     "chain order");
             }
             if (!c->paths_chain_order) CKC(c, gather_specular(ga, s), "gather");
@@ -2404,7 +2392,7 @@ static st_status simulate_batch_impl(st_ctx* c, int32_t n_jobs, const st_job* jo
         CKC(c, build_accum_tables(B.tables[j], S, J.n_bins, J.f_lo, J.f_hi, p.c, p.alpha0_db_m, p.alpha1_db_m_khz, s),
             "batch tables");
         if (J.n_rays > 0)
-            CKC(c, direction_order(J.dirs, J.n_rays, ptr<uint64_t>(B.ord_keys), ptr<uint32_t>(B.perm) + ray_o[j],
+            CKC(c, direction_order(J.dirs, J.n_rays, ptr<uint32_t>(B.ord_keys), ptr<uint32_t>(B.perm) + ray_o[j],
                                    B.ord_scr.p, s),
                 "batch order");
         JobDev& d = B.jobs[j];

@@ -117,10 +117,26 @@ inline unsigned grid_for(int64_t n, int block, int64_t cap = 152 * 32) {
 }
 
 // ------------------------------------------------------------------ primitives (st_sort.cu)
-// Stable LSD radix sort of (u64 key, u32 value) pairs over the low `bits` bits of the key.
-// Scratch must hold sort_scratch_bytes(n) bytes.
+// Sets up to kFillMax stretches of device memory (4-byte aligned, whole words) to a repeated word in one launch.
+constexpr int kFillMax = 12;
+struct Fill {
+    void* p;
+    size_t bytes;
+    uint32_t word;
+};
+cudaError_t fill_many(const Fill* f, int n, cudaStream_t s);
+// Stable LSD radix sort of (key, u32 value) pairs over the key's low `bits` bits, or its bits lo_bit .. hi_bit - 1;
+// d_n: the number of pairs on the device (at most n; null: n).  Scratch must hold sort_scratch_bytes(n) bytes.
 size_t sort_scratch_bytes(int64_t n);
-cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, void* scratch, cudaStream_t s);
+cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, void* scratch, cudaStream_t s,
+                           const uint32_t* d_n = nullptr);
+cudaError_t radix_sort_u32(uint32_t* keys, uint32_t* vals, int64_t n, int lo_bit, int hi_bit, void* scratch,
+                           cudaStream_t s, const uint32_t* d_n = nullptr);
+// Indices of the non-zero bytes of flags [n] (16-byte aligned) in order, their number in *total (device).  Scratch:
+// compact_scratch_bytes(n).
+size_t compact_scratch_bytes(int64_t n);
+cudaError_t compact_flags(const uint8_t* flags, int64_t n, uint32_t* idx, uint32_t* total, void* scratch,
+                          cudaStream_t s);
 // Exclusive scan of n u32 flags/counts into out (u32), total written to *total (device, may be null).
 size_t scan_scratch_bytes(int64_t n);
 cudaError_t exclusive_scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total, void* scratch,
@@ -219,8 +235,8 @@ struct TraceArgs {
     unsigned long long* queries;  // [0] closest-hit segments, [1] any-hit segments
 };
 cudaError_t trace_rays(TraceArgs& a, cudaStream_t s, int block);
-// perm = indices 0..n-1 sorted by an octahedral Morton key of dirs (keys: n u64 scratch)
-cudaError_t direction_order(const float* dirs, int64_t n, uint64_t* keys, uint32_t* perm, void* scratch,
+// perm = indices 0..n-1 sorted by an octahedral Morton key of dirs (keys: n u32 scratch)
+cudaError_t direction_order(const float* dirs, int64_t n, uint32_t* keys, uint32_t* perm, void* scratch,
                             cudaStream_t s);
 
 struct DiffArgs {
@@ -265,7 +281,7 @@ struct DiffArgs {
     uint32_t* flags;
     unsigned long long* queries;
     // optional: line-of-sight queue sorted by the Morton code of the candidate points (keys [K], scratch)
-    uint64_t* sort_keys; void* sort_scr;
+    uint32_t* sort_keys; void* sort_scr;
     float blo[3], bscale[3];
 };
 cudaError_t diffraction_sample(DiffArgs& a, cudaStream_t s);
@@ -412,14 +428,13 @@ struct GatherArgs {
     uint32_t* chk = nullptr;   // checked build: flags word
 };
 cudaError_t gather_specular(const GatherArgs& g, cudaStream_t s);
-// Stable sort of the compacted specular indices idx[0 .. cap) by emitter-table row (entries past *g.count
-// last); keys [cap] and scratch (sort_scratch_bytes(cap)) are the caller's.
-cudaError_t theta_order(const GatherArgs& g, int64_t cap, uint32_t* idx, uint64_t* keys, void* scratch,
+// Stable sort of the compacted specular indices idx[0 .. cap) by emitter-table row; keys [cap] and scratch (sort_scratch_bytes(cap)) are the caller's.
+cudaError_t theta_order(const GatherArgs& g, int64_t cap, uint32_t* idx, uint32_t* keys, void* scratch,
                         cudaStream_t s);
 // Stable sort of the compacted specular indices idx[0 .. cap) by the material counts of their reflection chains
-// (materials 0..3; last_only: by the last hit's material), entries past *g.count last: the adjoint forms its
+// (materials 0..3; last_only: by the last hit's material): the adjoint forms its
 // reflection sums once per run of equal counts.  keys [cap] and scratch (sort_scratch_bytes(cap)) are the caller's.
-cudaError_t chain_order(const GatherArgs& g, int64_t cap, int last_only, uint32_t* idx, uint64_t* keys, void* scratch,
+cudaError_t chain_order(const GatherArgs& g, int64_t cap, int last_only, uint32_t* idx, uint32_t* keys, void* scratch,
                         cudaStream_t s);
 cudaError_t gather_diffraction(const GatherArgs& g, cudaStream_t s);
 cudaError_t flags_visible_records(const int32_t* rec_tri, const uint8_t* rec_los, int64_t n, uint32_t* flags,

@@ -69,13 +69,14 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     return z;
 }
 
-__global__ void k_pos_keys(const float* V, int64_t nv, uint64_t* keys, uint32_t* vals) {
+// (32 bits of the hash: equal positions get equal keys, and k_weld_runs compares the positions of a run anyway)
+__global__ void k_pos_keys(const float* V, int64_t nv, uint32_t* keys, uint32_t* vals) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += stride) {
         uint64_t h = mix64(pos_bits(V[3 * i]));
         h = mix64(h ^ pos_bits(V[3 * i + 1]));
         h = mix64(h ^ ((uint64_t)pos_bits(V[3 * i + 2]) << 17));
-        keys[i] = h;
+        keys[i] = (uint32_t)(h >> 32);
         vals[i] = (uint32_t)i;
     }
 }
@@ -87,7 +88,7 @@ __device__ __forceinline__ bool same_pos(const float* V, uint32_t a, uint32_t b)
 }
 
 // One thread per run of equal hashes: canon[v] = smallest index with exactly the same position.
-__global__ void k_weld_runs(const float* V, int64_t nv, const uint64_t* keys, const uint32_t* vals, int32_t* canon) {
+__global__ void k_weld_runs(const float* V, int64_t nv, const uint32_t* keys, const uint32_t* vals, int32_t* canon) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nv; i += stride) {
         if (i > 0 && keys[i] == keys[i - 1]) continue;
@@ -277,10 +278,10 @@ __global__ void k_mesh_count(const int32_t* obj, int64_t nt, uint32_t* cnt) {
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += stride) atomicAdd(&cnt[obj[t]], 1u);
 }
 
-__global__ void k_mesh_keys(const int32_t* obj, int64_t nt, uint64_t* keys, uint32_t* vals) {
+__global__ void k_mesh_keys(const int32_t* obj, int64_t nt, uint32_t* keys, uint32_t* vals) {
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += stride) {
-        keys[t] = ((uint64_t)(uint32_t)obj[t] << 32) | (uint64_t)t;
+        keys[t] = (uint32_t)obj[t];
         vals[t] = (uint32_t)t;
     }
 }
@@ -477,7 +478,7 @@ __global__ void k_morton(const float* V, const int32_t* T, int64_t nt, const uin
             c = c * (1.0f / 3.0f);
             float u = ext[k] > 0.0f ? (c - lo[k]) / ext[k] : 0.5f;
             u = fminf(fmaxf(u, 0.0f), 1.0f);
-            uint32_t qi = (uint32_t)(u * 2097151.0f);
+            uint32_t qi = (uint32_t)(u * 65535.0f);
             q[k] = qi;
         }
         keys[t] = (spread21(q[0]) << 2) | (spread21(q[1]) << 1) | spread21(q[2]);
@@ -779,11 +780,11 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
         CK(grow(vals, (size_t)nmax * 4));
         CK(grow(sort_scr, sort_scratch_bytes(nmax) + scan_scratch_bytes(nmax + n_obj + 1)));
         note_launch();
-        k_pos_keys<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, ptr<uint64_t>(keys), ptr<uint32_t>(vals));
+        k_pos_keys<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, ptr<uint32_t>(keys), ptr<uint32_t>(vals));
         CK(cudaGetLastError());
-        CK(radix_sort_u64(ptr<uint64_t>(keys), ptr<uint32_t>(vals), nv, 64, sort_scr.p, s));
+        CK(radix_sort_u32(ptr<uint32_t>(keys), ptr<uint32_t>(vals), nv, 0, 32, sort_scr.p, s));
         note_launch();
-        k_weld_runs<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, ptr<uint64_t>(keys), ptr<uint32_t>(vals), ptr<int32_t>(canon));
+        k_weld_runs<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, ptr<uint32_t>(keys), ptr<uint32_t>(vals), ptr<int32_t>(canon));
         CK(cudaGetLastError());
 
         // ---- adjacency CSR over canonical vertices
@@ -833,13 +834,13 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
         CK(exclusive_scan_u32(ptr<uint32_t>(cnt), ptr<uint32_t>(moff), n_obj + 1, nullptr, sort_scr.p, s));
         CK(grow(S.mesh_tris, (size_t)nt * 4));
         {
-            // (mesh, triangle) keys sorted: triangles grouped by mesh, ascending inside a mesh
+            // triangles grouped by mesh, ascending inside a mesh (the sort is stable)
             int mesh_bits = 1;
             while ((1ll << mesh_bits) <= (int64_t)n_obj) ++mesh_bits;
             note_launch();
-            k_mesh_keys<<<grid_for(nt, kB), kB, 0, s>>>(obj, nt, ptr<uint64_t>(keys), ptr<uint32_t>(vals));
+            k_mesh_keys<<<grid_for(nt, kB), kB, 0, s>>>(obj, nt, ptr<uint32_t>(keys), ptr<uint32_t>(vals));
             CK(cudaGetLastError());
-            CK(radix_sort_u64(ptr<uint64_t>(keys), ptr<uint32_t>(vals), nt, 32 + mesh_bits, sort_scr.p, s));
+            CK(radix_sort_u32(ptr<uint32_t>(keys), ptr<uint32_t>(vals), nt, 0, mesh_bits, sort_scr.p, s));
             CK(cudaMemcpyAsync(S.mesh_tris.p, vals.p, (size_t)nt * 4, cudaMemcpyDeviceToDevice, s));
         }
         CK(grow(sumQ, (size_t)(n_obj + 1) * 8));
@@ -901,7 +902,7 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
         note_launch();
         k_morton<<<grid_for(nt, kB), kB, 0, s>>>(V, T, nt, ptr<uint32_t>(bnd), ptr<uint64_t>(keys), ptr<uint32_t>(vals));
         CK(cudaGetLastError());
-        CK(radix_sort_u64(ptr<uint64_t>(keys), ptr<uint32_t>(vals), nt, 63, sort_scr.p, s));
+        CK(radix_sort_u64(ptr<uint64_t>(keys), ptr<uint32_t>(vals), nt, 48, sort_scr.p, s));
         CK(grow(S.bvh_perm, (size_t)nt * 4));
         CK(cudaMemcpyAsync(S.bvh_perm.p, vals.p, (size_t)nt * 4, cudaMemcpyDeviceToDevice, s));
     }
@@ -1302,7 +1303,7 @@ static cudaError_t build_two_level(SceneDev& S, float pad_world, uint32_t* flags
             k_morton<<<grid_for(ntq, kB), kB, 0, s>>>(Vq, Tq, ntq, ptr<uint32_t>(bnd), ptr<uint64_t>(keys),
                                                       ptr<uint32_t>(vals));
             CK(cudaGetLastError());
-            CK(radix_sort_u64(ptr<uint64_t>(keys), ptr<uint32_t>(vals), ntq, 63, sort_scr.p, s));
+            CK(radix_sort_u64(ptr<uint64_t>(keys), ptr<uint32_t>(vals), ntq, 48, sort_scr.p, s));
             note_launch();
             k_reorder<<<grid_for(ntq, kB), kB, 0, s>>>(Vq, Tq, ntq, ptr<uint32_t>(vals),
                                                        ptr<float4>(S.blas_tri) + 3 * I.ptoff_h[q]);

@@ -118,3 +118,38 @@ def test_bounce_queues_match_oracle(torch_st, n_rays, bounces, los):
         assert np.array_equal(g[k][ref["rec"]["tri"] >= 0], ref["rec"][k][ref["rec"]["tri"] >= 0]), k
     if los:
         assert np.array_equal(ctx.receiver_masks(bounces), ref["rec"]["mask"])
+
+
+# radix sort tiles and odd / even pass counts through the orders that use them: direction order and line-of-sight queue
+# (sizes below, at and past a tile, past the small tiles' limit), mesh ids of one and of two digits, welded duplicates
+@pytest.mark.parametrize("n_rays,budget", [(1, 1), (1023, 1025), (1025, 4097), (70_001, 530_001)])
+def test_sorted_queues_match_oracle(torch_st, n_rays, budget):
+    _, st = torch_st
+    wl = synth.clutter(seed=31, target_tris=30_000, n_rays=n_rays, bounces=1, n_mics=3, n_bins=2)
+    ctx, sc, _, ref = simulate_and_compare(st, wl, budget=budget)
+    tri, p, keep = ctx.diffraction()
+    assert np.array_equal(tri, ref["cand_tri"]) and np.array_equal(p, ref["cand_p"])
+    assert np.array_equal(keep, ref["cand_keep"])
+
+
+@pytest.mark.parametrize("n_obj,copies", [(3, 1), (300, 3), (70_000, 1)])
+def test_mesh_order_and_welding_match_oracle(torch_st, n_obj, copies):
+    _, st = torch_st
+    import oracle
+    wl = synth.clutter(seed=32, target_tris=70_000 // copies, n_rays=64, bounces=1, n_mics=3, n_bins=2)
+    rng = np.random.default_rng(2)
+    # every triangle with vertices of its own (welding finds the shared positions), in a random order
+    v = wl.verts[wl.tris].reshape(-1, 3)
+    order = rng.permutation(len(wl.tris))
+    wl.tris = np.arange(len(v), dtype=np.int32).reshape(-1, 3)[order]
+    wl.verts = (v + np.float32(0)).astype(np.float32)
+    wl.tri_mat = wl.tri_mat[order]
+    wl.tri_obj = rng.integers(0, n_obj, len(wl.tris)).astype(np.int32)
+    ctx = st.Context(0)
+    sc = st.from_workload(ctx, wl, st.curv_params(sample_budget=50_000))
+    G, C, ns = sc.curvature()
+    oG = oracle.curvature(wl.verts, wl.tris)
+    oC = oracle.tri_metric(wl.verts, wl.tris, oG)
+    cd = oracle.diffraction_cdf(wl.verts, wl.tris, oC, wl.tri_obj, budget=50_000)
+    assert np.array_equal(G, oG) and np.array_equal(C, oC)
+    assert np.array_equal(ns, cd["n_samples"][:len(ns)])
