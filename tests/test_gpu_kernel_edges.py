@@ -153,3 +153,24 @@ def test_mesh_order_and_welding_match_oracle(torch_st, n_obj, copies):
     cd = oracle.diffraction_cdf(wl.verts, wl.tris, oC, wl.tri_obj, budget=50_000)
     assert np.array_equal(G, oG) and np.array_equal(C, oC)
     assert np.array_equal(ns, cd["n_samples"][:len(ns)])
+
+
+# hierarchy by clustering: one triangle more than a leaf, the tile of a round (496) and the last block (1024) and one more,
+# several tiles; triangles that all coincide (ties everywhere), big ones among small ones, and ones without an area
+@pytest.mark.parametrize("n,kind", [(5, ""), (495, ""), (496, ""), (497, "mixed"), (1024, ""), (1025, "mixed"), (1489, ""),
+                                    (5, "same"), (1025, "same"), (20_000, "mixed"), (30_000, "flat")])
+def test_clustered_hierarchy_matches_oracle(torch_st, n, kind):
+    _, st = torch_st
+    wl = synth.clutter(seed=41, target_tris=40_000, n_rays=4_000, bounces=2, n_mics=3, n_bins=4, diffraction=False)
+    rng = np.random.default_rng(n)
+    pick = np.zeros(n, np.int64) if kind == "same" else rng.choice(len(wl.tris), n, replace=False)
+    tri = wl.verts[wl.tris[pick]].copy()
+    if kind == "mixed":  # every 50th triangle 30 times as large
+        tri[::50] = tri[::50].mean(1, keepdims=True) + 30 * (tri[::50] - tri[::50].mean(1, keepdims=True))
+    elif kind == "flat":  # a third of them points, a third segments
+        tri[::3, 1:] = tri[::3, :1]
+        tri[1::3, 2] = tri[1::3, 1]
+    wl.verts = tri.reshape(-1, 3).astype(np.float32)
+    wl.tris = np.arange(3 * n, dtype=np.int32).reshape(-1, 3)
+    wl.tri_mat, wl.tri_obj = wl.tri_mat[pick], np.zeros(n, np.int32)
+    simulate_and_compare(st, wl, components=st.ST_COMP_SPECULAR | st.ST_COMP_DIRECT)
