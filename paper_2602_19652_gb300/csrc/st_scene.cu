@@ -281,6 +281,10 @@ __device__ __forceinline__ void philox10(uint32_t c0, uint32_t c1, uint32_t c2, 
     out[3] = c3;
 }
 
+__global__ void k_widen(const uint32_t* in, int64_t n, int64_t* out) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = in[i];
+}
 __global__ void k_mesh_count(const int32_t* obj, int64_t nt, uint32_t* cnt) {
     const int lane = threadIdx.x & 31;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -637,6 +641,8 @@ struct PlocArgs {
     int32_t* par_i;         // [n - 1], [n]
     int32_t* par_l;
     Box* box_tmp;           // [n - 1][2] the children's boxes by final node id
+    uint32_t* perm_in;      // [n] the order before
+    uint32_t* left;         // clusters left by the last block
 };
 
 __device__ __forceinline__ float union_area(const Box& a, const Box& b) {
@@ -795,17 +801,17 @@ __global__ void __launch_bounds__(kPlocThreads) k_ploc_merge(const PlocArgs a, i
     (it & 1 ? a.box[0] : a.box[1])[pos] = b;
 }
 
-// The last clusters (at most kPlocLast), a thread each, rounds in one block; *left: clusters left after at most
+// The last clusters (at most kPlocLast), a thread each, rounds in one block; *a.left: clusters left after at most
 // kPlocLastRounds (1).  About 28 dependent rounds: boxes, ids and sizes stay in shared memory, and one packed scan places
 // both the clusters kept (low half) and the nodes made.
-__global__ void __launch_bounds__(kPlocLast) k_ploc_last(const PlocArgs a, int it, uint32_t* left) {
+__global__ void __launch_bounds__(kPlocLast) k_ploc_last(const PlocArgs a, int it) {
     __shared__ Box box[kPlocLast];
     __shared__ int32_t ref[kPlocLast], sizes[kPlocLast], nn[kPlocLast];
     __shared__ uint32_t sums[kPlocLast / 32];
     int n = (int)a.count[it];
     int base = (int)a.nodes[it];
     if (n > kPlocLast) {
-        if (threadIdx.x == 0) *left = (uint32_t)n;
+        if (threadIdx.x == 0) *a.left = (uint32_t)n;
         return;
     }
     const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
@@ -857,12 +863,12 @@ __global__ void __launch_bounds__(kPlocLast) k_ploc_last(const PlocArgs a, int i
             size = sizes[i];
         }
     }
-    if (threadIdx.x == 0) *left = (uint32_t)n;
+    if (threadIdx.x == 0) *a.left = (uint32_t)n;
 }
 
 // the hierarchy in the radix tree's form: node ids from the root (0), leaves in depth-first order (a node's leaves are
 // a range), which permutes the triangles
-__global__ void k_ploc_layout(const PlocArgs a, const uint32_t* perm_in, uint32_t* perm, int32_t* pos_of) {
+__global__ void k_ploc_layout(const PlocArgs a, uint32_t* perm, int32_t* pos_of) {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.n; p += gridDim.x * blockDim.x) {
         int pos = 0, self = ~p;
         int node = a.par_l[p];
@@ -873,7 +879,7 @@ __global__ void k_ploc_layout(const PlocArgs a, const uint32_t* perm_in, uint32_
             node = a.par_i[node];
         }
         pos_of[p] = pos;
-        perm[pos] = perm_in[p];
+        perm[pos] = a.perm_in[p];
     }
 }
 
@@ -1041,49 +1047,48 @@ __global__ void k_reorder(const float* V, const int32_t* T, int64_t nt, const ui
 
 }  // namespace
 
-// Clustered hierarchy over n leaves in the order perm (permuted to the new leaf order): children, ranges and parents in the
-// radix tree's form.  *done = false, and nothing changed, when the clusters did not merge within the bounds.
-template <class LeafBox>
-static cudaError_t ploc_build(const LeafBox& leaf, int n, uint32_t* perm, int2* child, int2* range, int32_t* par_i,
-                              int32_t* par_l, Box* box_tmp, cudaStream_t s, bool* done) {
-    *done = false;
-    const int tiles = (n + kPlocTile - 1) / kPlocTile;
-    // one allocation: clusters of two rounds, partners, tile counts, round counters, raw nodes, parents, sizes
+// One allocation cut into pieces.  A build needs some 30 arrays of scratch; allocating and freeing each took about 35 us,
+// which was as long as the build's kernels.
+struct Pieces {
     size_t bytes = 0;
-    auto take = [&](size_t b) {
+    char* base = nullptr;  // null: only adds up
+    template <class T>
+    T* take(size_t count) {
         const size_t at = bytes;
-        bytes += (b + 255) & ~size_t(255);
-        return at;
-    };
-    const size_t o_ref0 = take((size_t)n * 4), o_ref1 = take((size_t)n * 4), o_box0 = take((size_t)n * sizeof(Box)),
-                 o_box1 = take((size_t)n * sizeof(Box)), o_mate = take((size_t)n * 4), o_tiles = take((size_t)tiles * 8),
-                 o_cnt = take((size_t)(2 * (kPlocRounds + 2) + 1) * 4), o_child = take((size_t)n * 8),
-                 o_pi = take((size_t)n * 4), o_pl = take((size_t)n * 4), o_size = take((size_t)n * 4),
-                 o_perm = take((size_t)n * 4);
-    DevBuf buf;
-    struct Free {
-        DevBuf& b;
-        ~Free() { release(b); }
-    } guard{buf};
-    CK(grow(buf, bytes));
-    char* p = ptr<char>(buf);
+        bytes += (count * sizeof(T) + 255) & ~size_t(255);
+        return base ? reinterpret_cast<T*>(base + at) : nullptr;
+    }
+};
+
+static PlocArgs ploc_pieces(Pieces& m, int n, Box* box_tmp) {
     PlocArgs a{};
     a.n = n;
-    a.ref[0] = reinterpret_cast<int32_t*>(p + o_ref0);
-    a.ref[1] = reinterpret_cast<int32_t*>(p + o_ref1);
-    a.box[0] = reinterpret_cast<Box*>(p + o_box0);
-    a.box[1] = reinterpret_cast<Box*>(p + o_box1);
-    a.mate = reinterpret_cast<int32_t*>(p + o_mate);
-    a.tiles = reinterpret_cast<uint2*>(p + o_tiles);
-    a.count = reinterpret_cast<uint32_t*>(p + o_cnt);
-    a.nodes = a.count + kPlocRounds + 2;
-    uint32_t* left = a.nodes + kPlocRounds + 2;
-    a.child = reinterpret_cast<int2*>(p + o_child);
-    a.par_i = reinterpret_cast<int32_t*>(p + o_pi);
-    a.par_l = reinterpret_cast<int32_t*>(p + o_pl);
-    a.size = reinterpret_cast<int32_t*>(p + o_size);
+    for (int k = 0; k < 2; ++k) {
+        a.ref[k] = m.take<int32_t>(n);
+        a.box[k] = m.take<Box>(n);
+    }
+    a.mate = m.take<int32_t>(n);
+    a.tiles = m.take<uint2>((n + kPlocTile - 1) / kPlocTile);
+    a.count = m.take<uint32_t>(kPlocRounds + 2);
+    a.nodes = m.take<uint32_t>(kPlocRounds + 2);
+    a.left = m.take<uint32_t>(1);
+    a.child = m.take<int2>(n);
+    a.size = m.take<int32_t>(n);
+    a.par_i = m.take<int32_t>(n);
+    a.par_l = m.take<int32_t>(n);
+    a.perm_in = m.take<uint32_t>(n);
     a.box_tmp = box_tmp;
-    uint32_t* perm_in = reinterpret_cast<uint32_t*>(p + o_perm);
+    return a;
+}
+
+// Clustered hierarchy over n leaves in the order perm (permuted to the new leaf order): children, ranges and parents in the
+// radix tree's form, and the boxes.  *done = false, and none of these changed but the boxes, when the clusters did not
+// merge within the bounds.
+template <class LeafBox>
+static cudaError_t ploc_build(const LeafBox& leaf, const PlocArgs& a, uint32_t* perm, int2* child, int2* range,
+                              int32_t* par_i, int32_t* par_l, cudaStream_t s, bool* done) {
+    *done = false;
+    const int n = a.n, tiles = (n + kPlocTile - 1) / kPlocTile;
     note_launch();
     k_ploc_init<<<grid_for(n, kB), kB, 0, s>>>(leaf, a);
     CK(cudaGetLastError());
@@ -1103,16 +1108,16 @@ static cudaError_t ploc_build(const LeafBox& leaf, int n, uint32_t* perm, int2* 
             CK(cudaGetLastError());
         }
         note_launch();
-        k_ploc_last<<<1, kPlocLast, 0, s>>>(a, it, left);
+        k_ploc_last<<<1, kPlocLast, 0, s>>>(a, it);
         CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(&h_left, left, 4, cudaMemcpyDeviceToHost, s));
+        CK(cudaMemcpyAsync(&h_left, a.left, 4, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         if (h_left <= (uint32_t)kPlocLast || it >= kPlocRounds) break;
     }
     if (h_left != 1) return cudaSuccess;
-    CK(cudaMemcpyAsync(perm_in, perm, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemcpyAsync(a.perm_in, perm, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
     note_launch();
-    k_ploc_layout<<<grid_for(n, kB), kB, 0, s>>>(a, perm_in, perm, a.mate);
+    k_ploc_layout<<<grid_for(n, kB), kB, 0, s>>>(a, perm, a.mate);
     CK(cudaGetLastError());
     note_launch();
     k_ploc_emit<<<grid_for(n, kB), kB, 0, s>>>(a, a.mate, child, range, par_i, par_l);
@@ -1132,20 +1137,14 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
     const float* V = ptr<float>(S.verts);
     const int32_t* T = ptr<int32_t>(S.tris);
     const int32_t* obj = ptr<int32_t>(S.tri_obj);
-    // ---- scratch (freed at the end of the build)
-    DevBuf flags, canon, keys, vals, sort_scr, cnt, off, cursor, adj, Gc, cmax, sumQ, Q, S64, nsu, bnd, boxes, visits,
-        moff, wscan_scr, wtotal;
-    auto cleanup = [&]() {
-        for (DevBuf* b : {&flags, &canon, &keys, &vals, &sort_scr, &cnt, &off, &cursor, &adj, &Gc, &cmax, &sumQ, &Q,
-                          &S64, &nsu, &bnd, &boxes, &visits, &moff, &wscan_scr, &wtotal})
-            release(*b);
-    };
+    DevBuf flags, scratch;
     struct Guard {
-        decltype(cleanup)& f;
-        ~Guard() { f(); }
-    } guard{cleanup};
-
-    const int64_t nmax = std::max<int64_t>(std::max<int64_t>(nv, nt), 1);
+        DevBuf &a, &b;
+        ~Guard() {
+            release(a);
+            release(b);
+        }
+    } guard{flags, scratch};
     CK(grow(flags, 16));
     CK(cudaMemsetAsync(flags.p, 0, 16, s));
     note_launch();
@@ -1160,127 +1159,148 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
         *msg = (hflags & kFlagBadVertex) ? "non-finite vertex coordinate" : "triangle index, material or object out of range";
         return cudaSuccess;
     }
-    // n_obj from the host copy is known by the caller (S.n_obj)
-    const int32_t n_obj = S.n_obj;
+    // ---- scratch: one allocation (its sizes are known once the mesh is found valid), freed at the end of the build
+    const int32_t n_obj = S.n_obj;  // known from the host copy
+    const int64_t nmax = std::max<int64_t>(std::max<int64_t>(nv, nt), 1);
+    const bool curv = !keep_curvature, flat = !S.two_level && nt > kLeafMax;
+    struct Scratch {
+        uint32_t *bnd, *vals, *cnt, *off, *cursor, *cmax, *moff, *visits, *wtotal;
+        uint64_t *keys, *Q, *S64;
+        unsigned long long *sumQ, *nsu;
+        int32_t *canon, *adj;
+        float* Gc;
+        char *sort_scr, *wscan_scr;
+        Box* boxes;
+        PlocArgs ploc;
+    } w{};
+    auto lay = [&](Pieces m) {
+        w.bnd = m.take<uint32_t>(16);
+        w.keys = m.take<uint64_t>(nmax);
+        w.vals = m.take<uint32_t>(nmax);
+        w.sort_scr = m.take<char>(sort_scratch_bytes(nmax) + scan_scratch_bytes(nmax + n_obj + 1));
+        if (curv) {
+            w.canon = m.take<int32_t>(nv);
+            w.cnt = m.take<uint32_t>(std::max<int64_t>(nv, n_obj) + 1);
+            w.off = m.take<uint32_t>(nv + 1);
+            w.cursor = m.take<uint32_t>(nv + 1);
+            w.adj = m.take<int32_t>(std::max<int64_t>(3 * nt, 1));
+            w.Gc = m.take<float>(nv);
+            w.cmax = m.take<uint32_t>(n_obj + 1);
+            w.moff = m.take<uint32_t>(n_obj + 2);
+            w.sumQ = m.take<unsigned long long>(n_obj + 1);
+            w.Q = m.take<uint64_t>(nmax);
+            w.S64 = m.take<uint64_t>(nmax);
+            w.nsu = m.take<unsigned long long>(n_obj + 1);
+        }
+        if (flat) {
+            w.boxes = m.take<Box>(2 * (nt - 1));
+            w.visits = m.take<uint32_t>(nt - 1);
+            if (!refit) {
+                w.wscan_scr = m.take<char>(scan_scratch_bytes(nt - 1));
+                w.wtotal = m.take<uint32_t>(1);
+                w.ploc = ploc_pieces(m, (int)nt, w.boxes);
+            }
+        }
+        return m.bytes;
+    };
+    CK(grow(scratch, lay(Pieces{})));
+    lay(Pieces{0, ptr<char>(scratch)});
+    uint32_t* keys32 = reinterpret_cast<uint32_t*>(w.keys);  // (the 32-bit sorts' keys)
 
     CK(grow(S.nrm, (size_t)nt * 3 * sizeof(float)));
     note_launch();
     k_normals<<<grid_for(nt, kB), kB, 0, s>>>(V, T, nt, ptr<float>(S.nrm));
     CK(cudaGetLastError());
 
-    CK(grow(keys, (size_t)nmax * 8));
-    CK(grow(vals, (size_t)nmax * 4));
-    CK(grow(sort_scr, sort_scratch_bytes(nmax) + scan_scratch_bytes(nmax + n_obj + 1)));
     if (!keep_curvature) {
         // ---- weld
-        CK(grow(canon, (size_t)nv * 4));
-        CK(grow(keys, (size_t)nmax * 8));
-        CK(grow(vals, (size_t)nmax * 4));
-        CK(grow(sort_scr, sort_scratch_bytes(nmax) + scan_scratch_bytes(nmax + n_obj + 1)));
         note_launch();
-        k_pos_keys<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, ptr<uint32_t>(keys), ptr<uint32_t>(vals));
+        k_pos_keys<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, keys32, w.vals);
         CK(cudaGetLastError());
-        CK(radix_sort_u32(ptr<uint32_t>(keys), ptr<uint32_t>(vals), nv, 0, 32, sort_scr.p, s));
+        CK(radix_sort_u32(keys32, w.vals, nv, 0, 32, w.sort_scr, s));
         note_launch();
-        k_weld_runs<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, ptr<uint32_t>(keys), ptr<uint32_t>(vals), ptr<int32_t>(canon));
+        k_weld_runs<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, keys32, w.vals, w.canon);
         CK(cudaGetLastError());
 
         // ---- adjacency CSR over canonical vertices
-        CK(grow(cnt, (size_t)(nv + 1) * 4));
-        CK(grow(off, (size_t)(nv + 1) * 4));
-        CK(grow(cursor, (size_t)(nv + 1) * 4));
-        CK(grow(adj, (size_t)std::max<int64_t>(3 * nt, 1) * 4));
-        CK(cudaMemsetAsync(cnt.p, 0, (size_t)(nv + 1) * 4, s));
-        CK(cudaMemsetAsync(cursor.p, 0, (size_t)(nv + 1) * 4, s));
+        CK(cudaMemsetAsync(w.cnt, 0, (size_t)(nv + 1) * 4, s));
+        CK(cudaMemsetAsync(w.cursor, 0, (size_t)(nv + 1) * 4, s));
         note_launch();
-        k_adj_count<<<grid_for(nt, kB), kB, 0, s>>>(ptr<int32_t>(canon), T, nt, ptr<uint32_t>(cnt));
+        k_adj_count<<<grid_for(nt, kB), kB, 0, s>>>(w.canon, T, nt, w.cnt);
         CK(cudaGetLastError());
-        CK(exclusive_scan_u32(ptr<uint32_t>(cnt), ptr<uint32_t>(off), nv + 1, nullptr, sort_scr.p, s));
+        CK(exclusive_scan_u32(w.cnt, w.off, nv + 1, nullptr, w.sort_scr, s));
         note_launch();
-        k_adj_fill<<<grid_for(nt, kB), kB, 0, s>>>(ptr<int32_t>(canon), T, nt, ptr<uint32_t>(off), ptr<uint32_t>(cursor),
-                                                  ptr<int32_t>(adj));
+        k_adj_fill<<<grid_for(nt, kB), kB, 0, s>>>(w.canon, T, nt, w.off, w.cursor,
+                                                  w.adj);
         CK(cudaGetLastError());
         note_launch();
-        k_adj_sort<<<grid_for(nv, kB), kB, 0, s>>>(nv, ptr<uint32_t>(off), ptr<int32_t>(adj));
+        k_adj_sort<<<grid_for(nv, kB), kB, 0, s>>>(nv, w.off, w.adj);
         CK(cudaGetLastError());
 
         // ---- curvature and metric
-        CK(grow(Gc, (size_t)nv * 4));
         CK(grow(S.G, (size_t)nv * 4));
         CK(grow(S.C, (size_t)nt * 4));
         note_launch();
-        k_curvature<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, T, ptr<int32_t>(canon), ptr<uint32_t>(off), ptr<int32_t>(adj),
-                                                   ptr<float>(Gc));
+        k_curvature<<<grid_for(nv, kB), kB, 0, s>>>(V, nv, T, w.canon, w.off, w.adj,
+                                                   w.Gc);
         CK(cudaGetLastError());
         note_launch();
-        k_expand_G<<<grid_for(nv, kB), kB, 0, s>>>(ptr<int32_t>(canon), nv, ptr<float>(Gc), ptr<float>(S.G));
+        k_expand_G<<<grid_for(nv, kB), kB, 0, s>>>(w.canon, nv, w.Gc, ptr<float>(S.G));
         CK(cudaGetLastError());
-        CK(grow(cmax, (size_t)(n_obj + 1) * 4));
-        CK(cudaMemsetAsync(cmax.p, 0, (size_t)(n_obj + 1) * 4, s));
+        CK(cudaMemsetAsync(w.cmax, 0, (size_t)(n_obj + 1) * 4, s));
         note_launch();
-        k_metric<<<grid_for(nt, kB), kB, 0, s>>>(V, T, nt, ptr<int32_t>(canon), ptr<float>(S.G), cp.eta, cp.area_ref,
-                                                ptr<float>(S.C), ptr<uint32_t>(cmax), obj);
+        k_metric<<<grid_for(nt, kB), kB, 0, s>>>(V, T, nt, w.canon, ptr<float>(S.G), cp.eta, cp.area_ref,
+                                                ptr<float>(S.C), w.cmax, obj);
         CK(cudaGetLastError());
 
         // ---- per-mesh triangle lists (ascending), integer weights, CDFs
-        CK(grow(moff, (size_t)(n_obj + 2) * 4));
-        CK(cudaMemsetAsync(cnt.p, 0, (size_t)(n_obj + 1) * 4, s));
-        CK(cudaMemsetAsync(cursor.p, 0, (size_t)(n_obj + 1) * 4, s));
+        CK(cudaMemsetAsync(w.cnt, 0, (size_t)(n_obj + 1) * 4, s));
         note_launch();
-        k_mesh_count<<<grid_for(nt, kB), kB, 0, s>>>(obj, nt, ptr<uint32_t>(cnt));
+        k_mesh_count<<<grid_for(nt, kB), kB, 0, s>>>(obj, nt, w.cnt);
         CK(cudaGetLastError());
-        CK(exclusive_scan_u32(ptr<uint32_t>(cnt), ptr<uint32_t>(moff), n_obj + 1, nullptr, sort_scr.p, s));
+        CK(exclusive_scan_u32(w.cnt, w.moff, n_obj + 1, nullptr, w.sort_scr, s));
         CK(grow(S.mesh_tris, (size_t)nt * 4));
         {
             // triangles grouped by mesh, ascending inside a mesh (the sort is stable)
             int mesh_bits = 1;
             while ((1ll << mesh_bits) <= (int64_t)n_obj) ++mesh_bits;
             note_launch();
-            k_mesh_keys<<<grid_for(nt, kB), kB, 0, s>>>(obj, nt, ptr<uint32_t>(keys), ptr<uint32_t>(vals));
+            k_mesh_keys<<<grid_for(nt, kB), kB, 0, s>>>(obj, nt, keys32, w.vals);
             CK(cudaGetLastError());
-            CK(radix_sort_u32(ptr<uint32_t>(keys), ptr<uint32_t>(vals), nt, 0, mesh_bits, sort_scr.p, s));
-            CK(cudaMemcpyAsync(S.mesh_tris.p, vals.p, (size_t)nt * 4, cudaMemcpyDeviceToDevice, s));
+            CK(radix_sort_u32(keys32, w.vals, nt, 0, mesh_bits, w.sort_scr, s));
+            CK(cudaMemcpyAsync(S.mesh_tris.p, w.vals, (size_t)nt * 4, cudaMemcpyDeviceToDevice, s));
         }
-        CK(grow(sumQ, (size_t)(n_obj + 1) * 8));
-        CK(cudaMemsetAsync(sumQ.p, 0, (size_t)(n_obj + 1) * 8, s));
-        CK(grow(Q, (size_t)nmax * 8));
-        CK(grow(S64, (size_t)nmax * 8));
+        CK(cudaMemsetAsync(w.sumQ, 0, (size_t)(n_obj + 1) * 8, s));
         note_launch();
-        k_quantize<<<grid_for(nt, kB), kB, 0, s>>>(ptr<int32_t>(S.mesh_tris), nt, obj, ptr<float>(S.C), ptr<uint32_t>(cmax),
-                                                  ptr<uint64_t>(Q), ptr<unsigned long long>(sumQ));
+        k_quantize<<<grid_for(nt, kB), kB, 0, s>>>(ptr<int32_t>(S.mesh_tris), nt, obj, ptr<float>(S.C), w.cmax,
+                                                  w.Q, w.sumQ);
         CK(cudaGetLastError());
         note_launch();
-        k_dither<<<grid_for(nt, kB), kB, 0, s>>>(ptr<int32_t>(S.mesh_tris), nt, obj, ptr<uint32_t>(moff),
-                                                ptr<unsigned long long>(sumQ), cp.dither, cp.seed, ptr<uint64_t>(Q));
+        k_dither<<<grid_for(nt, kB), kB, 0, s>>>(ptr<int32_t>(S.mesh_tris), nt, obj, w.moff,
+                                                w.sumQ, cp.dither, cp.seed, w.Q);
         CK(cudaGetLastError());
-        CK(inclusive_scan_u64(ptr<uint64_t>(Q), ptr<uint64_t>(S64), nt, sort_scr.p, s));
+        CK(inclusive_scan_u64(w.Q, w.S64, nt, w.sort_scr, s));
         CK(grow(S.cdf, (size_t)nt * 8));
         note_launch();
-        k_cdf_fix<<<grid_for(nt, kB), kB, 0, s>>>(ptr<uint64_t>(S64), nt, ptr<int32_t>(S.mesh_tris), obj,
-                                                 ptr<uint32_t>(moff), ptr<uint64_t>(S.cdf));
+        k_cdf_fix<<<grid_for(nt, kB), kB, 0, s>>>(w.S64, nt, ptr<int32_t>(S.mesh_tris), obj,
+                                                 w.moff, ptr<uint64_t>(S.cdf));
         CK(cudaGetLastError());
         // mesh offsets as int64 for the sampling kernels
         CK(grow(S.mesh_off, (size_t)(n_obj + 1) * 8));
-        {
-            std::vector<uint32_t> h32(n_obj + 1);
-            CK(cudaMemcpyAsync(h32.data(), moff.p, (size_t)(n_obj + 1) * 4, cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-            std::vector<int64_t> h64(h32.begin(), h32.end());
-            CK(cudaMemcpyAsync(S.mesh_off.p, h64.data(), (size_t)(n_obj + 1) * 8, cudaMemcpyHostToDevice, s));
-            CK(cudaStreamSynchronize(s));
-        }
-        // sample counts
-        CK(grow(nsu, (size_t)(n_obj + 1) * 8));
-        CK(cudaMemsetAsync(nsu.p, 0, (size_t)(n_obj + 1) * 8, s));
         note_launch();
-        k_hc_vertices<<<grid_for(nv, kB), kB, 0, s>>>(nv, ptr<int32_t>(canon), ptr<uint32_t>(off), ptr<int32_t>(adj), obj,
-                                                     ptr<float>(S.C), ptr<uint32_t>(cmax), cp.hc_frac,
-                                                     cp.samples_per_vertex, ptr<unsigned long long>(nsu));
+        k_widen<<<grid_for(n_obj + 1, kB), kB, 0, s>>>(w.moff, n_obj + 1, ptr<int64_t>(S.mesh_off));
+        CK(cudaGetLastError());
+        // sample counts
+        CK(cudaMemsetAsync(w.nsu, 0, (size_t)(n_obj + 1) * 8, s));
+        note_launch();
+        k_hc_vertices<<<grid_for(nv, kB), kB, 0, s>>>(nv, w.canon, w.off, w.adj, obj,
+                                                     ptr<float>(S.C), w.cmax, cp.hc_frac,
+                                                     cp.samples_per_vertex, w.nsu);
         CK(cudaGetLastError());
         CK(grow(S.n_samples, (size_t)(n_obj + 1) * 8));
         CK(grow(S.sample_off, (size_t)(n_obj + 1) * 8));
         note_launch();
-        k_sample_counts<<<1, kScThreads, 0, s>>>(n_obj, ptr<uint32_t>(moff), ptr<uint64_t>(S.cdf), ptr<unsigned long long>(nsu),
+        k_sample_counts<<<1, kScThreads, 0, s>>>(n_obj, w.moff, ptr<uint64_t>(S.cdf), w.nsu,
                                         cp.budget, ptr<int64_t>(S.n_samples), ptr<int64_t>(S.sample_off));
         CK(cudaGetLastError());
         CK(cudaMemcpyAsync(&S.total_samples, ptr<int64_t>(S.sample_off) + n_obj, 8, cudaMemcpyDeviceToHost, s));
@@ -1288,24 +1308,23 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
     }  // !keep_curvature
 
     // ---- LBVH
-    CK(grow(bnd, 64));
     {
         uint32_t init[6] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
-        CK(cudaMemcpyAsync(bnd.p, init, sizeof(init), cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(w.bnd, init, sizeof(init), cudaMemcpyHostToDevice, s));
     }
     note_launch();
-    k_bounds<<<grid_for(nv, kB, 152 * 4), kB, 0, s>>>(V, nv, ptr<uint32_t>(bnd));
+    k_bounds<<<grid_for(nv, kB, 152 * 4), kB, 0, s>>>(V, nv, w.bnd);
     CK(cudaGetLastError());
     if (!refit && !S.two_level) {
         note_launch();
-        k_morton<<<grid_for(nt, kB), kB, 0, s>>>(V, T, nt, ptr<uint32_t>(bnd), ptr<uint64_t>(keys), ptr<uint32_t>(vals));
+        k_morton<<<grid_for(nt, kB), kB, 0, s>>>(V, T, nt, w.bnd, w.keys, w.vals);
         CK(cudaGetLastError());
-        CK(radix_sort_u64(ptr<uint64_t>(keys), ptr<uint32_t>(vals), nt, 48, sort_scr.p, s));
+        CK(radix_sort_u64(w.keys, w.vals, nt, 48, w.sort_scr, s));
         CK(grow(S.bvh_perm, (size_t)nt * 4));
-        CK(cudaMemcpyAsync(S.bvh_perm.p, vals.p, (size_t)nt * 4, cudaMemcpyDeviceToDevice, s));
+        CK(cudaMemcpyAsync(S.bvh_perm.p, w.vals, (size_t)nt * 4, cudaMemcpyDeviceToDevice, s));
     }
     uint32_t hb[6];
-    CK(cudaMemcpyAsync(hb, bnd.p, sizeof(hb), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(hb, w.bnd, sizeof(hb), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     {
         double diag2 = 0;
@@ -1348,47 +1367,41 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
                     CK(grow(S.bvh_par_l, (size_t)n * 4));
                     child_p = ptr<int2>(S.bvh_child);
                     range_p = ptr<int2>(S.bvh_range);
-                    CK(grow(boxes, (size_t)(n - 1) * 2 * sizeof(Box)));
-                    CK(ploc_build(TriLeafBox{V, T, ptr<uint32_t>(S.bvh_perm), pad}, n, ptr<uint32_t>(S.bvh_perm), child_p,
-                                  range_p, ptr<int32_t>(S.bvh_par_i), ptr<int32_t>(S.bvh_par_l), ptr<Box>(boxes), s,
-                                  &clustered));
+                    CK(ploc_build(TriLeafBox{V, T, ptr<uint32_t>(S.bvh_perm), pad}, w.ploc, ptr<uint32_t>(S.bvh_perm),
+                                  child_p, range_p, ptr<int32_t>(S.bvh_par_i), ptr<int32_t>(S.bvh_par_l), s, &clustered));
                     if (!clustered) {
                         note_launch();
-                        k_karras<<<grid_for(n - 1, kB), kB, 0, s>>>(ptr<uint64_t>(keys), n, child_p, range_p,
+                        k_karras<<<grid_for(n - 1, kB), kB, 0, s>>>(w.keys, n, child_p, range_p,
                                                                     ptr<int32_t>(S.bvh_par_i), ptr<int32_t>(S.bvh_par_l));
                         CK(cudaGetLastError());
                     }
                 }
                 if (!clustered) {
-                    CK(grow(boxes, (size_t)(n - 1) * 2 * sizeof(Box)));
-                    CK(grow(visits, (size_t)(n - 1) * 4));
-                    CK(cudaMemsetAsync(visits.p, 0, (size_t)(n - 1) * 4, s));
+                    CK(cudaMemsetAsync(w.visits, 0, (size_t)(n - 1) * 4, s));
                     note_launch();
                     k_boxes<<<grid_for(n, kB), kB, 0, s>>>(TriLeafBox{V, T, ptr<uint32_t>(S.bvh_perm), pad}, n, child_p,
                                                            ptr<int32_t>(S.bvh_par_i), ptr<int32_t>(S.bvh_par_l),
-                                                           ptr<Box>(boxes), ptr<uint32_t>(visits), ptr<uint32_t>(flags));
+                                                           w.boxes, w.visits, ptr<uint32_t>(flags));
                     CK(cudaGetLastError());
                 }
                 if (!refit) {
                     // 4-wide BVH: flag the binary nodes that become wide nodes, number them
                     CK(grow(S.bvh_wflag, (size_t)(n - 1) * 4));
                     CK(grow(S.bvh_widx, (size_t)(n - 1) * 4));
-                    CK(grow(wscan_scr, scan_scratch_bytes(n - 1)));
-                    CK(grow(wtotal, 4));
                     note_launch();
                     k_wide_flags<<<grid_for(n - 1, kB), kB, 0, s>>>(n, range_p, ptr<int32_t>(S.bvh_par_i),
                                                                     ptr<uint32_t>(S.bvh_wflag), ptr<uint32_t>(flags));
                     CK(cudaGetLastError());
                     CK(exclusive_scan_u32(ptr<uint32_t>(S.bvh_wflag), ptr<uint32_t>(S.bvh_widx), n - 1,
-                                          ptr<uint32_t>(wtotal), wscan_scr.p, s));
+                                          w.wtotal, w.wscan_scr, s));
                     uint32_t n4 = 0;
-                    CK(cudaMemcpyAsync(&n4, wtotal.p, 4, cudaMemcpyDeviceToHost, s));
+                    CK(cudaMemcpyAsync(&n4, w.wtotal, 4, cudaMemcpyDeviceToHost, s));
                     CK(cudaStreamSynchronize(s));
                     CK(grow(S.nodes, (size_t)std::max<uint32_t>(n4, 1) * 8 * sizeof(float4)));
                     S.n_nodes = n4;
                 }
                 note_launch();
-                k_pack_wide<<<grid_for(n - 1, kB), kB, 0, s>>>(n, child_p, range_p, ptr<Box>(boxes),
+                k_pack_wide<<<grid_for(n - 1, kB), kB, 0, s>>>(n, child_p, range_p, w.boxes,
                                                                ptr<uint32_t>(S.bvh_wflag), ptr<uint32_t>(S.bvh_widx),
                                                                ptr<float4>(S.nodes), 0, 0);
                 CK(cudaGetLastError());
