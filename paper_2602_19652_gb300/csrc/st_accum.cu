@@ -92,6 +92,7 @@ __global__ void k_tables(int32_t F, int32_t n_mat, int32_t n_bands, const float*
 template <int KT, int KIND, int DIR, int SPLIT = 0>
 __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int bx, int by, float4* smem4) {
     static_assert((KT & (KT - 1)) == 0 && KT >= 2, "KT must be a power of two");
+    constexpr int RL = row_pairs(KT), RX = row_floats(KT);
     const int PT = g.PT, NS = g.NS, TP = g.TP, KB = g.KB, MP = g.MP;
     const Buf B0 = buf_at<KT>(smem4, g, 0), B1 = buf_at<KT>(smem4, g, 1);
     float* pdb = reinterpret_cast<float*>(reinterpret_cast<char*>(smem4) + 2 * g.buf_bytes);  // [2][PT][12]
@@ -115,13 +116,12 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
 #pragma unroll
     for (int kk = 0; kk < KT; ++kk) Sr[kk] = Si[kk] = 0ull;
 
-    const float invNS = 1.0f / (float)NS, invKB = 1.0f / (float)KB;
-    // per-bin band interpolation of the CTA's bins in table order (directional receivers)
-    float2* bwt = reinterpret_cast<float2*>(mt + (g.mat_cached ? 2 * a.n_mat_tab * KB : 0));
+    const float invKB = 1.0f / (float)KB;
+    // per-bin band interpolation of the CTA's bins, in the tables' rows (directional receivers)
+    float2* bwt = reinterpret_cast<float2*>(mt + g.mat_floats);
     if (DIR && t0 < t1) {
         for (int i = tid; i < KB; i += nthr) {
-            const int kk = __float2int_rz(((float)i + 0.5f) * invNS), s_ = i - kk * NS;
-            bwt[i] = a.bw[min(kb + s_ * KT + kk, a.F - 1)];
+            bwt[(i / KT) * RL + i % KT] = a.bw[min(kb + i, a.F - 1)];
         }
     }
     if (t0 < t1) {
@@ -129,14 +129,14 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
             const int nm = a.n_mat_tab;
             for (int e = tid; e < nm * KB; e += nthr) {
                 const int mat = e / KB, i = e - mat * KB;
-                const int kk = __float2int_rz(((float)i + 0.5f) * invNS), s_ = i - kk * NS;
-                const int k = min(kb + s_ * KT + kk, a.F - 1);
+                const int k = min(kb + i, a.F - 1);
                 if (KIND == 0) {
                     mt[e] = a.lk[(int64_t)mat * a.F + k];
-                    mt[nm * KB + e] = a.g2[(int64_t)mat * a.F + k];
+                    // (finite: a path that is not there has -gamma^2 = 0)
+                    mt[nm * KB + mat * g.RX + (i / KT) * RX + i % KT] = fminf(a.g2[(int64_t)mat * a.F + k], 3.0e38f);
                 } else if (g.mat_direct) {  // the factor itself, as a pair for the two microphones of a thread
-                    const float x = (kb + s_ * KT + kk < a.F) ? ex2(a.lid[(int64_t)mat * a.F + k]) : 0.0f;
-                    reinterpret_cast<u64*>(mt)[e] = pk2(x, x);
+                    const float x = (kb + i < a.F) ? ex2(a.lid[(int64_t)mat * a.F + k]) : 0.0f;
+                    reinterpret_cast<u64*>(mt)[mat * g.RB + (i / KT) * RL + i % KT] = pk2(x, x);
                 } else {
                     mt[e] = a.lid[(int64_t)mat * a.F + k];
                 }
@@ -145,7 +145,7 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
         load_paths<KIND>(a, PT, t0 * PT, count, pdb, pvb);
         if (t0 + 1 < t1) load_paths<KIND>(a, PT, (t0 + 1) * PT, count, pdb + PT * 12, pvb + PT);
         __syncthreads();
-        produce<KT, KIND, 0, SPLIT>(a, g, B0, pdb, pvb, mt, mic0, kb, invNS, invKB, nullptr, pb0 + t0 * PT);
+        produce<KT, KIND, 0, SPLIT>(a, g, B0, pdb, pvb, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, nullptr, pb0 + t0 * PT);
         __syncthreads();
     }
     // software pipeline: consume tile t from buffer b while producing tile t+1 into buffer b^1
@@ -158,37 +158,53 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
         if (tile + 2 < t1) load_paths_cp<KIND>(a, PT, (tile + 2) * PT, count, pdb + b * PT * 12, pvb + b * PT);
         if (tile + 1 < t1) {
             const int nb = b ^ 1;  // path data of tile+1 sits in pd buffer nb
-            produce<KT, KIND, 0, SPLIT>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, mic0, kb, invNS, invKB, nullptr,
+            produce<KT, KIND, 0, SPLIT>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, nullptr,
                               pb0 + (tile + 1) * PT);
         }
-        for (int p = 0; p < (cons ? PT : 0); ++p) {
-            const ulonglong2 z0 = C.za[(p * NS + s) * TP + tp];
-            const u64* w = C.wst + p * 4 * TP + tp;  // component-major: conflict-free 64-bit loads
-            const u64 w1r = w[0], w1i = w[TP], w2r = w[2 * TP], w2i = w[3 * TP];
+        const ulonglong2* zp = C.za + s * TP + tp;
+        const ulonglong2* wp = C.wst + tp;
+        const u64* np = C.ngp + tp;
+        const float* xp = C.tab + s * RX;
+        const float* gb = reinterpret_cast<const float*>(smem4) + s * RX;
+        for (int p = 0; p < (cons ? PT : 0); ++p, zp += NS * TP, wp += 2 * TP, np += TP, xp += NS * RX) {
+            const ulonglong2 z0 = zp[0], w1 = wp[0], w2 = wp[TP];
+            const u64 w1r = w1.x, w1i = w1.y, w2r = w2.x, w2i = w2.y;
             const u64 nw2i = fmul2(w2i, pk2(-1.0f, -1.0f));
-            const u64 ng = C.ngp[p * TP + tp];
+            const u64 ng = np[0];
             u64 er = z0.x, ei = z0.y;  // even chain: bins 0, 2, 4, ...
             u64 orr = er, oi = ei;     // odd chain: bins 1, 3, 5, ...
             cmul2(orr, oi, w1r, w1i, fmul2(w1i, pk2(-1.0f, -1.0f)));
-            const float2* trow = reinterpret_cast<const float2*>(C.tab) + p * KB + s;
+            const float2* xrow = reinterpret_cast<const float2*>(xp);  // two bins each
+            const float2* grow = reinterpret_cast<const float2*>(gb + (KIND == 0 ? C.goff[p] : 0));
             const float2 ngv = up2(ng);  // -gamma^2 of the two microphones
             // diffraction with the material table read directly: the producer left the offset of the path's
             // material row in the (otherwise unused) lobe slot
-            const u64* mrow = reinterpret_cast<const u64*>(mt) + s;
-            if (KIND == 1 && g.mat_direct) mrow += (int)(uint32_t)ng;
+            const ulonglong2* mrow = reinterpret_cast<const ulonglong2*>(reinterpret_cast<const u64*>(mt) + s * RL);
+            if (KIND == 1 && g.mat_direct)
+                mrow = reinterpret_cast<const ulonglong2*>(reinterpret_cast<const u64*>(mrow) + (int)(uint32_t)ng);
+            u64 E2[2];  // factors of bins kk and kk + 1
 #pragma unroll
             for (int kk = 0; kk < KT; ++kk) {
-                u64 E;
-                if (KIND == 1 && g.mat_direct) {
-                    E = mrow[kk * NS];
-                } else if (KIND == 0) {
-                    const float2 t = trow[kk * NS];  // (log2 X, g)
-                    E = pk2(ex2(fmaf(ngv.x, t.y, t.x)), ex2(fmaf(ngv.y, t.y, t.x)));
-                } else {
-                    E = reinterpret_cast<const u64*>(trow)[kk * NS];  // (X, X)
+                if ((kk & 1) == 0) {
+                    if (KIND == 1 && g.mat_direct) {
+                        const ulonglong2 t = mrow[kk >> 1];
+                        E2[0] = t.x;
+                        E2[1] = t.y;
+                    } else {
+                        const float2 x = xrow[kk >> 1];
+                        if (KIND == 0) {
+                            const float2 t = grow[kk >> 1];
+                            E2[0] = pk2(ex2(fmaf(ngv.x, t.x, x.x)), ex2(fmaf(ngv.y, t.x, x.x)));
+                            E2[1] = pk2(ex2(fmaf(ngv.x, t.y, x.y)), ex2(fmaf(ngv.y, t.y, x.y)));
+                        } else {
+                            E2[0] = pk2(x.x, x.x);
+                            E2[1] = pk2(x.y, x.y);
+                        }
+                    }
                 }
+                u64 E = E2[kk & 1];
                 if (DIR) {  // receiver directivity, linear between bands
-                    const float2 bwv = bwt[kk * NS + s];
+                    const float2 bwv = bwt[s * RL + kk];
                     const int b0 = (int)bwv.x;
                     const float* d1 = C.dband + (p * MP + 2 * tp) * g.NB;
                     const float* d2 = d1 + g.NB;
@@ -237,9 +253,10 @@ __global__ void __launch_bounds__(256, DIR ? 1 : 2) k_accum(const AccumArgs a, c
 // Persistent accumulation of a batch: each CTA takes work items -- one CTA's worth of one (job, path kind)
 // accumulation: its microphone block, bin block and chunk -- from a device counter until none is left, and
 // runs them with the single-pose CTA body.  Items are claimed in task order; no item waits for another.  One
-// launch per path kind (the tasks of that kind).
+// launch per path kind (the tasks of that kind).  The table is declared unaliased: its fields are then read again where they
+// are used instead of spilled (228 -> 164 bytes a thread; 20 poses 16.4 -> 16.0 ms).
 template <int KIND>
-__global__ void __launch_bounds__(256, 2) k_accum_queue(const AccumTask* tasks, int32_t n_tasks, int64_t n_items,
+__global__ void __launch_bounds__(256, 2) k_accum_queue(const AccumTask* __restrict__ tasks, int32_t n_tasks, int64_t n_items,
                                                         unsigned long long* counter) {
     extern __shared__ float4 smem4[];
     __shared__ long long item_s;
@@ -504,7 +521,7 @@ __global__ void k_gather_diff(const GatherArgs g, float* px, float* py, float* p
 
 // accumulator tile shape: mic pairs per CTA and shared-memory budget (set by the tuner or ST_ACCUM_TILE="tp,kb")
 int g_tile_tp = 16;
-size_t g_tile_budget = 104 * 1024;  // two CTAs per SM (swept 88-110 KB: 104 fastest on the clutter workload)
+size_t g_tile_budget = 108 * 1024;  // two CTAs per SM (clutter, 1M rays: 96 KB 5.46 ms, 104 and 108 KB 5.20)
 int g_tile_kt = 16;
 bool g_tile_env_read = false;
 bool g_tile_env_set = false;  // ST_ACCUM_TILE gave the tile shape

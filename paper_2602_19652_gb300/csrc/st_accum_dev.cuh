@@ -155,6 +155,7 @@ __device__ __forceinline__ void cmul2(u64& zr, u64& zi, u64 wr, u64 wi, u64 nwi)
 
 struct Geom {
     int TP, NS, MP, KB, PT;  // mic pairs per CTA (threads along x), subtiles, mics per CTA, bins per CTA, paths/tile
+    int RB, RX;              // the CTA's bins as NS rows of pairs (row_pairs) and of floats (row_floats)
     int n_mb, n_bb;
     int NB;                  // receiver directivity bands held per (path, mic); 0 = omni receivers
     int ADJ;                 // adjoint layout: per (path, pair) position-gradient vectors after ngp
@@ -162,39 +163,61 @@ struct Geom {
     int mat_direct;          // diffraction without an emitter table: the term loop reads the per-(material, bin)
                              // factor from the cached material table, at the row offset the producer leaves in
                              // ngp; no per-(path, bin) table (tab has no space in the buffers)
-    size_t mat_bytes;        // their size
+    size_t mat_bytes;        // their size, with the per-bin band interpolation behind them
+    int mat_floats;          // of the material tables alone
     size_t buf_bytes;        // one pipeline buffer (tables + anchors of PT paths)
     size_t smem;
 };
 
+// A thread's KT bins are a row of its own in the per-bin tables: the term loop reads several bins per 128-bit load at
+// offsets known to the compiler, and the padding starts the rows of a warp's subtiles in different banks.
+// What bounds the accumulator is the number of instructions: of 20.8 per pair of microphones and bin 11 are the term's
+// own (6 packed FMA, 2 FMA and 2 ex2, loads).  With the bins transposed (entry kk * NS + s) every load had its address
+// computed, 16 in the term loop and 21.3 in all; with the lobe exponents read from the material table instead of copied
+// per path, two pipeline buffers of 8 paths fit two CTAs to an SM instead of 7, and the tables' half of the producer
+// shrinks: 19.7.  200k-ray clutter, 32 microphones x 512 bins: 1.145 -> 1.073 ms; 1M rays 5.60 -> 5.26; 24 x 257 with a
+// receiver test each 0.184 -> 0.164; the pose sweep's queue 16.1 -> 15.2 ms in all.  (Scalar instead of packed FMA costs
+// issue slots: 6.10; four bins per load in the term loop: 5.20, but the queue then spills and loses 5 %.)
+constexpr __host__ __device__ int row_floats(int KT) { return KT + 4; }
+constexpr __host__ __device__ int row_pairs(int KT) { return KT + 2; }
+
 // Shared memory: two pipeline buffers, each
-//   tab [PT][KB] float2      per (path, bin): (log2 X, g) specular, (X, X) diffraction,
-//                            bin kb + s*KT + kk stored at i = kk*NS + s
+//   tab [PT][NS][row_floats] float  per (path, bin): log2 X specular, X diffraction
+//   gtab                         the same for the lobe exponent g, when the material tables are not cached (specular)
 //   za  [PT][NS][TP] ulonglong2  phasor at bin kb + s*KT of the two mics of pair tp (re pair, im pair)
-//   wst [PT][4][TP] u64      one-bin step re, im and two-bin step re, im of the pair (component-major)
+//   wst [PT][2][TP] ulonglong2   one-bin step, two-bin step of the pair (re pair, im pair)
 //   ngp [PT][TP] u64         -gamma^2 of the pair (diffraction, mat_direct: the path's material row offset)
 //   adj [PT][TP][7] u64      (adjoint only) unit(m - P) xyz, lobe-angle vector xyz (specular) or
 //                            -unit(o - s) xyz (diffraction), 1 / r of the pair
 // then two path-data buffers pd [PT][12] + valid [PT], then the per-CTA material tables.
 struct Buf {
-    float4* tab;
+    float* tab;
+    float* gtab;
     ulonglong2* za;
-    u64* wst;
+    ulonglong2* wst;
     u64* ngp;
     u64* adj;
+    int* goff;     // [PT] the path's lobe exponents: offset in floats from the buffers' base (specular)
     float* dband;  // [PT][MP][NB] receiver directivity band values (directional receivers only)
 };
+
+// bytes of one path in tab and gtab
+__host__ __device__ __forceinline__ size_t tab_bytes(const Geom& g) {
+    return g.mat_direct ? (size_t)0 : (size_t)g.RX * (g.mat_cached ? 4 : 8);
+}
 
 template <int KT>
 __device__ __forceinline__ Buf buf_at(float4* base, const Geom& g, int b) {
     Buf B;
     char* p = reinterpret_cast<char*>(base) + (size_t)b * g.buf_bytes;
-    B.tab = reinterpret_cast<float4*>(p);
-    B.za = reinterpret_cast<ulonglong2*>(p + (g.mat_direct ? (size_t)0 : (size_t)g.PT * g.KB * 8));
-    B.wst = reinterpret_cast<u64*>(B.za + (size_t)g.PT * g.NS * g.TP);
-    B.ngp = B.wst + (size_t)g.PT * g.TP * 4;
+    B.tab = reinterpret_cast<float*>(p);
+    B.gtab = B.tab + (size_t)g.PT * g.RX;
+    B.za = reinterpret_cast<ulonglong2*>(p + tab_bytes(g) * g.PT);
+    B.wst = B.za + (size_t)g.PT * g.NS * g.TP;
+    B.ngp = reinterpret_cast<u64*>(B.wst + (size_t)g.PT * g.TP * 2);
     B.adj = B.ngp + (size_t)g.PT * g.TP;
-    B.dband = reinterpret_cast<float*>(B.adj + (g.ADJ ? (size_t)g.PT * g.TP * 7 : 0));
+    B.goff = reinterpret_cast<int*>(B.adj + (g.ADJ ? (size_t)g.PT * g.TP * 7 : 0));
+    B.dband = reinterpret_cast<float*>(B.goff + g.PT);
     return B;
 }
 
@@ -345,30 +368,31 @@ __device__ __forceinline__ void load_paths_async(const AccumArgs& a, int PT, int
     cp_async_commit();
 }
 
-// Scalar values of microphone mic0 + ml for path p of the tile: writes its half of the pair's step words, lobe
-// (or material row) word, receiver band values and, in the adjoint, gradient vectors; returns its phasor at the
-// CTA's first bin and the step over one subtile (KT bins), both zero for a microphone the path does not reach.
+// Values of microphone mic0 + ml for path p of the tile: its phasor at the CTA's first bin, the steps over one bin, two
+// bins and a subtile (KT bins), and its lobe word (-gamma^2, or the offset of the path's row in the material table); all
+// zero for a microphone the path does not reach.  Writes its receiver band values and, in the adjoint, gradient vectors.
+struct MicAnchor {
+    float2 z, w1, w2, wk;
+    float ng;
+};
 template <int KT, int KIND, int ADJ>
-__device__ __forceinline__ void anchor_mic(const AccumArgs& a, const Geom& g, const Buf& B, const float* pd,
-                                           const int* pv, int p, int ml, int mic0, int kb, const float* es,
-                                           int64_t pglob, float2* z_out, float2* wk_out) {
-    const int TP = g.TP, KB = g.KB, MP = g.MP;
+__device__ __forceinline__ MicAnchor anchor_mic(const AccumArgs& a, const Geom& g, const Buf& B, const float* pd,
+                                                const int* pv, int p, int ml, int mic0, int kb, const float* es,
+                                                int64_t pglob) {
+    const int TP = g.TP, MP = g.MP;
     const int pair = ml >> 1, half = ml & 1;
     const int m = mic0 + ml;
-    float* wf = reinterpret_cast<float*>(B.wst + p * 4 * TP + pair);  // component c at wf[2 TP c]
-    float* nf = reinterpret_cast<float*>(B.ngp + p * TP + pair);
+    MicAnchor o;
     // (per-microphone receiver test: a microphone that does not see the path gets a zero anchor)
     if (!pv[p] || m >= a.M || (a.mask && !((a.mask[pglob + p] >> m) & 1ull))) {
-        *z_out = make_float2(0.0f, 0.0f);
-        *wk_out = make_float2(0.0f, 0.0f);
-        for (int q = 0; q < 4; ++q) wf[2 * TP * q + half] = 0.0f;
-        nf[half] = 0.0f;
+        o.z = o.w1 = o.w2 = o.wk = make_float2(0.0f, 0.0f);
+        o.ng = 0.0f;
         for (int b = 0; b < g.NB; ++b) B.dband[(p * MP + ml) * g.NB + b] = 0.0f;
         if (ADJ) {
             float* af = reinterpret_cast<float*>(B.adj + (p * TP + pair) * 7);
             for (int q = 0; q < 7; ++q) af[2 * q + half] = 0.0f;
         }
-        return;
+        return o;
     }
     const float* d = pd + p * 12;
     const float mx = a.mics[3 * m], my = a.mics[3 * m + 1], mz = a.mics[3 * m + 2];
@@ -413,34 +437,29 @@ __device__ __forceinline__ void anchor_mic(const AccumArgs& a, const Geom& g, co
     float s0, c0;
     sincospif(2.0f * ff_frac(x0), &s0, &c0);
     const float A0 = ex2(L0);
-    const float2 z = make_float2(A0 * c0, A0 * s0);
+    o.z = make_float2(A0 * c0, A0 * s0);
     const ff xs = ff_mul(r, ff{a.dq_hi, a.dq_lo});
     float s1, c1;
     sincospif(2.0f * ff_frac(xs), &s1, &c1);
     const float a1 = ex2(rh * a.atm2_step);
-    const float2 W1 = make_float2(a1 * c1, a1 * s1);
-    const float2 W2 = cmul(W1, W1);  // two bins
-    wf[0 + half] = W1.x;
-    wf[2 * TP + half] = W1.y;
-    wf[4 * TP + half] = W2.x;
-    wf[6 * TP + half] = W2.y;
-    if (KIND == 1 && g.mat_direct) {  // offset of the path's row in the material table (term loop)
+    o.w1 = make_float2(a1 * c1, a1 * s1);
+    o.w2 = cmul(o.w1, o.w1);
+    if (KIND == 1 && g.mat_direct) {
         const int matp = min((int)((__float_as_uint(d[8]) >> 8) & 255u), a.n_mat_tab - 1);
-        reinterpret_cast<int*>(nf)[half] = matp * KB;
+        o.ng = __int_as_float(matp * g.RB);
     } else {
-        nf[half] = -gam2;
+        o.ng = -gam2;
     }
-    float2 WK = W2;  // KT bins by repeated squaring (KT is a power of two)
-    for (int q = 2; q < KT; q *= 2) WK = cmul(WK, WK);
-    *z_out = z;
-    *wk_out = WK;
+    o.wk = o.w2;  // KT bins by repeated squaring (KT is a power of two)
+    for (int q = 2; q < KT; q *= 2) o.wk = cmul(o.wk, o.wk);
+    return o;
 }
 
 // tables and anchors of one tile (reads pd / pv, writes buffer B); ADJ: also the position-gradient
 // vectors of the adjoint (es = emitter position, diffraction only); SPLIT: see below
 template <int KT, int KIND, int ADJ = 0, int SPLIT = 0>
 __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const Buf& B, const float* pd, const int* pv,
-                                        const float* mt, int mic0, int kb, float invNS, float invKB,
+                                        const float* mt, const float* base, int mic0, int kb, float invKB,
                                         const float* es = nullptr, int64_t pglob = 0) {
     const int PT = g.PT, NS = g.NS, TP = g.TP, KB = g.KB, MP = g.MP;
     const bool cached = g.mat_cached > 0;
@@ -453,18 +472,24 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
     const int n_anc = (KIND == 0 && !ADJ && SPLIT) ? ((PT * TP + 31) & ~31) : 0;
     const bool split = n_anc > 0 && nthr - n_anc >= 32;
     const int t_tab = split ? tid - n_anc : tid, n_tab = split ? nthr - n_anc : nthr;
-    // 1a: per (path, bin) factors, written in table order (not needed when the term loop reads the
-    // material table directly).  With NS % 4 == 0 and the material tables in
-    // shared memory, a thread builds four adjacent entries (same path and kk, subtiles s..s+3): one chain
-    // decode, 128-bit loads of the material rows and four conflict-free 128-bit stores.
+    // 1a: per (path, bin) factors (not needed when the term loop reads the material table directly).  With the material
+    // tables in shared memory a thread builds four bins of a row: one chain decode, 128-bit loads and stores.
+    constexpr int RX = row_floats(KT);
+    if (KIND == 0) {  // where the term loop finds the path's lobe exponents
+        for (int p = tid; p < PT; p += nthr) {
+            const int matj = pv[p] ? (int)((__float_as_uint(pd[p * 12 + 8]) >> 8) & 255u) : 0;
+            const float* row = cached ? mt + a.n_mat_tab * KB + matj * g.RX : B.gtab + p * g.RX;
+            B.goff[p] = (int)(row - base);
+        }
+    }
     if (KIND == 1 && g.mat_direct) {
-    } else if (cached && (NS & 3) == 0 && !a.etab) {
+    } else if (cached && !a.etab) {
         const int KB4 = KB >> 2;
-        const float invKB4 = 1.0f / (float)KB4;
+        const float invKB4 = 4.0f * invKB;
+        const bool last = kb + KB > a.F;  // bins beyond the grid contribute nothing
         for (int e = t_tab; e >= 0 && e < PT * KB4; e += n_tab) {
             const int p = __float2int_rz(((float)e + 0.5f) * invKB4), i = (e - p * KB4) * 4;
-            const int kk = __float2int_rz(((float)i + 0.5f) * invNS), s_ = i - kk * NS;
-            float4 lx4 = make_float4(kNegInf, kNegInf, kNegInf, kNegInf), g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 lx4 = make_float4(kNegInf, kNegInf, kNegInf, kNegInf);
             if (pv[p]) {
                 const float* d = pd + p * 12;
                 const uint32_t meta = __float_as_uint(d[8]);
@@ -474,50 +499,39 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                         lx4 = *reinterpret_cast<const float4*>(mt + matj * KB + i);
                     } else {
                         const int len = meta & 15;
-                        const uint32_t c0 = __float_as_uint(d[9]), c1 = __float_as_uint(d[10]);
+                        uint64_t chain = __float_as_uint(d[9]) | ((uint64_t)__float_as_uint(d[10]) << 32);
                         lx4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                        for (int q = 0; q < len; ++q) {
-                            const int mq = (q < 4 ? (c0 >> (8 * q)) : (c1 >> (8 * (q - 4)))) & 255;
-                            const float4 v = *reinterpret_cast<const float4*>(mt + mq * KB + i);
+                        for (int q = 0; q < len; ++q, chain >>= 8) {
+                            const float4 v = *reinterpret_cast<const float4*>(mt + ((int)chain & 255) * KB + i);
                             lx4.x += v.x;
                             lx4.y += v.y;
                             lx4.z += v.z;
                             lx4.w += v.w;
                         }
                     }
-                    g4 = *reinterpret_cast<const float4*>(mt + a.n_mat_tab * KB + matj * KB + i);
                 } else {
                     lx4 = *reinterpret_cast<const float4*>(mt + matj * KB + i);
                 }
-                // bins beyond the grid contribute nothing
-                const int k0 = kb + s_ * KT + kk;
-                if (k0 >= a.F) lx4.x = kNegInf;
-                if (k0 + KT >= a.F) lx4.y = kNegInf;
-                if (k0 + 2 * KT >= a.F) lx4.z = kNegInf;
-                if (k0 + 3 * KT >= a.F) lx4.w = kNegInf;
+                if (last) {
+                    const int k0 = kb + i;
+                    if (k0 >= a.F) lx4.x = kNegInf;
+                    if (k0 + 1 >= a.F) lx4.y = kNegInf;
+                    if (k0 + 2 >= a.F) lx4.z = kNegInf;
+                    if (k0 + 3 >= a.F) lx4.w = kNegInf;
+                }
             }
-            // four 8-byte entries (32-byte aligned: i is a multiple of 4)
-            float4* dst = reinterpret_cast<float4*>(reinterpret_cast<float2*>(B.tab) + p * KB + i);
-            if (KIND == 0) {
-                dst[0] = make_float4(lx4.x, g4.x, lx4.y, g4.y);
-                dst[1] = make_float4(lx4.z, g4.z, lx4.w, g4.w);
-            } else {
-                const float x0 = ex2(lx4.x), x1 = ex2(lx4.y), x2 = ex2(lx4.z), x3 = ex2(lx4.w);
-                dst[0] = make_float4(x0, x0, x1, x1);
-                dst[1] = make_float4(x2, x2, x3, x3);
-            }
+            if (KIND == 1) lx4 = make_float4(ex2(lx4.x), ex2(lx4.y), ex2(lx4.z), ex2(lx4.w));
+            *reinterpret_cast<float4*>(B.tab + (p * NS + i / KT) * RX + i % KT) = lx4;
         }
     } else {
         for (int e = t_tab; e >= 0 && e < PT * KB; e += n_tab) {
             const int p = __float2int_rz(((float)e + 0.5f) * invKB), i = e - p * KB;
-            const int kk = __float2int_rz(((float)i + 0.5f) * invNS), s_ = i - kk * NS;
-            const int k = kb + s_ * KT + kk;
+            const int k = kb + i;
             float lx = kNegInf, gg = 0.0f;
             if (pv[p] && k < a.F) {
                 const float* d = pd + p * 12;
                 const uint32_t meta = __float_as_uint(d[8]);
                 const int matj = (meta >> 8) & 255;
-                const int nm = a.n_mat_tab;
                 if (KIND == 0) {
                     if (a.reflection_mode == 1) {
                         lx = cached ? mt[matj * KB + i] : a.lk[(int64_t)matj * a.F + k];
@@ -531,7 +545,7 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                         }
                         lx = acc;
                     }
-                    gg = cached ? mt[nm * KB + matj * KB + i] : a.g2[(int64_t)matj * a.F + k];
+                    if (!cached) gg = a.g2[(int64_t)matj * a.F + k];
                 } else {
                     lx = cached ? mt[matj * KB + i] : a.lid[(int64_t)matj * a.F + k];
                 }
@@ -543,12 +557,9 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                     lx += de > 0.0f ? log2f(de) : kNegInf;
                 }
             }
-            if (KIND == 0) {
-                reinterpret_cast<float2*>(B.tab)[p * KB + i] = make_float2(lx, gg);
-            } else {
-                const float x = ex2(lx);
-                reinterpret_cast<float2*>(B.tab)[p * KB + i] = make_float2(x, x);
-            }
+            const int at = (p * NS + i / KT) * RX + i % KT;
+            B.tab[at] = KIND == 0 ? lx : ex2(lx);
+            if (KIND == 0 && !cached) B.gtab[at] = gg;
         }
     }
     // 1b: per (path, mic) anchors and the phasors at the subtile starts.  Specular paths of the forward go by
@@ -558,13 +569,17 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
     if (KIND == 0 && !ADJ) {
         for (int e = tid; e < PT * TP && (!split || tid < n_anc); e += split ? n_anc : nthr) {
             const int p = e / TP, pair = e - p * TP;
-            float2 zz[2], wk[2];
+            MicAnchor o[2];
 #pragma unroll
             for (int half = 0; half < 2; ++half)
-                anchor_mic<KT, KIND, ADJ>(a, g, B, pd, pv, p, 2 * pair + half, mic0, kb, es, pglob, &zz[half],
-                                                &wk[half]);
-            u64 zr = pk2(zz[0].x, zz[1].x), zi = pk2(zz[0].y, zz[1].y);
-            const u64 kr = pk2(wk[0].x, wk[1].x), ki = pk2(wk[0].y, wk[1].y), nki = pk2(-wk[0].y, -wk[1].y);
+                o[half] = anchor_mic<KT, KIND, ADJ>(a, g, B, pd, pv, p, 2 * pair + half, mic0, kb, es, pglob);
+            ulonglong2* w = B.wst + p * 2 * TP + pair;
+            w[0] = make_ulonglong2(pk2(o[0].w1.x, o[1].w1.x), pk2(o[0].w1.y, o[1].w1.y));
+            w[TP] = make_ulonglong2(pk2(o[0].w2.x, o[1].w2.x), pk2(o[0].w2.y, o[1].w2.y));
+            B.ngp[p * TP + pair] = pk2(o[0].ng, o[1].ng);
+            u64 zr = pk2(o[0].z.x, o[1].z.x), zi = pk2(o[0].z.y, o[1].z.y);
+            const u64 kr = pk2(o[0].wk.x, o[1].wk.x), ki = pk2(o[0].wk.y, o[1].wk.y),
+                      nki = pk2(-o[0].wk.y, -o[1].wk.y);
             ulonglong2* zo = B.za + p * NS * TP + pair;
             for (int s_ = 0; s_ < NS; ++s_) {
                 zo[s_ * TP] = make_ulonglong2(zr, zi);
@@ -575,13 +590,19 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
         for (int e = tid; e < PT * MP; e += nthr) {
             const int p = e / MP, ml = e - p * MP;
             const int pair = ml >> 1, half = ml & 1;
-            float2 z, wk;
-            anchor_mic<KT, KIND, ADJ>(a, g, B, pd, pv, p, ml, mic0, kb, es, pglob, &z, &wk);
+            const MicAnchor o = anchor_mic<KT, KIND, ADJ>(a, g, B, pd, pv, p, ml, mic0, kb, es, pglob);
+            float* wf = reinterpret_cast<float*>(B.wst + p * 2 * TP + pair) + half;
+            wf[0] = o.w1.x;
+            wf[2] = o.w1.y;
+            wf[4 * TP] = o.w2.x;
+            wf[4 * TP + 2] = o.w2.y;
+            reinterpret_cast<float*>(B.ngp + p * TP + pair)[half] = o.ng;
+            float2 z = o.z;
             float* zf = reinterpret_cast<float*>(B.za + p * NS * TP + pair);
             for (int s_ = 0; s_ < NS; ++s_) {
                 zf[s_ * TP * 4 + half] = z.x;
                 zf[s_ * TP * 4 + 2 + half] = z.y;
-                z = cmul(z, wk);
+                z = cmul(z, o.wk);
             }
         }
     }
@@ -602,9 +623,9 @@ inline Geom make_geom(int M, int F, int KT, int n_mat, int tp_max = 8, size_t bu
     g.TP = std::max(1, std::min(pairs, tp_max));
     g.NS = std::max(1, std::min(ns_need, 256 / g.TP));
     if (balance && g.NS > 2 && g.NS * KT <= 512) {
-        // bins spread evenly over their blocks, in subtiles a multiple of four: the tile's tables are then built with
-        // 128-bit accesses (104k paths: 32 microphones x 257 bins, whose second block held one bin, 0.75 -> 0.63 ms; 17
-        // x 257 0.50 -> 0.36; 24 x 512 1.06 -> 0.65).  Blocks of more than 512 bins stay, and with them the distance a phasor's rounding grows over.
+        // bins spread evenly over their blocks (104k paths: 32 microphones x 257 bins, whose second block held one bin,
+        // 0.75 -> 0.63 ms; 17 x 257 0.50 -> 0.36; 24 x 512 1.06 -> 0.65), in subtiles a multiple of four.  Blocks of more
+        // than 512 bins stay, and with them the distance a phasor's rounding grows over.
         const int blocks = (ns_need + g.NS - 1) / g.NS, ns = (ns_need + blocks - 1) / blocks, ns4 = (ns + 3) & ~3;
         g.NS = ns4 * g.TP <= 256 ? ns4 : ns;
     }
@@ -615,15 +636,19 @@ inline Geom make_geom(int M, int F, int KT, int n_mat, int tp_max = 8, size_t bu
     }
     g.MP = 2 * g.TP;
     g.KB = g.NS * KT;
+    g.RB = g.NS * row_pairs(KT);
+    g.RX = g.NS * row_floats(KT);
     g.n_mb = (M + g.MP - 1) / g.MP;
     g.n_bb = (F + g.KB - 1) / g.KB;
     const size_t mat_bytes = (size_t)2 * n_mat * g.KB * 4;  // two floats or one packed pair per (material, bin)
     g.mat_cached = mat_bytes <= 24 * 1024 ? 1 : 0;
     g.mat_direct = (mat_direct && g.mat_cached) ? 1 : 0;
-    const size_t per_path = (g.mat_direct ? (size_t)0 : (size_t)g.KB * 8) + (size_t)g.NS * g.TP * 16 +
-                            (size_t)g.TP * 40 + (size_t)g.MP * dir_nb * 4;
-    // fixed region: cached material tables, then (directional receivers) per-bin band interpolation
-    g.mat_bytes = (g.mat_cached ? mat_bytes : 0) + (dir_nb ? (size_t)g.KB * 8 : 0);
+    const size_t per_path =
+        tab_bytes(g) + (size_t)g.NS * g.TP * 16 + (size_t)g.TP * 40 + 4 + (size_t)g.MP * dir_nb * 4;
+    // fixed region: cached material tables (pairs; or log2 X in bin order and the lobe exponents in rows), then
+    // (directional receivers) per-bin band interpolation
+    g.mat_floats = g.mat_cached ? n_mat * (g.mat_direct ? 2 * g.RB : g.KB + g.RX) : 0;
+    g.mat_bytes = (size_t)g.mat_floats * 4 + (dir_nb ? (size_t)g.RB * 8 : 0);
     const size_t fixed = g.mat_bytes;
     const size_t avail = budget > fixed + 4096 ? budget - fixed : 4096;
     g.PT = (int)std::min<size_t>(8, std::max<size_t>(1, avail / (2 * per_path + 2 * 52)));

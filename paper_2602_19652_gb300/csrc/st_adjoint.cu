@@ -77,7 +77,7 @@ template <int KT, int KIND, int TPL, int EMIT>
 __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
     k_adjoint(const AccumArgs a, const AdjointArgs j, const Geom g) {
     static_assert(KIND == 1 || KT == 8, "the reduce-scatter of the reflection sums takes 8 bins per thread");
-    constexpr int VR = RS<TPL>::VR;
+    constexpr int VR = RS<TPL>::VR, RL = row_pairs(KT), RX = row_floats(KT);
     extern __shared__ float4 smem4[];
     const int PT = g.PT, NS = g.NS, TP = g.TP, KB = g.KB;
     const Buf B0 = buf_at<KT>(smem4, g, 0), B1 = buf_at<KT>(smem4, g, 1);
@@ -182,20 +182,20 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
     const u64 ArS = pk2(ars, ars), nAiS = pk2(nais, nais);
     const u64 D1r = pk2(-j.a_step, -j.a_step), nD1i = pk2(-j.w_step, -j.w_step);
 
-    const float invNS = 1.0f / (float)NS, invKB = 1.0f / (float)KB;
+    const float invKB = 1.0f / (float)KB;
     if (t0 < t1) {
         if (g.mat_cached) {
             const int nm = a.n_mat_tab;
             for (int e = tid; e < nm * KB; e += nthr) {
                 const int mat = e / KB, i = e - mat * KB;
-                const int kk = __float2int_rz(((float)i + 0.5f) * invNS), s_ = i - kk * NS;
-                const int k = min(kb + s_ * KT + kk, a.F - 1);
+                const int k = min(kb + i, a.F - 1);
                 if (KIND == 0) {
                     mt[e] = a.lk[(int64_t)mat * a.F + k];
-                    mt[nm * KB + e] = a.g2[(int64_t)mat * a.F + k];
+                    // (finite: a path that is not there has -gamma^2 = 0)
+                    mt[nm * KB + mat * g.RX + (i / KT) * RX + i % KT] = fminf(a.g2[(int64_t)mat * a.F + k], 3.0e38f);
                 } else if (g.mat_direct) {  // the factor itself, as a pair for the two microphones of a thread
-                    const float x = (kb + s_ * KT + kk < a.F) ? ex2(a.lid[(int64_t)mat * a.F + k]) : 0.0f;
-                    reinterpret_cast<u64*>(mt)[e] = pk2(x, x);
+                    const float x = (kb + i < a.F) ? ex2(a.lid[(int64_t)mat * a.F + k]) : 0.0f;
+                    reinterpret_cast<u64*>(mt)[mat * g.RB + (i / KT) * RL + i % KT] = pk2(x, x);
                 } else {
                     mt[e] = a.lid[(int64_t)mat * a.F + k];
                 }
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
         }
         cp_async_wait_all();
         __syncthreads();
-        produce<KT, KIND, 1>(a, g, B0, pdb, pvb, mt, mic0, kb, invNS, invKB, j.s, t0 * PT);
+        produce<KT, KIND, 1>(a, g, B0, pdb, pvb, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, j.s, t0 * PT);
         chain_counts(pdb, pvb, pcb, psg);
         __syncthreads();
     }
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
         }
         if (tile + 1 < t1) {
             const int nb = (int)((tile + 1 - t0) % 3);
-            produce<KT, KIND, 1>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, mic0, kb, invNS, invKB, j.s,
+            produce<KT, KIND, 1>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, j.s,
                                  (tile + 1) * PT);
             chain_counts(pdb + nb * PT * 12, pvb + nb * PT, pcb + nb * PT, psg + nb * PT);
         }
@@ -238,8 +238,8 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
         for (int kk = 0; kk < KT; ++kk) Y[kk] = 0.0f;
         for (int p = 0; p < PT; ++p) {
             const ulonglong2 z0 = C.za[(p * NS + s) * TP + tp];
-            const u64* w = C.wst + p * 4 * TP + tp;  // component-major: conflict-free 64-bit loads
-            const u64 w1r = w[0], w1i = w[TP], w2r = w[2 * TP], w2i = w[3 * TP];
+            const ulonglong2 w1 = C.wst[p * 2 * TP + tp], w2 = C.wst[(p * 2 + 1) * TP + tp];
+            const u64 w1r = w1.x, w1i = w1.y, w2r = w2.x, w2i = w2.y;
             const u64 nw2i = fmul2(w2i, pk2(-1.0f, -1.0f));
             const u64 ng = C.ngp[p * TP + tp];
             u64 er = z0.x, ei = z0.y, orr = er, oi = ei;
@@ -247,9 +247,10 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
             u64 c0r = 0ull, c0i = 0ull, qr = 0ull, qi = 0ull, cg = 0ull;
             u64 c1r = 0ull, c1i = 0ull;  // diffraction: C1 = sum_kk kk conj(G) T directly
             const float2 ngv = up2(ng);  // -gamma^2 of the two microphones (lobe sums)
-            const float2* trow = reinterpret_cast<const float2*>(C.tab) + p * KB + s;
+            const float* xrow = C.tab + (p * NS + s) * RX;
+            const float* grow = reinterpret_cast<const float*>(smem4) + (KIND == 0 ? C.goff[p] : 0) + s * RX;
             // diffraction with the material table read directly: row offset left by the producer in ngp
-            const u64* mrow = reinterpret_cast<const u64*>(mt) + s;
+            const u64* mrow = reinterpret_cast<const u64*>(mt) + s * RL;
             if (KIND == 1 && g.mat_direct) mrow += (int)(uint32_t)ng;
             if (KIND == 1) {
                 // Diffraction (positions only): with u_kk = conj(G_kk) E_kk and z_kk = z0 W^kk,
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
                 // P and P' by Horner's scheme from the top bin (no explicit phasor chain).
                 const u64 nw1i = fmul2(w1i, pk2(-1.0f, -1.0f));
                 auto Eat = [&](int kk) -> u64 {
-                    return g.mat_direct ? mrow[kk * NS] : reinterpret_cast<const u64*>(trow)[kk * NS];
+                    return g.mat_direct ? mrow[kk] : pk2(xrow[kk], xrow[kk]);
                 };
                 u64 E = Eat(KT - 1);
                 u64 pr = fmul2(Gr[KT - 1], E), pim = fmul2(Gi[KT - 1], E), dpr = 0ull, dpi = 0ull;
@@ -280,9 +281,17 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
                 c1r = ffma2(er, tr, fmul2(fmul2(ei, pk2(-1.0f, -1.0f)), ti));
                 c1i = ffma2(er, ti, fmul2(ei, tr));
             } else {
+                float4 x4, g4;
 #pragma unroll
                 for (int kk = 0; kk < KT; ++kk) {  // specular
-                    const float2 t = trow[kk * NS];  // (log2 X, g)
+                    if ((kk & 3) == 0) {
+                        x4 = *reinterpret_cast<const float4*>(xrow + kk);
+                        g4 = *reinterpret_cast<const float4*>(grow + kk);
+                    }
+                    const float2 t = (kk & 3) == 0   ? make_float2(x4.x, g4.x)  // (log2 X, g)
+                                     : (kk & 3) == 1 ? make_float2(x4.y, g4.y)
+                                     : (kk & 3) == 2 ? make_float2(x4.z, g4.z)
+                                                     : make_float2(x4.w, g4.w);
                     const u64 E = pk2(ex2(fmaf(ngv.x, t.y, t.x)), ex2(fmaf(ngv.y, t.y, t.x)));
                     const u64 zr = (kk & 1) ? orr : er, zi = (kk & 1) ? oi : ei;
                     const u64 Tr = fmul2(E, zr), Ti = fmul2(E, zi);
@@ -687,8 +696,7 @@ cudaError_t launch_adjoint(const AccumArgs& a, const AdjointArgs& j, const Geom&
 namespace {
 
 size_t adjoint_per_path(const acc::Geom& g) {
-    return (g.mat_direct ? (size_t)0 : (size_t)g.KB * 8) + (size_t)g.NS * g.TP * 16 + (size_t)g.TP * 40 +
-           (size_t)g.TP * 56;
+    return acc::tab_bytes(g) + (size_t)g.NS * g.TP * 16 + (size_t)g.TP * 40 + 4 + (size_t)g.TP * 56;
 }
 
 }  // namespace
@@ -713,7 +721,7 @@ acc::Geom adjoint_geom(int M, int F, int n_mat, int mat_direct, int tp_max, int 
     const size_t per_path = adjoint_per_path(g);
     const size_t per_tile = 2 * per_path + 3 * 52;
     const size_t fixed = (g.mat_cached ? g.mat_bytes : 0) + 16 + 64 + 512;
-    const size_t budget = 100 * 1024;
+    const size_t budget = 108 * 1024;
     g.PT = (int)std::max<size_t>(1, std::min<size_t>(8, budget > fixed ? (budget - fixed) / per_tile : 1));
     g.buf_bytes = (per_path * g.PT + 255) & ~size_t(255);
     g.smem = adjoint_smem(g);

@@ -616,7 +616,7 @@ struct InstLeafBox {
 // (Meister and Bittner, TVCG 2018.)  Clusters start as the triangles in Morton order; in every round each looks kPlocR
 // places to either side for the neighbour whose union with it has the least surface, and clusters that choose each other
 // merge.  Against the radix tree over the Morton codes (below, kept for prototypes and instances and as the way out):
-// closest-hit queries of a 1M-triangle clutter visit 9.4 wide nodes instead of 20.8, of the instanced forest 29 instead
+// closest-hit queries of a 1M-triangle clutter visit 9.4 wide nodes instead of 20.8, of a forest 29 instead
 // of 57 (large triangles beside small ones spoil the radix tree's boxes), among equal leaves 58 instead of 63; the passes
 // over these took 9.52 ms instead of 10.15, 2.71 instead of 3.56, 13.7 instead of 14.7.  A round is two launches; the last
 // kPlocLast clusters merge in one block.  What bounds it is the chain of rounds (200k triangles: 23 of ~8 us each and one

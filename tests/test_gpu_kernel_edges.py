@@ -104,6 +104,23 @@ def test_general_tile_bin_blocks_match_oracle(torch_st, n_mics, n_bins):
     simulate_and_compare(st, wl, budget=3_000)
 
 
+# the general accumulator's per-bin rows: materials that do and do not fit shared memory (lobe exponents from the material
+# table or from rows of their own), an emitter table, last-material reflection, paths that some microphones do not see
+@pytest.mark.parametrize("n_mat,etab,mode,los", [(4, True, 0, 0), (60, False, 0, 0), (60, True, 1, 0), (3, False, 1, 1)])
+def test_general_tile_rows_match_oracle(torch_st, n_mat, etab, mode, los):
+    _, st = torch_st
+    rng = np.random.default_rng(9)
+    wl = synth.clutter(seed=15, target_tris=2_500, n_rays=1_200, bounces=5, n_mics=12, n_bins=141)
+    wl.mics = (wl.mics + rng.uniform(-4, 4, wl.mics.shape) * [1, 1, 0.1]).astype(np.float32)
+    wl.tri_mat = (np.arange(wl.n_tris) % n_mat).astype(np.int32)
+    wl.k_band = synth.smooth_band_curves(rng, n_mat, 16, 0.3, 0.95)
+    wl.beta_band = np.deg2rad(synth.smooth_band_curves(rng, n_mat, 16, 5.0, 30.0)).astype(np.float32)
+    wl.diff_band = synth.smooth_band_curves(rng, n_mat, 16, 0.02, 0.08)
+    if etab:
+        wl.emitter_table = rng.uniform(0.1, 1.0, (37, 141)).astype(np.float32)
+    simulate_and_compare(st, wl, budget=3_000, reflection_mode=mode, los_mode=los)
+
+
 # fused bounce launches: one ray, fewer queries than warps, a few lanes a warp, full warps; the last launch (visibility
 # only) after a single bounce and after the most; both receiver tests
 @pytest.mark.parametrize("n_rays,bounces,los", [(1, 1, 0), (33, 8, 0), (20_001, 2, 0), (60_007, 3, 0), (170_003, 2, 0),
