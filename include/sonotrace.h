@@ -158,11 +158,11 @@ st_status st_scene_load(st_ctx* ctx, const float* verts, int64_t n_verts, const 
  * centres (beta through the lobe exponent 1/(2 beta^2)) and constant beyond the end bands. */
 st_status st_scene_set_materials(st_scene* scene, int32_t n_mat, int32_t n_bands, const float* band_hz,
                                  const float* k, const float* beta, const float* diffr);
-/* Build the device LBVH, triangle normals, curvature (G_v, C_i) and diffraction CDFs.
+/* Build the device hierarchy, triangle normals, curvature (G_v, C_i) and diffraction CDFs.
  * params may be NULL (defaults).  Synchronises the stream once (to size the sample buffers). */
 st_status st_scene_precompute(st_scene* scene, const st_curv_params* params);
 /* Dynamic scenes: new positions for the same vertices (n_verts [3] floats, host or device per mem)
- * of a precomputed scene, then a refit: the LBVH topology and leaf order of the last precompute are
+ * of a precomputed scene, then a refit: the hierarchy's topology and leaf order of the last precompute are
  * kept and the boxes, wide nodes, leaf triangles and normals recomputed (results stay exact: the
  * boxes are conservative for any positions, only the traversal cost can grow with large motions).
  * Welding, curvature, metric, CDFs and sample counts are recomputed too, unless flags holds
@@ -344,7 +344,7 @@ typedef struct st_job {
 
 /* Launch shapes picked by st_autotune (0 = default). */
 typedef struct st_tune {
-    int32_t rays_per_block;     /* tracing block size: 64, 128 or 256 */
+    int32_t rays_per_block;     /* tracing block size: 64, 128 or 256 (256 traces in blocks of 128) */
     int32_t mic_pairs_per_cta;  /* accumulator: microphone pairs per CTA, 1..16 */
     int32_t smem_kb;            /* accumulator: shared-memory budget per CTA, 32..160 KB */
     int32_t stack_depth;        /* traversal stack entries per query, 1..128 (0 = 128).  A query that would

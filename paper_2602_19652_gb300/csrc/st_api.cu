@@ -2546,11 +2546,11 @@ st_status st_autotune(st_ctx* c, const st_job* J, const st_sim_params* params, s
     const bool saved_overlap = c->overlap;
     c->overlap = false;  // each stage timed on its own
     const int rpb[3] = {64, 128, 256};
-    const int tiles[5][2] = {{16, 96}, {8, 96}, {16, 64}, {4, 96}, {16, 128}};
+    const int tiles[5][2] = {{16, 108}, {8, 108}, {16, 64}, {4, 108}, {16, 128}};
     const int kts[2] = {16, 8};
     const int depths[3] = {0, 48, 24};
     const int refills[4] = {0, 12, 20, 32};
-    st_tune best = {128, 16, 96, 0, 0, 0};
+    st_tune best = {128, 16, 108, 0, 0, 0};
     // one parameter at a time, each with the best of the earlier ones: the tracing block size, the accumulator
     // tile (microphone pairs and shared memory), its bins per thread (frequency tile), the traversal stack depth
     // and the lane-refill threshold (rays per warp refill); tracing phases are timed on tracing and diffraction,

@@ -65,12 +65,12 @@ struct SceneDev {
     DevBuf tri_mat;    // [T] i32
     DevBuf tri_obj;    // [T] i32
     DevBuf nrm;        // [T][3] f32 geometric normals (input triangle order)
-    // LBVH
+    // hierarchy
     DevBuf nodes;      // 4-wide BVH: [n4][8] float4: lo.x, hi.x, lo.y, hi.y, lo.z, hi.z of the 4 children, refs, pad
     DevBuf tri_v;      // [T][3] float4 in leaf order; tri_v[3i].w = triangle index bits
     int32_t root = 0;  // child-ref encoding of the root
     int64_t n_nodes = 0;  // 4-wide nodes
-    // LBVH topology kept for refits: binary children, leaf ranges, parents, leaf order, wide-node flags
+    // topology kept for refits: binary children, leaf ranges, parents, leaf order, wide-node flags
     // and numbering
     DevBuf bvh_child, bvh_range, bvh_par_i, bvh_par_l, bvh_perm, bvh_wflag, bvh_widx;
     bool bvh_ready = false;
@@ -152,8 +152,8 @@ struct CurvParamsDev {
     uint64_t seed;
 };
 // Validates indices and vertices (flags), computes normals, welds, curvature, C, CDFs, sample
-// counts and the LBVH.  Synchronises once.  Returns a CUDA error or sets *mesh_error.
-// refit: keep the LBVH topology of an earlier build (new vertex positions, same triangles): boxes,
+// counts and the hierarchy.  Synchronises once.  Returns a CUDA error or sets *mesh_error.
+// refit: keep the topology of an earlier build (new vertex positions, same triangles): boxes,
 // wide nodes and leaf triangles are recomputed; keep_curvature: also keep curvature, metric, CDFs and
 // sample counts (valid for rigid motions of whole meshes)
 cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bool* mesh_error, std::string* msg,

@@ -1307,7 +1307,7 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
 
     }  // !keep_curvature
 
-    // ---- LBVH
+    // ---- hierarchy
     {
         uint32_t init[6] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
         CK(cudaMemcpyAsync(w.bnd, init, sizeof(init), cudaMemcpyHostToDevice, s));
