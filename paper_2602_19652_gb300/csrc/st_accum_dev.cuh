@@ -622,10 +622,11 @@ inline Geom make_geom(int M, int F, int KT, int n_mat, int tp_max = 8, size_t bu
     const int ns_need = (F + KT - 1) / KT;
     g.TP = std::max(1, std::min(pairs, tp_max));
     g.NS = std::max(1, std::min(ns_need, 256 / g.TP));
-    if (balance && g.NS > 2 && g.NS * KT <= 512) {
+    if (balance && g.NS > 2 && g.NS * KT <= 400) {
         // bins spread evenly over their blocks (104k paths: 32 microphones x 257 bins, whose second block held one bin,
-        // 0.75 -> 0.63 ms; 17 x 257 0.50 -> 0.36; 24 x 512 1.06 -> 0.65), in subtiles a multiple of four.  Blocks of more
-        // than 512 bins stay, and with them the distance a phasor's rounding grows over.
+        // 0.75 -> 0.63 ms; 24 x 512 1.06 -> 0.65), in subtiles a multiple of four.  Blocks of more than 400 bins (18
+        // microphones and fewer) stay, and with them the places where a phasor starts anew: its rounding grows over a
+        // block, to 1.5e-5 of a spectrum at 512 bins, and other blocks would differ by as much.
         const int blocks = (ns_need + g.NS - 1) / g.NS, ns = (ns_need + blocks - 1) / blocks, ns4 = (ns + 3) & ~3;
         g.NS = ns4 * g.TP <= 256 ? ns4 : ns;
     }
