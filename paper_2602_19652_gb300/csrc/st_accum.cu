@@ -6,7 +6,8 @@
 // The work is (paths x microphones x bins).  A CTA owns a tile of microphones x bins and streams
 // a chunk of paths in tiles of P_T; partial spectra of the chunks are summed afterwards in a fixed
 // order (deterministic, no float atomics).  Per path tile:
-//   1a. per (path, bin):  log2(X_p(k) D_e) and the lobe exponent g(T_p, f_k)   -> shared memory
+//   1a. per (path, bin):  log2(X_p(k) D_e)   -> shared memory (the lobe exponent g(T_p, f_k) is read from the CTA's
+//       material table, or from a row beside it where that does not fit)
 //   1b. per (path, mic):  r = r_pre + |m - P| in float-float (~44 bits), gamma^2, the phasor at the
 //       first bin of every thread's bin run (range-reduced phase, sincospi), and the per-bin step
 //       W = 2^(r log2-decay per bin) e^(j 2 pi frac(r df / c))                   -> shared memory

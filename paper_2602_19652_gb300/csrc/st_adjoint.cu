@@ -710,7 +710,7 @@ size_t adjoint_smem(const acc::Geom& g) {
 acc::Geom adjoint_geom(int M, int F, int n_mat, int mat_direct, int tp_max, int kt) {
     // tile shape of the forward with kt bins per thread (8 where the reflection sums are reduce-scattered across
     // the pair lanes, 16 for diffraction paths) and up to tp_max microphone pairs per CTA, the pair count a power
-    // of two; paths per tile as many as fit about 100 KB, so that two CTAs share an SM
+    // of two; paths per tile as many as fit about 108 KB (8 at 32 microphones), so that two CTAs share an SM
     acc::Geom g = acc::make_geom(M, F, kt, n_mat, tp_max, 200 * 1024, 0, mat_direct);
     int tp2 = 1;
     while (tp2 * 2 <= g.TP) tp2 *= 2;
