@@ -74,7 +74,9 @@ __global__ void k_tables(int32_t F, int32_t n_mat, int32_t n_bands, const float*
     }
     double dv = interp(drow);
     lk[idx] = kv > 0.0 ? (float)log2(kv) : kNegInf;
-    g2[idx] = (float)(gv * 1.4426950408889634);
+    // finite for any beta > 0: the exponent is multiplied by gamma^2, which is 0 for a microphone that does not see the path
+    // and may be 0 for one that does
+    g2[idx] = (float)fmin(gv * 1.4426950408889634, 3.0e38);
     lid[idx] = dv > 0.0 ? (float)log2(dv) : kNegInf;
     if (mat == 0) {
         double q = f / c;
@@ -133,8 +135,7 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
                 const int k = min(kb + i, a.F - 1);
                 if (KIND == 0) {
                     mt[e] = a.lk[(int64_t)mat * a.F + k];
-                    // (finite: a path that is not there has -gamma^2 = 0)
-                    mt[nm * KB + mat * g.RX + (i / KT) * RX + i % KT] = fminf(a.g2[(int64_t)mat * a.F + k], 3.0e38f);
+                    mt[nm * KB + mat * g.RX + (i / KT) * RX + i % KT] = a.g2[(int64_t)mat * a.F + k];
                 } else if (g.mat_direct) {  // the factor itself, as a pair for the two microphones of a thread
                     const float x = (kb + i < a.F) ? ex2(a.lid[(int64_t)mat * a.F + k]) : 0.0f;
                     reinterpret_cast<u64*>(mt)[mat * g.RB + (i / KT) * RL + i % KT] = pk2(x, x);

@@ -191,8 +191,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
                 const int k = min(kb + i, a.F - 1);
                 if (KIND == 0) {
                     mt[e] = a.lk[(int64_t)mat * a.F + k];
-                    // (finite: a path that is not there has -gamma^2 = 0)
-                    mt[nm * KB + mat * g.RX + (i / KT) * RX + i % KT] = fminf(a.g2[(int64_t)mat * a.F + k], 3.0e38f);
+                    mt[nm * KB + mat * g.RX + (i / KT) * RX + i % KT] = a.g2[(int64_t)mat * a.F + k];
                 } else if (g.mat_direct) {  // the factor itself, as a pair for the two microphones of a thread
                     const float x = (kb + i < a.F) ? ex2(a.lid[(int64_t)mat * a.F + k]) : 0.0f;
                     reinterpret_cast<u64*>(mt)[mat * g.RB + (i / KT) * RL + i % KT] = pk2(x, x);

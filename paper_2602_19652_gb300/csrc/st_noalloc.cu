@@ -84,7 +84,7 @@ __global__ void k_na_tables(int F, int n_mat, int n_bands, const float* band, co
         g = (1.0 - w) * g + w / (2.0 * (double)br[b0 + 1] * (double)br[b0 + 1]);
     }
     lk[idx] = kv > 0.0 ? (float)log2(kv) : -__builtin_huge_valf();
-    g2[idx] = (float)(g * 1.4426950408889634);
+    g2[idx] = (float)fmin(g * 1.4426950408889634, 3.0e38);  // (finite: a path may have gamma = 0)
     if (mat == 0) {
         const double q = f / c;
         const float h = (float)q;
