@@ -352,8 +352,9 @@ typedef struct st_tune {
                                    child order, parent references in the nodes), keeping its best hit, so
                                    results do not depend on it; st_stats.stack_restarts counts the restarts */
     int32_t refill_lanes;       /* rays per warp refill: the persistent traversal kernels give new queries to a
-                                   warp's idle lanes once this many of its 32 lanes wait, 1..32 (0 = 16 for
-                                   closest hits, 28 for visibility rays) */
+                                   warp's idle lanes once this many of its lanes wait, 1..32, at most those that
+                                   the launch uses (0 = 16 where closest hits are traced, alone or beside the
+                                   visibility rays of the bounce before; 28 for visibility rays alone) */
     int32_t bins_per_thread;    /* frequency tile: bins a thread of the general accumulator advances, 8 or 16
                                    (0 = 16; the batched form takes 16) */
 } st_tune;

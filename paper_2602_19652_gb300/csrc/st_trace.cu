@@ -58,7 +58,7 @@ __global__ void ST_TRAV_BOUNDS k_bounce(const TraceArgs a, int j, int lanes) {
     const uint32_t* vis_in = a.vis_q[(j & 1) ^ 1];
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const int refill = min(T.refill > 0 ? T.refill : kRefillClosest, max(1, lanes / 2));
+    const int refill = refill_at(T.refill, kRefillClosest, lanes, lanes / 2);
     int2 stack[kStack];
     typename TravStateOf<TL>::type S;
     uint32_t id = 0;  // ray of a closest-hit query, record of a visibility query
@@ -214,7 +214,7 @@ __global__ void ST_TRAV_BOUNDS k_visible(const Trav T, const uint32_t* queue, co
     typename TravStateOf<TL>::type S;
     int64_t id = -1;
     bool live = false, exhausted = (int)(threadIdx.x & 31) >= lanes;
-    const int refill = min(T.refill > 0 ? T.refill : kRefillAny, max(1, lanes - 4));
+    const int refill = refill_at(T.refill, kRefillAny, lanes, lanes - 4);
     while (true) {
         const bool need = !live && !exhausted;
         const int64_t idx = claim(ctr, need);

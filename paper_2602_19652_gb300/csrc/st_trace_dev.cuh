@@ -540,6 +540,12 @@ constexpr int kTravBlock = 128;
 // any-hit kernels)
 constexpr int kRefillClosest = 16;
 constexpr int kRefillAny = 28;
+// that number for a warp of `lanes` lanes in use: the caller's where one is set, else the kernel's default kept
+// below the lanes in use (most: the largest default that still leaves lanes at work)
+__host__ __device__ __forceinline__ int refill_at(int tuned, int dflt, int lanes, int most) {
+    const int n = tuned > 0 ? (tuned < lanes ? tuned : lanes) : (dflt < most ? dflt : most);
+    return n > 1 ? n : 1;
+}
 
 // Visibility of `target` from o: direction normalize(target - o), t in (t_min, |target - o| - eps).
 template <bool TL = false>
