@@ -14,8 +14,8 @@ pytestmark = pytest.mark.gpu
 def test_lobes_beyond_float32(torch_st, n_mics, n_bins, n_mat):
     _, st = torch_st
     rng = np.random.default_rng(5)
-    wl = synth.clutter(seed=12, target_tris=2_500, n_rays=1_500, bounces=3, n_mics=n_mics, n_bins=n_bins)
-    wl.mics = (wl.mics + rng.uniform(-4, 4, wl.mics.shape) * [1, 1, 0.1]).astype(np.float32)
+    wl = synth.clutter(seed=12, target_tris=20_000, n_rays=1_500, bounces=3, n_mics=n_mics, n_bins=n_bins)
+    wl.mics = rng.uniform([2, 2, 0.3], [18, 18, 2], (n_mics, 3)).astype(np.float32)
     wl.tri_mat = (np.arange(wl.n_tris) % n_mat).astype(np.int32)
     wl.k_band = synth.smooth_band_curves(rng, n_mat, 16, 0.3, 0.95)
     wl.beta_band = np.deg2rad(synth.smooth_band_curves(rng, n_mat, 16, 5.0, 30.0)).astype(np.float32)
