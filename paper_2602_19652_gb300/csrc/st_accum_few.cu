@@ -332,7 +332,7 @@ FewGeom few_geom(const AccumArgs& a) {
     g.direct = a.kind == 1 && !a.etab && g.cached ? 1 : 0;
     const int per_path = g.TM * (8 * g.NS + 12) + (g.direct ? 0 : g.NS * st * 4) + 4;
     const int fixed = (g.cached ? rows : 0) + g.TM * 12 + 64;
-    const int budget = a.tile_kb > 0 ? a.tile_kb * 1024 : 72 * 1024;  // three CTAs per SM
+    const int budget = few_budget(a.tile_kb);
     const int most = std::max(1, std::min(128, (budget - fixed) / (2 * per_path + 2 * 52)));
     while (g.PG > most) g.PG = (g.PG + 1) / 2;
     // paths per tile: about two rounds of anchors for the CTA's threads

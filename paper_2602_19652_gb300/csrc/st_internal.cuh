@@ -383,6 +383,9 @@ int32_t accum_chunks(const AccumArgs& a, int64_t n_paths);
 // 0.29 / 0.24, 64 x 48 0.27 / 0.31, 64 x 64 0.39 / 0.28, 17 x 96 0.16 / 0.21, 17 x 128 0.22 / 0.21, 10 x 331 0.31 /
 // 0.34, 10 x 512 0.61 / 0.40, 6 x 512 0.29 / 0.39, 3 x 331 0.14 / 0.39, 3 x 1024 0.56 / 1.47).
 inline bool few_accum(int32_t M, int32_t F) { return M > 2 && (int64_t)M * F <= 3400 && (F <= 96 || M <= 10); }
+// Its shared memory in bytes for the caller's smem_kb (0: none): three CTAs an SM, as its registers allow, so a larger budget
+// only takes one away (10 microphones x 330 bins: 72 KB 0.50 ms a call, 108 KB 0.55, 128 KB 0.61).
+inline int few_budget(int32_t smem_kb) { return (smem_kb > 0 && smem_kb < 72 ? smem_kb : 72) * 1024; }
 int32_t few_chunks(const AccumArgs& a, int64_t n_paths);
 cudaError_t accumulate_few(const AccumArgs& a, cudaStream_t s);
 // emitter ray sets (st_rays.cu): kind 0 spherical Fibonacci, 1 zonal equal-area centres

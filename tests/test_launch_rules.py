@@ -34,3 +34,9 @@ def test_refill_lanes_are_the_callers(rules):
                                       "trv::refill_at(0, trv::kRefillAny, 32, 28)",
                                       "trv::refill_at(0, trv::kRefillClosest, 4, 2)",
                                       "trv::refill_at(0, trv::kRefillClosest, 1, 0)"]) == [16, 28, 2, 1]
+
+
+def test_few_bin_budget_keeps_three_ctas(rules):
+    """A budget set for the general accumulator's two CTAs an SM does not reach the few-bin kernel; a smaller one does."""
+    assert rules("st_internal.cuh", [f"few_budget({kb})" for kb in (0, 32, 71, 72, 73, 108, 160)]) == [
+        1024 * kb for kb in (72, 32, 71, 72, 72, 72, 72)]
