@@ -615,7 +615,7 @@ struct InstLeafBox {
 // ---------------------------------------------------------------- hierarchy by parallel locally-ordered clustering
 // (Meister and Bittner, TVCG 2018.)  Clusters start as the triangles in Morton order; in every round each looks kPlocR
 // places to either side for the neighbour whose union with it has the least surface, and clusters that choose each other
-// merge.  Against the radix tree over the Morton codes (below, kept for prototypes and instances and as the way out):
+// merge.  Against the radix tree over the Morton codes (below, kept for prototypes and instances):
 // closest-hit queries of a 1M-triangle clutter visit 9.4 wide nodes instead of 20.8, of a forest 29 instead
 // of 57 (large triangles beside small ones spoil the radix tree's boxes), among equal leaves 58 instead of 63; the passes
 // over these took 9.52 ms instead of 10.15, 2.71 instead of 3.56, 13.7 instead of 14.7.  A round is two launches; the last
@@ -623,8 +623,10 @@ struct InstLeafBox {
 // block's 28 in 52 us, ~0.42 ms of device time, where the radix tree with its climbs for boxes takes 0.09).
 constexpr int kPlocR = 8;
 constexpr int kPlocLast = 1024;       // clusters that one block merges to the end, one a thread
-constexpr int kPlocRounds = 64;       // rounds of launches, and of the last block, at most before the radix tree is taken
-constexpr int kPlocLastRounds = 192;  // instead (a round adds at most one level, so they bound the depth as well)
+// Rounds can stall: of concentric shapes each prefers its smaller neighbour, and only the innermost two prefer each other.
+// After a round that left more than 15 of 16 clusters (ordinary meshes: 0.73 to 0.78 of them) neighbours in order are paired
+// where one lies within the other, and after another one all of them, so three rounds leave half at most.
+constexpr int kPlocRounds = 320;      // of launches, and of the last block, at most: 226 of 15/16 each from 2^31 clusters
 constexpr int kPlocThreads = 512;
 constexpr int kPlocTile = kPlocThreads - 2 * kPlocR;  // clusters per block of a round: the others are its margins
 
@@ -679,6 +681,19 @@ __device__ __forceinline__ int ploc_best(int i, int n, const Box& b, const F& bo
     return at;
 }
 
+// whether a round that found `before` clusters and left n hardly merged any
+__device__ __forceinline__ bool ploc_stalled(int before, int n) { return n > before - before / 16; }
+// the partner that cluster i chooses; stalls: how many of the last two rounds in a row stalled
+template <class F>
+__device__ __forceinline__ int ploc_choose(int i, int n, const Box& b, const F& box, int stalls) {
+    const int j = i ^ 1;
+    if (stalls > 0 && j < n) {
+        const Box o = box(j);
+        if (stalls > 1 || union_area(b, o) <= 1.125f * fmaxf(union_area(b, b), union_area(o, o))) return j;
+    }
+    return stalls > 1 ? -1 : ploc_best(i, n, b, box);
+}
+
 template <class LeafBox>
 __global__ void k_ploc_init(const LeafBox leaf, const PlocArgs a) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
@@ -711,6 +726,8 @@ __global__ void __launch_bounds__(kPlocThreads) k_ploc_mate(const PlocArgs a, in
     __shared__ int32_t nn[kPlocThreads];
     const int n = (int)a.count[it], base = (int)blockIdx.x * kPlocTile;
     if (base >= n) return;
+    const bool stalled = it > 0 && ploc_stalled((int)a.count[it - 1], n);
+    const int stalls = !stalled ? 0 : it > 1 && ploc_stalled((int)a.count[it - 2], (int)a.count[it - 1]) ? 2 : 1;
     const Box* box = it & 1 ? a.box[1] : a.box[0];
     for (int e = threadIdx.x; e < kPlocThreads + 2 * kPlocR; e += kPlocThreads) {
         const int i = base - 2 * kPlocR + e;
@@ -718,7 +735,8 @@ __global__ void __launch_bounds__(kPlocThreads) k_ploc_mate(const PlocArgs a, in
     }
     __syncthreads();
     const int at = base - kPlocR, i = at + (int)threadIdx.x;  // nn[e]: chosen by cluster at + e
-    nn[threadIdx.x] = i >= 0 && i < n ? ploc_best(i, n, t[threadIdx.x + kPlocR], [&](int j) { return t[j - at + kPlocR]; }) : -1;
+    auto boxes = [&](int j) { return t[j - at + kPlocR]; };
+    nn[threadIdx.x] = i >= 0 && i < n ? ploc_choose(i, n, t[threadIdx.x + kPlocR], boxes, stalls) : -1;
     __syncthreads();
     uint32_t kept = 0, merged = 0;
     if (i >= base && i < base + kPlocTile && i < n) {
@@ -801,8 +819,8 @@ __global__ void __launch_bounds__(kPlocThreads) k_ploc_merge(const PlocArgs a, i
     (it & 1 ? a.box[0] : a.box[1])[pos] = b;
 }
 
-// The last clusters (at most kPlocLast), a thread each, rounds in one block; *a.left: clusters left after at most
-// kPlocLastRounds (1).  About 28 dependent rounds: boxes, ids and sizes stay in shared memory, and one packed scan places
+// The last clusters (at most kPlocLast), a thread each, rounds in one block; *a.left: clusters left (1, or all of them if
+// they are more).  About 28 dependent rounds: boxes, ids and sizes stay in shared memory, and one packed scan places
 // both the clusters kept (low half) and the nodes made.
 __global__ void __launch_bounds__(kPlocLast) k_ploc_last(const PlocArgs a, int it) {
     __shared__ Box box[kPlocLast];
@@ -823,8 +841,9 @@ __global__ void __launch_bounds__(kPlocLast) k_ploc_last(const PlocArgs a, int i
         sizes[i] = size = r < 0 ? 1 : a.size[r];
     }
     __syncthreads();
-    for (int round = 0; n > 1 && round < kPlocLastRounds; ++round) {
-        if (i < n) nn[i] = ploc_best(i, n, b, [&](int j) { return box[j]; });
+    int stalls = 0;
+    for (int round = 0; n > 1 && round < kPlocRounds; ++round) {
+        if (i < n) nn[i] = ploc_choose(i, n, b, [&](int j) { return box[j]; }, stalls);
         __syncthreads();
         const int j = i < n ? nn[i] : -1;
         const bool both = j >= 0 && nn[j] == i, join = both && i < j, keep = i < n && (!both || join);
@@ -854,6 +873,7 @@ __global__ void __launch_bounds__(kPlocLast) k_ploc_last(const PlocArgs a, int i
             ref[pos] = r;
             sizes[pos] = size;
         }
+        stalls = ploc_stalled(n, (int)(all & 0xffffu)) ? min(stalls + 1, 2) : 0;
         n = (int)(all & 0xffffu);
         base += (int)(all >> 16);
         __syncthreads();
@@ -1082,12 +1102,10 @@ static PlocArgs ploc_pieces(Pieces& m, int n, Box* box_tmp) {
 }
 
 // Clustered hierarchy over n leaves in the order perm (permuted to the new leaf order): children, ranges and parents in the
-// radix tree's form, and the boxes.  *done = false, and none of these changed but the boxes, when the clusters did not
-// merge within the bounds.
+// radix tree's form, and the boxes.
 template <class LeafBox>
 static cudaError_t ploc_build(const LeafBox& leaf, const PlocArgs& a, uint32_t* perm, int2* child, int2* range,
-                              int32_t* par_i, int32_t* par_l, cudaStream_t s, bool* done) {
-    *done = false;
+                              int32_t* par_i, int32_t* par_l, cudaStream_t s) {
     const int n = a.n, tiles = (n + kPlocTile - 1) / kPlocTile;
     note_launch();
     k_ploc_init<<<grid_for(n, kB), kB, 0, s>>>(leaf, a);
@@ -1097,9 +1115,9 @@ static cudaError_t ploc_build(const LeafBox& leaf, const PlocArgs& a, uint32_t* 
     uint32_t h_left = (uint32_t)n;
     for (;;) {
         int more = 0;
-        for (double c = h_left; c > kPlocLast && more < kPlocRounds; c *= 0.79) ++more;
-        more = std::min(more, kPlocRounds - it);
-        for (int r = 0; r < more; ++r, ++it) {
+        for (double c = h_left; c > kPlocLast && it + more < kPlocRounds; c *= 0.79) ++more;
+        double left = h_left;
+        for (int r = 0; r < more; ++r, ++it, left *= 0.79) {
             note_launch();
             k_ploc_mate<<<(unsigned)tiles, kPlocThreads, 0, s>>>(a, it);
             CK(cudaGetLastError());
@@ -1114,16 +1132,14 @@ static cudaError_t ploc_build(const LeafBox& leaf, const PlocArgs& a, uint32_t* 
         CK(cudaStreamSynchronize(s));
         if (h_left <= (uint32_t)kPlocLast || it >= kPlocRounds) break;
     }
-    if (h_left != 1) return cudaSuccess;
+    if (h_left != 1) return cudaErrorUnknown;  // (not reached: the bounds above)
     CK(cudaMemcpyAsync(a.perm_in, perm, (size_t)n * 4, cudaMemcpyDeviceToDevice, s));
     note_launch();
     k_ploc_layout<<<grid_for(n, kB), kB, 0, s>>>(a, perm, a.mate);
     CK(cudaGetLastError());
     note_launch();
     k_ploc_emit<<<grid_for(n, kB), kB, 0, s>>>(a, a.mate, child, range, par_i, par_l);
-    CK(cudaGetLastError());
-    *done = true;
-    return cudaSuccess;
+    return cudaGetLastError();
 }
 
 static cudaError_t build_two_level(SceneDev& S, float pad_world, uint32_t* flags, cudaStream_t s);
@@ -1359,7 +1375,6 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
                 S.root = 0;
                 int2* child_p = ptr<int2>(S.bvh_child);
                 int2* range_p = ptr<int2>(S.bvh_range);
-                bool clustered = false;  // which made the boxes as well
                 if (!refit) {
                     CK(grow(S.bvh_child, (size_t)(n - 1) * sizeof(int2)));
                     CK(grow(S.bvh_range, (size_t)(n - 1) * sizeof(int2)));
@@ -1368,15 +1383,8 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
                     child_p = ptr<int2>(S.bvh_child);
                     range_p = ptr<int2>(S.bvh_range);
                     CK(ploc_build(TriLeafBox{V, T, ptr<uint32_t>(S.bvh_perm), pad}, w.ploc, ptr<uint32_t>(S.bvh_perm),
-                                  child_p, range_p, ptr<int32_t>(S.bvh_par_i), ptr<int32_t>(S.bvh_par_l), s, &clustered));
-                    if (!clustered) {
-                        note_launch();
-                        k_karras<<<grid_for(n - 1, kB), kB, 0, s>>>(w.keys, n, child_p, range_p,
-                                                                    ptr<int32_t>(S.bvh_par_i), ptr<int32_t>(S.bvh_par_l));
-                        CK(cudaGetLastError());
-                    }
-                }
-                if (!clustered) {
+                                  child_p, range_p, ptr<int32_t>(S.bvh_par_i), ptr<int32_t>(S.bvh_par_l), s));
+                } else {
                     CK(cudaMemsetAsync(w.visits, 0, (size_t)(n - 1) * 4, s));
                     note_launch();
                     k_boxes<<<grid_for(n, kB), kB, 0, s>>>(TriLeafBox{V, T, ptr<uint32_t>(S.bvh_perm), pad}, n, child_p,
