@@ -636,6 +636,7 @@ struct PlocArgs {
     Box* box[2];
     int32_t* mate;          // per cluster of a round: its partner, or -1
     uint2* tiles;           // per tile of a round: clusters kept, merges
+    char* scan;             // scratch of their scan
     uint32_t* count;        // [kPlocRounds + 2] clusters at the start of a round
     uint32_t* nodes;        // [kPlocRounds + 2] nodes made before it
     int2* child;            // [n - 1] raw nodes
@@ -778,16 +779,24 @@ __device__ __forceinline__ uint2 block_excl2(uint2 v, uint2* s, int warps, uint2
     return make_uint2(before.x + x.x - v.x, before.y + x.y - v.y);
 }
 
+// SCANNED: a.tiles hold the sums up to and with each tile, else a block adds up the tiles before it itself, which grows with
+// the square of the clusters (kPlocSelf tiles, 4M clusters: 0.3 GB of reads from L2)
+constexpr int kPlocSelf = 8192;
+template <bool SCANNED>
 __global__ void __launch_bounds__(kPlocThreads) k_ploc_merge(const PlocArgs a, int it) {
     constexpr int kWarps = kPlocThreads / 32;
     __shared__ uint2 s[kWarps];
     const int n = (int)a.count[it], base = (int)blockIdx.x * kPlocTile;
     if (base >= n) return;
     uint2 pre = make_uint2(0u, 0u), own = make_uint2(0u, 0u), before, total;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kPlocThreads) {
-        const uint2 t = a.tiles[b];
-        pre.x += t.x;
-        pre.y += t.y;
+    if (SCANNED) {
+        if (threadIdx.x == 0 && blockIdx.x > 0) pre = a.tiles[blockIdx.x - 1];
+    } else {
+        for (int b = threadIdx.x; b < (int)blockIdx.x; b += kPlocThreads) {
+            const uint2 t = a.tiles[b];
+            pre.x += t.x;
+            pre.y += t.y;
+        }
     }
     const int i = base + (int)threadIdx.x;
     const bool live = (int)threadIdx.x < kPlocTile && i < n;
@@ -1089,6 +1098,7 @@ static PlocArgs ploc_pieces(Pieces& m, int n, Box* box_tmp) {
     }
     a.mate = m.take<int32_t>(n);
     a.tiles = m.take<uint2>((n + kPlocTile - 1) / kPlocTile);
+    a.scan = m.take<char>(scan_scratch_bytes((n + kPlocTile - 1) / kPlocTile));
     a.count = m.take<uint32_t>(kPlocRounds + 2);
     a.nodes = m.take<uint32_t>(kPlocRounds + 2);
     a.left = m.take<uint32_t>(1);
@@ -1121,8 +1131,15 @@ static cudaError_t ploc_build(const LeafBox& leaf, const PlocArgs& a, uint32_t* 
             note_launch();
             k_ploc_mate<<<(unsigned)tiles, kPlocThreads, 0, s>>>(a, it);
             CK(cudaGetLastError());
+            // (both counts of a tile as one 64-bit word: the sums of either stay below 2^32)
+            const bool scanned = left > (double)kPlocSelf * kPlocTile;
+            if (scanned) {
+                uint64_t* t64 = reinterpret_cast<uint64_t*>(a.tiles);
+                CK(inclusive_scan_u64(t64, t64, tiles, a.scan, s));
+            }
             note_launch();
-            k_ploc_merge<<<(unsigned)tiles, kPlocThreads, 0, s>>>(a, it);
+            if (scanned) k_ploc_merge<true><<<(unsigned)tiles, kPlocThreads, 0, s>>>(a, it);
+            else k_ploc_merge<false><<<(unsigned)tiles, kPlocThreads, 0, s>>>(a, it);
             CK(cudaGetLastError());
         }
         note_launch();

@@ -202,14 +202,23 @@ __global__ void __launch_bounds__(kCmpThreads) k_cmp_count(const uint8_t* __rest
     }
 }
 
-// the flagged indices in order; a block adds up the counts of the tiles before it itself (tiles of 4096 flags: 1,221 for
-// five million), and the last one writes the total
+// tiles up to which a block adds up the counts of the tiles before it itself: 8192 (34M flags) are 134 MB of reads from L2,
+// about 20 us; the sum grows with the square of the flags, so beyond it the counts are scanned first (three launches)
+constexpr unsigned kCmpSelf = 8192;
+
+// the flagged indices in order; SCANNED: counts hold the sums of the tiles before each (and *total is written), else the
+// tiles' own counts, and the last block writes the total
+template <bool SCANNED>
 __global__ void __launch_bounds__(kCmpThreads) k_cmp_write(const uint8_t* __restrict__ f, int64_t n,
                                                            const uint32_t* __restrict__ counts, uint32_t* __restrict__ idx,
                                                            uint32_t* __restrict__ total) {
     __shared__ uint32_t s_w[kRsWarps];
     uint32_t before = 0;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kCmpThreads) before += counts[b];
+    if (SCANNED) {
+        if (threadIdx.x == 0) before = counts[blockIdx.x];
+    } else {
+        for (int b = threadIdx.x; b < (int)blockIdx.x; b += kCmpThreads) before += counts[b];
+    }
     const int64_t i = (int64_t)blockIdx.x * kCmpTile + (int64_t)threadIdx.x * kCmpItems;
     uint32_t m = cmp_mask(f, i, n);
     const uint32_t c = (uint32_t)__popc(m);
@@ -218,7 +227,7 @@ __global__ void __launch_bounds__(kCmpThreads) k_cmp_write(const uint8_t* __rest
     __shared__ uint32_t s_base;
     if (threadIdx.x == kCmpThreads - 1) {
         s_base = before_incl;
-        if (blockIdx.x == gridDim.x - 1) *total = before_incl + incl;
+        if (!SCANNED && blockIdx.x == gridDim.x - 1) *total = before_incl + incl;
     }
     __syncthreads();
     uint32_t pos = s_base + incl - c;
@@ -370,7 +379,10 @@ cudaError_t fill_many(const Fill* f, int n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-size_t compact_scratch_bytes(int64_t n) { return (size_t)((n + kCmpTile - 1) / kCmpTile + 1) * 4; }
+size_t compact_scratch_bytes(int64_t n) {
+    const int64_t nb = (n + kCmpTile - 1) / kCmpTile;
+    return (((size_t)(nb + 1) * 4 + 255) & ~size_t(255)) + scan_scratch_bytes(nb);
+}
 
 cudaError_t compact_flags(const uint8_t* flags, int64_t n, uint32_t* idx, uint32_t* total, void* scratch,
                           cudaStream_t s) {
@@ -381,8 +393,14 @@ cudaError_t compact_flags(const uint8_t* flags, int64_t n, uint32_t* idx, uint32
     k_cmp_count<<<nb, kCmpThreads, 0, s>>>(flags, n, counts);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    const bool scanned = nb > kCmpSelf;
+    if (scanned) {
+        void* scan = static_cast<char*>(scratch) + (((size_t)(nb + 1) * 4 + 255) & ~size_t(255));
+        if ((e = exclusive_scan_u32(counts, counts, nb, total, scan, s)) != cudaSuccess) return e;
+    }
     note_launch();
-    k_cmp_write<<<nb, kCmpThreads, 0, s>>>(flags, n, counts, idx, total);
+    if (scanned) k_cmp_write<true><<<nb, kCmpThreads, 0, s>>>(flags, n, counts, idx, total);
+    else k_cmp_write<false><<<nb, kCmpThreads, 0, s>>>(flags, n, counts, idx, total);
     return cudaGetLastError();
 }
 
