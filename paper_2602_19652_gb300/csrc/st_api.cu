@@ -127,6 +127,7 @@ struct st_ctx {
     bool overlap = true;
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    DevBuf refit_scr;                // scratch of refits that keep the curvature
     DevBuf los_keys, los_scr, didx, dscratch, dpartial;
     // backward: the specular path list of the last simulate put in chain order (keys and sort scratch)
     bool paths_chain_order = false;
@@ -401,7 +402,7 @@ st_status st_destroy(st_ctx* c) {
         release(*b);
     for (auto& e : c->ev)
         if (e) cudaEventDestroy(e);
-    for (DevBuf* b : {&c->los_keys, &c->los_scr, &c->didx, &c->dscratch, &c->dpartial,
+    for (DevBuf* b : {&c->refit_scr, &c->los_keys, &c->los_scr, &c->didx, &c->dscratch, &c->dpartial,
                       &c->ck_keys, &c->ck_scr})
         release(*b);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
@@ -532,7 +533,7 @@ static st_status refit_scene(st_scene* sc, int32_t flags, const char* what) {
     std::string msg;
     const bool refit = sc->S.built;
     cudaError_t e = scene_build(sc->S, sc->cp, c->stream, &mesh_err, &msg, refit,
-                                refit && (flags & ST_REFIT_KEEP_CURVATURE) != 0);
+                                refit && (flags & ST_REFIT_KEEP_CURVATURE) != 0, &c->refit_scr);
     sc->version = g_scene_version++;
     if (e != cudaSuccess || mesh_err) sc->S.built = false;  // precompute again before the next simulate
     if (e != cudaSuccess) return cuda_fail(c, e, what);

@@ -155,9 +155,9 @@ struct CurvParamsDev {
 // counts and the hierarchy.  Synchronises once.  Returns a CUDA error or sets *mesh_error.
 // refit: keep the topology of an earlier build (new vertex positions, same triangles): boxes,
 // wide nodes and leaf triangles are recomputed; keep_curvature: also keep curvature, metric, CDFs and
-// sample counts (valid for rigid motions of whole meshes)
+// sample counts (valid for rigid motions of whole meshes); kept: scratch of such a refit, grown on demand and left to the caller
 cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bool* mesh_error, std::string* msg,
-                        bool refit = false, bool keep_curvature = false);
+                        bool refit = false, bool keep_curvature = false, DevBuf* kept = nullptr);
 
 // Instanced scene: the prototypes (concatenated) and the instance table, kept on the device so that new
 // transforms expand the world vertices again.  Instance i is a copy of prototype iproto[i]; it owns world

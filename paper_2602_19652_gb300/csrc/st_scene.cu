@@ -1162,7 +1162,7 @@ static cudaError_t ploc_build(const LeafBox& leaf, const PlocArgs& a, uint32_t* 
 static cudaError_t build_two_level(SceneDev& S, float pad_world, uint32_t* flags, cudaStream_t s);
 
 cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bool* mesh_error, std::string* msg,
-                        bool refit, bool keep_curvature) {
+                        bool refit, bool keep_curvature, DevBuf* kept) {
     *mesh_error = false;
     refit = refit && (S.two_level ? S.tl_ready : S.bvh_ready);
     keep_curvature = keep_curvature && refit;
@@ -1170,14 +1170,17 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
     const float* V = ptr<float>(S.verts);
     const int32_t* T = ptr<int32_t>(S.tris);
     const int32_t* obj = ptr<int32_t>(S.tri_obj);
-    DevBuf flags, scratch;
+    // A refit that keeps the curvature is a handful of launches, so its scratch (52 bytes a triangle) stays with the caller:
+    // whether an allocation found room in the driver's pages or mapped new ones made it 150 or 310 us at 8,000 triangles.
+    DevBuf flags, own;
+    DevBuf& scratch = keep_curvature && kept ? *kept : own;
     struct Guard {
         DevBuf &a, &b;
         ~Guard() {
             release(a);
             release(b);
         }
-    } guard{flags, scratch};
+    } guard{flags, own};
     CK(grow(flags, 16));
     CK(cudaMemsetAsync(flags.p, 0, 16, s));
     note_launch();
@@ -1196,6 +1199,7 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
     const int32_t n_obj = S.n_obj;  // known from the host copy
     const int64_t nmax = std::max<int64_t>(std::max<int64_t>(nv, nt), 1);
     const bool curv = !keep_curvature, flat = !S.two_level && nt > kLeafMax;
+    const bool sorts = curv || (!refit && !S.two_level);
     struct Scratch {
         uint32_t *bnd, *vals, *cnt, *off, *cursor, *cmax, *moff, *visits, *wtotal;
         uint64_t *keys, *Q, *S64;
@@ -1208,9 +1212,11 @@ cudaError_t scene_build(SceneDev& S, const CurvParamsDev& cp, cudaStream_t s, bo
     } w{};
     auto lay = [&](Pieces m) {
         w.bnd = m.take<uint32_t>(16);
-        w.keys = m.take<uint64_t>(nmax);
-        w.vals = m.take<uint32_t>(nmax);
-        w.sort_scr = m.take<char>(sort_scratch_bytes(nmax) + scan_scratch_bytes(nmax + n_obj + 1));
+        if (sorts) {
+            w.keys = m.take<uint64_t>(nmax);
+            w.vals = m.take<uint32_t>(nmax);
+            w.sort_scr = m.take<char>(sort_scratch_bytes(nmax) + scan_scratch_bytes(nmax + n_obj + 1));
+        }
         if (curv) {
             w.canon = m.take<int32_t>(nv);
             w.cnt = m.take<uint32_t>(std::max<int64_t>(nv, n_obj) + 1);
