@@ -77,6 +77,7 @@ struct st_ctx {
     int64_t N = 0;
     DevBuf dirs, etab, perm, ord_keys, ord_scr;
     DevBuf th_keys, th_scr;          // emitter-table row order of the specular path list
+    DevBuf vs_keys, vs_scr;          // hit-point Morton order of the visibility queries
     int32_t n_theta = 0;
     float fov_half = 4.0f;
     // receivers
@@ -294,6 +295,11 @@ cudaMemcpyKind kind_out(int32_t mem) { return mem == ST_MEM_DEVICE ? cudaMemcpyD
 // of a million paths or more takes them all: it is accumulated on its own)
 constexpr int kBatchChunkDiv = 8;
 
+// Rays from which the visibility queries of a two-level scene are sorted by hit point: all go to one point, and neighbours in
+// that order enter the same instances.  1M rays x 3 among 8,000 plants 21.6 -> 19.9 ms, x 5 among 1,000 15.6 -> 14.8;
+// 300k rays 13.3 -> 12.7 and 5.78 -> 5.80; 100k 6.1 -> 6.3 and 2.9 -> 3.2.  (Flat scenes: 3.21 -> 3.28 ms at 300k rays.)
+constexpr int64_t kVisSortRays = 512 * 1024;
+
 // traversal counters: 64 bytes of the diffraction stage's, then the trace's queue lengths and claim counters by bounce
 constexpr size_t kTravCounts = 64 + (kMaxBounces + 1) * 16;
 
@@ -385,7 +391,7 @@ st_status st_destroy(st_ctx* c) {
     cudaStreamSynchronize(c->stream);
     if (c->side) cudaStreamSynchronize(c->side);
     for (DevBuf* b : {&c->mic_q, &c->mic_tab, &c->tables.bw}) release(*b);
-    for (DevBuf* b : {&c->dirs, &c->etab, &c->perm, &c->ord_keys, &c->ord_scr, &c->th_keys, &c->th_scr, &c->mics, &c->st_o[0], &c->st_o[1], &c->st_o[2], &c->st_d[0], &c->st_d[1],
+    for (DevBuf* b : {&c->dirs, &c->etab, &c->perm, &c->ord_keys, &c->ord_scr, &c->th_keys, &c->th_scr, &c->vs_keys, &c->vs_scr, &c->mics, &c->st_o[0], &c->st_o[1], &c->st_o[2], &c->st_d[0], &c->st_d[1],
                       &c->st_d[2], &c->st_r, &c->st_prev, &c->q0, &c->q1, &c->counts, &c->queries, &c->flags, &c->R, &c->rec_tri,
                       &c->rec_p, &c->rec_d, &c->rec_r, &c->rec_los, &c->sidx, &c->scratch,
                       &c->cand_tri, &c->cand_p, &c->keep, &c->dvis, &c->partial, &c->host_out, &c->mat_off, &c->mat_scr, &c->tables.lk,
@@ -922,6 +928,11 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
     CKC(c, grow(c->rec_los, (size_t)std::max<int64_t>(NB, 1) + 3), "alloc");  // (whole words are cleared)
     CKC(c, grow(c->sidx, (size_t)std::max<int64_t>(NB, 1) * 4), "alloc");
     CKC(c, grow(c->scratch, compact_scratch_bytes(NB)), "alloc");
+    const bool vsort = S.two_level && N >= kVisSortRays && !per_mic;
+    if (vsort) {
+        CKC(c, grow(c->vs_keys, (size_t)N * 4), "alloc");
+        CKC(c, grow(c->vs_scr, sort_scratch_bytes(N)), "alloc");
+    }
     if (K > 1) {  // the line-of-sight queue of the diffraction candidates is sorted by Morton code
         CKC(c, grow(c->los_keys, (size_t)K * 8), "alloc");
         CKC(c, grow(c->los_scr, sort_scratch_bytes(K)), "alloc");
@@ -1083,6 +1094,13 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
             ta.rec_mask = per_mic ? ptr<uint64_t>(c->rec_mask) : nullptr;
             ta.mics = ptr<float>(c->mics);
             ta.M = M;
+            ta.sort_keys = vsort ? ptr<uint32_t>(c->vs_keys) : nullptr;
+            ta.sort_scr = vsort ? c->vs_scr.p : nullptr;
+            for (int k = 0; k < 3; ++k) {
+                const float ext = S.bounds_hi[k] - S.bounds_lo[k];
+                ta.blo[k] = S.bounds_lo[k];
+                ta.bscale[k] = ext > 0.0f ? 1024.0f / ext : 0.0f;
+            }
             CKC(c, trace_rays(ta, s, c->tune.rays_per_block > 0 ? c->tune.rays_per_block : 128), "trace");
         }
         return ST_OK;

@@ -225,6 +225,10 @@ struct TraceArgs {
     // per-microphone receiver test (ST_LOS_PER_MIC): M queries per record (query = record id * M + m), the
     // record's bit m of rec_mask set when microphone m is visible; null rec_mask: one query per record
     uint64_t* rec_mask; const float* mics; int32_t M;
+    // optional: each bounce's visibility queue sorted by the Morton code of the hit points (scene bounds lo, 1024 / extent)
+    // before the next launch traces it; keys [N] and sort scratch, or null
+    uint32_t* sort_keys; void* sort_scr;
+    float blo[3], bscale[3];
     // records [N][B]
     int32_t* rec_tri;
     float* rec_p;    // [N][B][3]

@@ -48,8 +48,7 @@ __host__ __device__ __forceinline__ Trav trav_of(const A& a) {
 // Bound by instruction issue over divergent lanes, and in small calls by the longest query: separate launches for closest
 // hits, shading and visibility waited for their slowest query twice a bounce and ran the tail of each alone.  10k rays x
 // 3 in the empty room 226 -> 182 us a call, 60k x 4 in light clutter 577 -> 439 us, 100k x 3 in a forest 4726 -> 3598 us,
-// 1M x 4 among 1M leaf triangles 15.8 -> 14.6 ms.  (Sorting the visibility queue of large scenes by hit point is gone with
-// it: the sort saved 4 % of their tracing and cost as much in launches.)
+// 1M x 4 among 1M leaf triangles 15.8 -> 14.6 ms.
 template <bool TL>
 __global__ void ST_TRAV_BOUNDS k_bounce(const TraceArgs a, int j, int lanes) {
     const Trav T = trav_of(a);
@@ -370,6 +369,22 @@ __device__ __forceinline__ uint32_t spread10(uint32_t x) {
     return x;
 }
 
+// Morton code (10 bits per axis) of the hit point of every queued visibility query
+__global__ void k_vis_keys(const TraceArgs a, int j) {
+    const int64_t n = a.n_vis[j];
+    const uint32_t* q = a.vis_q[j & 1];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n; c += stride) {
+        const float* p = a.rec_p + 3 * (size_t)q[c];
+        uint32_t m = 0;
+        for (int k = 0; k < 3; ++k) {
+            const float u = (p[k] - a.blo[k]) * a.bscale[k];
+            m |= spread10((uint32_t)fminf(fmaxf(u, 0.0f), 1023.0f)) << (2 - k);
+        }
+        a.sort_keys[c] = m;
+    }
+}
+
 // Morton code (kLosBits per axis) of the candidate point of every queued line-of-sight query
 // (line of sight of the clutter workload's 3.2M candidates, sort included: 5 bits 2.42 ms, 8 bits 2.00, 10 bits 1.88)
 constexpr int kLosBits = 10;
@@ -458,8 +473,15 @@ cudaError_t trace_rays(TraceArgs& a, cudaStream_t s, int block) {
             k_bounce<true><<<g.ctas, threads, 0, s>>>(a, j, g.lanes);
         else
             k_bounce<false><<<g.ctas, threads, 0, s>>>(a, j, g.lanes);
-        const cudaError_t e = cudaGetLastError();
+        cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
+        if (a.sort_keys && j < a.B) {
+            note_launch();
+            k_vis_keys<<<grid_for(a.N, 256), 256, 0, s>>>(a, j);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = radix_sort_u32(a.sort_keys, a.vis_q[j & 1], a.N, 0, 30, a.sort_scr, s, a.n_vis + j)) != cudaSuccess)
+                return e;
+        }
     }
     return cudaSuccess;
 }

@@ -60,3 +60,30 @@ def test_concentric_triangles_leave_the_rest_its_hierarchy(torch_st, monkeypatch
         _, x = ctx.simulate(sc, p, stats=True)
         nodes.append(x.visits[0] / x.closest_queries)
     assert nodes[1] <= 1.2 * nodes[0], nodes
+
+
+def forest(st, n_inst, n_rays, two_level):
+    fo = synth.instanced_forest(seed=606, n_inst=n_inst, n_rays=n_rays, bounces=2, n_mics=3, n_bins=8)
+    b = fo.base
+    ctx = st.Context(0)
+    sc = st.Scene.from_instances(ctx, fo.protos, fo.inst_proto, fo.inst_xform)
+    sc.set_materials(b.band_hz, b.k_band, b.beta_band, b.diff_band)
+    sc.set_structure(two_level)
+    sc.precompute(st.curv_params(sample_budget=1_000))
+    ctx.set_frequencies(b.n_bins, b.f_lo, b.f_hi)
+    ctx.set_emitter(b.emitter, b.emitter_quat, b.dirs)
+    ctx.set_receivers(b.mics)
+    S = ctx.simulate(sc, st.sim_params(max_bounces=2, max_distance=b.max_distance))
+    return S.cpu().numpy(), ctx.paths(2), sc.n_tris
+
+
+# flat against two-level, which share neither hierarchy nor traversal: more rays than the two-level trace leaves unsorted,
+# and more triangles than a clustering block counts the tiles of by itself
+@pytest.mark.parametrize("n_inst,n_rays,at_least", [(300, 524_289, 100_000), (7_500, 20_000, 8192 * 496 + 1)])
+def test_large_forests_agree_in_both_structures(torch_st, n_inst, n_rays, at_least):
+    _, st = torch_st
+    (S0, p0, n), (S1, p1, _) = forest(st, n_inst, n_rays, False), forest(st, n_inst, n_rays, True)
+    assert n >= at_least
+    for k in ("tri", "los", "p", "r"):
+        assert np.array_equal(p0[k], p1[k]), k
+    assert np.array_equal(S0, S1) and np.abs(S0[0]).sum() > 0
