@@ -648,10 +648,10 @@ __global__ void k_gather_diff_batch(const BatchArgs a, const uint32_t* idx, cons
 
 }  // namespace
 
-int32_t accum_chunks(const AccumArgs& a, int64_t n_paths_hint) {
+int32_t accum_chunks(const AccumArgs& a, int64_t n_paths_hint, bool queued) {
     const int32_t M = a.M, F = a.F, n_mat = a.n_mat_tab, dir_nb = a.mic_tab ? a.n_bands_tab : 0;
     if (narrow_accum(M)) return narrow_chunks(n_paths_hint, M, F, n_mat, dir_nb);
-    if (!a.mic_tab && few_accum(M, F)) return few_chunks(a, n_paths_hint);
+    if (!queued && !a.mic_tab && few_accum(M, F)) return few_chunks(a, n_paths_hint);
     read_tile_env();
     const int tp = a.tile_tp > 0 ? a.tile_tp : g_tile_tp;
     const size_t budget = a.tile_kb > 0 ? (size_t)a.tile_kb * 1024 : g_tile_budget;

@@ -1917,12 +1917,16 @@ void batch_release(BatchState& B) {
 }
 
 // Jobs accumulated one after the other by the single-pose path's launch (not through the work queue): one
-// microphone pair (the narrow accumulator is several times faster for them), receiver directivity tables
+// microphone pair (the narrow accumulator is several times faster for them), few bins, receiver directivity tables
 // (the tile's per-microphone band tables), and jobs of a million paths or more, which fill the GPU alone
 // with their full chunk count (in the queue they would take a fraction of it).
+// Where the queue is the better one for few bins: six microphones or more with half to all of the 512 bins that its tile
+// holds (64 poses of 10k rays x 3, on their own / in the queue, ms: 6 x 500 5.12 / 4.60, 8 x 400 5.01 / 4.61, 6 x 350 4.64 /
+// 4.53, 10 x 340 5.05 / 5.05; but 4 x 400 4.26 / 4.14 beside 4 x 800 5.34 / 5.94, 10 x 150 4.43 / 4.97, 3 x 128 3.64 / 4.04).
+static bool few_alone(int32_t M, int32_t F) { return few_accum(M, F) && !(M >= 6 && F > 256 && F <= 512); }
 static bool big_job(const JobDev& d) { return d.N * (int64_t)d.B >= (1 << 20) || d.K >= (1 << 20); }
 static bool solo_accum(const JobDev& d) {
-    return narrow_accum(d.M) || few_accum(d.M, d.F) || d.mic_tab != nullptr || big_job(d);
+    return narrow_accum(d.M) || few_alone(d.M, d.F) || d.mic_tab != nullptr || big_job(d);
 }
 
 // All stages of one batch on stream s.
@@ -2478,14 +2482,15 @@ static st_status simulate_batch_impl(st_ctx* c, int32_t n_jobs, const st_job* jo
         probe.mic_tab = d.mic_tab;
         probe.tile_tp = tn.mic_pairs_per_cta;
         probe.tile_kb = tn.smem_kb;
-        const int32_t chunks_spec = accum_chunks(probe, d.N * d.B);
+        const bool queued = !solo_accum(d);
+        const int32_t chunks_spec = accum_chunks(probe, d.N * d.B, queued);
         probe.kind = 1;
         d.diff_mma = d.K > 0 && diffraction_mma_applies(probe) ? 1 : 0;
         B.any_mma = B.any_mma || d.diff_mma;
         B.any_table_order = B.any_table_order || (d.etab != nullptr && d.K > 0 && !d.diff_mma);
         B.chunks_spec[j] = std::max(1, chunks_spec / nb);
         B.chunks_diff[j] =
-            std::max(1, (d.diff_mma ? diffraction_mma_chunks(d.K, d.M, d.F, S.n_mat) : accum_chunks(probe, d.K)) / nb);
+            std::max(1, (d.diff_mma ? diffraction_mma_chunks(d.K, d.M, d.F, S.n_mat) : accum_chunks(probe, d.K, queued)) / nb);
         if (solo_accum(d))
             narrow_part = std::max(narrow_part, (size_t)std::max(B.chunks_spec[j], B.chunks_diff[j]) * d.M * d.F * 8);
     }

@@ -379,8 +379,9 @@ cudaError_t build_accum_tables(AccumTables& T, const SceneDev& S, int32_t F, dou
                                double a0, double a1, cudaStream_t s);
 cudaError_t accumulate(const AccumArgs& a, cudaStream_t s);
 cudaError_t reduce_partials(const float2* partial, int32_t n_chunks, int64_t MF, float2* out, cudaStream_t s);
-// chunks for an accumulation of at most n_paths paths; a: kind, sizes, directivity and tile set
-int32_t accum_chunks(const AccumArgs& a, int64_t n_paths);
+// chunks for an accumulation of at most n_paths paths; a: kind, sizes, directivity and tile set; queued: by the general
+// accumulator's work queue, whatever the sizes
+int32_t accum_chunks(const AccumArgs& a, int64_t n_paths, bool queued = false);
 // Few frequency bins, omni receivers, three microphones or more (st_accum_few.cu).  Where the line lies: the general
 // accumulator shares a path's factors and anchors between 16 pairs and 16 subtiles and wins when it has that many
 // (specular accumulation of 104k paths, few-bin kernel / general, ms: 32 x 48 0.15 / 0.25, 32 x 96 0.22 / 0.24, 32 x 120
