@@ -915,7 +915,8 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
     CKC(c, grow(c->R, 16), "alloc");
     const bool per_mic = p.los_mode == ST_LOS_PER_MIC;
     const size_t n_visq = (size_t)std::max<int64_t>(N, 1) * (per_mic ? (size_t)M : 1);
-    CKC(c, grow(c->vis_q, 2 * n_visq * 4), "alloc");
+    const size_t visqs = B > 1 ? 2 : 1;  // a launch reads the last bounce's queue and fills its own
+    CKC(c, grow(c->vis_q, visqs * n_visq * 4), "alloc");
     if (per_mic) {
         CKC(c, grow(c->rec_mask, (size_t)std::max<int64_t>(NB, 1) * 8), "alloc");
         CKC(c, grow(c->paths.mask, (size_t)std::max<int64_t>(NB, 1) * 8), "alloc");
@@ -1086,7 +1087,7 @@ static st_status simulate_impl(st_ctx* c, st_scene* sc, const st_sim_params* par
             ta.flags = ptr<uint32_t>(c->flags);
             ta.queries = qctr;
             ta.vis_q[0] = ptr<uint32_t>(c->vis_q);
-            ta.vis_q[1] = ta.vis_q[0] + n_visq;
+            ta.vis_q[1] = ta.vis_q[0] + (visqs - 1) * n_visq;
             char* tc = ptr<char>(c->trav_cnt) + 64;
             ta.ctr = reinterpret_cast<unsigned long long*>(tc);
             ta.n_live = reinterpret_cast<uint32_t*>(tc + (kMaxBounces + 1) * 8);
@@ -2569,7 +2570,7 @@ st_status st_autotune(st_ctx* c, const st_job* J, const st_sim_params* params, s
     const st_tune saved = c->tune;
     const bool saved_overlap = c->overlap;
     c->overlap = false;  // each stage timed on its own
-    const int rpb[3] = {64, 128, 256};
+    const int rpb[2] = {64, 128};  // (256 traces in blocks of 128)
     const int tiles[5][2] = {{16, 108}, {8, 108}, {16, 64}, {4, 108}, {16, 128}};
     const int kts[2] = {16, 8};
     const int depths[3] = {0, 48, 24};
@@ -2579,7 +2580,7 @@ st_status st_autotune(st_ctx* c, const st_job* J, const st_sim_params* params, s
     // tile (microphone pairs and shared memory), its bins per thread (frequency tile), the traversal stack depth
     // and the lane-refill threshold (rays per warp refill); tracing phases are timed on tracing and diffraction,
     // the others on the accumulator kernels
-    const int n_phase[5] = {3, 5, 2, 3, 4};
+    const int n_phase[5] = {2, 5, 2, 3, 4};
     for (int phase = 0; phase < 5; ++phase) {
         const int n_cand = n_phase[phase];
         st_tune winner = best;

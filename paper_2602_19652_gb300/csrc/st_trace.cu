@@ -198,17 +198,16 @@ __global__ void ST_TRAV_BOUNDS k_bounce(const TraceArgs a, int j, int lanes) {
 
 // Visibility of `target` from the points of a queue (record or candidate ids): out[id] = 1 when no
 // triangle other than excl[id] lies on the segment (t_min, |target - p| - eps).
-// The target is tgt_dev[0..2] when given (the receiver reference point, written on the device), else (tx, ty, tz).
 template <bool TL>
 __global__ void ST_TRAV_BOUNDS k_visible(const Trav T, const uint32_t* queue, const uint32_t* count,
                                                            const float* pts, const int32_t* excl,
-                                                           const float* tgt_dev, float tx, float ty, float tz,
-                                                           float t_min, float eps, uint8_t* out,
+                                                           float tx, float ty, float tz, float t_min, float eps,
+                                                           uint8_t* out,
                                                            unsigned long long* ctr, uint32_t* flags,
                                                            unsigned long long* queries, int lanes) {
     const int64_t n = *count;
     const unsigned full = 0xffffffffu;
-    const f3 target = tgt_dev ? f3{tgt_dev[0], tgt_dev[1], tgt_dev[2]} : f3{tx, ty, tz};
+    const f3 target{tx, ty, tz};
     int2 stack[kStack];
     typename TravStateOf<TL>::type S;
     int64_t id = -1;
@@ -506,7 +505,7 @@ cudaError_t diffraction_sample(DiffArgs& a, cudaStream_t s) {
     note_launch();
     const TravGrid g = trav_grid(a.K, tl);
     (tl ? k_visible<true> : k_visible<false>)<<<g.ctas, kTravBlock, 0, s>>>(
-        T, a.los_q, a.los_n, a.cand_p, a.cand_tri, nullptr, a.s[0], a.s[1], a.s[2], a.t_min, a.los_eps, a.keep, a.ctr,
+        T, a.los_q, a.los_n, a.cand_p, a.cand_tri, a.s[0], a.s[1], a.s[2], a.t_min, a.los_eps, a.keep, a.ctr,
         a.flags, a.queries, g.lanes);
     return cudaGetLastError();
 }

@@ -87,3 +87,24 @@ def test_large_forests_agree_in_both_structures(torch_st, n_inst, n_rays, at_lea
     for k in ("tri", "los", "p", "r"):
         assert np.array_equal(p0[k], p1[k]), k
     assert np.array_equal(S0, S1) and np.abs(S0[0]).sum() > 0
+
+
+def test_refits_of_several_scenes_share_scratch(torch_st):
+    """Scenes of different sizes in one context, moved in turn with their curvature kept: each as if it were alone."""
+    _, st = torch_st
+    rng = np.random.default_rng(4)
+    parts = st.ST_COMP_SPECULAR
+    wls = [workload(scattered(n), 3_000) for n in (900, 20_000, 5)]
+    ctx = st.Context(0)
+    scenes = [st.from_workload(ctx, wl, st.curv_params(sample_budget=1_000)) for wl in wls]
+    p = st.sim_params(max_bounces=2, max_distance=60.0, components=parts)
+    for _ in range(2):
+        for wl, sc in zip(wls, scenes):
+            wl.verts = (wl.verts + rng.uniform(-0.2, 0.2, 3)).astype(np.float32)
+            sc.update_vertices(wl.verts, keep_curvature=True)
+    for wl, sc in zip(wls, scenes):
+        S = ctx.simulate(sc, p).cpu().numpy()
+        tri = ctx.paths(2)["tri"]
+        alone = st.Context(0)
+        ref = alone.simulate(st.from_workload(alone, wl, st.curv_params(sample_budget=1_000)), p).cpu().numpy()
+        assert np.array_equal(tri, alone.paths(2)["tri"]) and np.array_equal(S, ref)
