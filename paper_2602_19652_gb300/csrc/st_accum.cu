@@ -658,8 +658,11 @@ int32_t accum_chunks(const AccumArgs& a, int64_t n_paths_hint, bool queued) {
     const Geom g =
         make_geom(M, F, dir_nb ? 16 : (a.tile_kt > 0 ? a.tile_kt : g_tile_kt), n_mat, tp, budget, dir_nb, 0, 1);
     const int ctas_per_chunk = g.n_mb * g.n_bb;
-    const int threads = g.TP * g.NS;
-    int resident = std::max(1, std::min(2048 / std::max(threads, 32), (int)((220 * 1024) / std::max<size_t>(g.smem, 1))));
+    // CTAs an SM holds at once, by shared memory and registers (128 a thread, 255 with receiver tables: 48 x 97, two and not
+    // three, 0.43 -> 0.36 ms); the work queue's CTAs do not depend on the job's tile, and its chunks go by threads
+    const int threads = g.TP * g.NS, warps = (threads + 31) / 32;
+    const int by_threads = queued ? 2048 / std::max(threads, 32) : (dir_nb ? 8 : 16) / warps;
+    int resident = std::max(1, std::min(by_threads, (int)((220 * 1024) / std::max<size_t>(g.smem, 1))));
     int64_t want = (int64_t)152 * resident / std::max(ctas_per_chunk, 1);
     int64_t tiles = (n_paths_hint + g.PT - 1) / g.PT;
     want = std::min<int64_t>(want, std::max<int64_t>(tiles, 1));

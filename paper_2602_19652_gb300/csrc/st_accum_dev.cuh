@@ -629,11 +629,16 @@ inline Geom make_geom(int M, int F, int KT, int n_mat, int tp_max = 8, size_t bu
     g.NS = std::max(1, std::min(ns_need, 256 / g.TP));
     if (balance && g.NS > 2 && g.NS * KT <= 400) {
         // bins spread evenly over their blocks (104k paths: 32 microphones x 257 bins, whose second block held one bin,
-        // 0.75 -> 0.63 ms; 24 x 512 1.06 -> 0.65), in subtiles a multiple of four.  Blocks of more than 400 bins (18
+        // 0.75 -> 0.63 ms; 24 x 512 1.06 -> 0.65).  Blocks of more than 400 bins (18
         // microphones and fewer) stay, and with them the places where a phasor starts anew: its rounding grows over a
         // block, to 1.5e-5 of a spectrum at 512 bins, and other blocks would differ by as much.
-        const int blocks = (ns_need + g.NS - 1) / g.NS, ns = (ns_need + blocks - 1) / blocks, ns4 = (ns + 3) & ~3;
-        g.NS = ns4 * g.TP <= 256 ? ns4 : ns;
+        const int blocks = (ns_need + g.NS - 1) / g.NS;
+        g.NS = (ns_need + blocks - 1) / blocks;
+        // A tile's eight paths take a thread each per pair for their anchors: with seven subtiles the producer makes a second
+        // round for one path (200k rays x 3, 12 microphones x 97 bins, seven / eight: 0.186 / 0.154 ms, 48 x 97 0.36 / 0.32).
+        // Not where it takes another microphone block (200 x 97, three blocks / four: 1.30 / 1.53); and otherwise a subtile
+        // past the last bin only costs (100 x 129, nine / twelve: 0.79 / 1.14).
+        if (g.NS == 7 && (pairs + 256 / 8 - 1) / (256 / 8) == (pairs + 256 / 7 - 1) / (256 / 7)) g.NS = 8;
     }
     g.TP = std::max(1, std::min(pairs, 256 / g.NS));
     if (balance) {
