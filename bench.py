@@ -704,7 +704,7 @@ def measure_traversal(st, torch, wl, ms_trace: float, ms_diffraction: float, hbm
     ft, fd = bt / (ms_trace / 1e3) / 1e9, bd / (ms_diffraction / 1e3) / 1e9
     return {"bytes_per_node": 112, "bytes_per_triangle": 48, "l2_probe_gbs": l2,
             "frac_of_l2_probe": {"bounces": ft / l2, "diffraction": fd / l2},
-            "bounces": {"kernels": "k_closest + k_shade + k_visible (records), all bounces",
+            "bounces": {"kernels": "k_bounce (closest hits, shading, visibility of the bounce before), all launches",
                         "queries": int(q_t), "nodes": int(vs[0] + vs[2]), "triangles": int(vs[1] + vs[3]),
                         "nodes_per_query": (vs[0] + vs[2]) / max(q_t, 1), "ms": ms_trace,
                         "fetch_gbs": ft},
@@ -797,6 +797,8 @@ def run_case(st, torch, case: str, reps: int):
         wl = synth.clutter(seed=202, n_rays=200_000)
     elif case == "narrow":
         wl = synth.vegetation(seed=303, n_rays=500_000)
+    elif case == "few":
+        wl = synth.clutter(seed=202, n_rays=200_000, bounces=3, n_mics=64, n_bins=14)
     else:
         raise SystemExit(f"unknown case {case}")
     ctx = st.Context(dev)
@@ -920,7 +922,7 @@ def main():
     ap.add_argument("--no-emitters", action="store_true", help="skip the several-emitters timing")
     ap.add_argument("--no-instances", action="store_true", help="skip the instanced-forest timing")
     ap.add_argument("--case", default=None,
-                    choices=["accum", "adjoint", "trace", "trace_per_mic", "narrow", "emitters", "instances", "batched_bat",
+                    choices=["accum", "adjoint", "trace", "trace_per_mic", "narrow", "few", "emitters", "instances", "batched_bat",
                              "batched", "batched_bat_only", "batched_only"],
                     help="run a small case of one kernel family a few times and exit (for profiler captures)")
     args = ap.parse_args()
