@@ -16,8 +16,9 @@
 // Diffraction paths without an emitter table skip 1a: their factor depends on the material and the bin
 // only, and the term loop reads it from the CTA's material table at the row the producer names.
 // With the per-microphone receiver test a microphone that does not see the path gets a zero anchor.
-// The phase never loses precision: only frac(f r / c) enters FP32, and the recurrence runs at most
-// KT steps from an exactly reduced anchor.
+// Only frac(f r / c) enters FP32, reduced exactly at the CTA's first bin; from there a chain of steps W^KT reaches every
+// subtile's first bin and one of W, W^2 the bins within, so the rounding grows over a CTA's block of bins, at most 512: to
+// 1.5e-5 of a spectrum.
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -810,8 +811,8 @@ cudaError_t compact_indices(const uint32_t* flags, const uint32_t* scan, int64_t
     return cudaGetLastError();
 }
 
-// Emitter-table row of every compacted specular path (the floor of its angle coordinate), 0xffff past the
-// count: sorting the compacted list by it lets the paths of an accumulator tile share table rows.
+// Emitter-table row of every compacted specular path (the floor of its angle coordinate): sorting the compacted
+// list by it lets the paths of an accumulator tile share table rows.
 __global__ void k_theta_keys(const GatherArgs g, uint32_t* keys) {
     const int64_t n = *g.count;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;

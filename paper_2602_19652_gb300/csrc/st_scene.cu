@@ -514,6 +514,9 @@ __global__ void k_morton(const float* V, const int32_t* T, int64_t nt, const uin
             c = c * (1.0f / 3.0f);
             float u = ext[k] > 0.0f ? (c - lo[k]) / ext[k] : 0.5f;
             u = fminf(fmaxf(u, 0.0f), 1.0f);
+            // 16 bits an axis: cells as fine as the boxes' padding, 1e-5 of the scene's diagonal, below which no hierarchy
+            // tells triangles apart.  (21 bits took two more passes and 3 % of a build, and among 160k triangles of 2-10 cm
+            // objects in scenes of 10 to 3,000 m traversal was between 0.92 and 1.05 of this.)
             uint32_t qi = (uint32_t)(u * 65535.0f);
             q[k] = qi;
         }

@@ -6,8 +6,8 @@
 // twice a tile: equal keys keep their input order.  The number of keys may be on the device (tiles past it do nothing).
 // Bound by launches and latency for short arrays, by the scattered writes for long ones.  Against the form before (a
 // histogram scanned over three launches, a scatter of 16 rounds with three block barriers each, always 64-bit keys and an
-// even number of passes over the array's capacity): mesh pre-processing of 200k triangles 3290 -> 2615 us, a frame of 80k
-// rays and 500k candidates 961 -> 826 us, a training step in the room 1120 -> 991 us.
+// even number of passes over the array's capacity): mesh pre-processing of 200k triangles 3250 -> 2640 us, a frame of 80k
+// rays and 500k candidates 970 -> 767 us, a training step in the room 1110 -> 957 us.
 #include <algorithm>
 #include <utility>
 

@@ -12,8 +12,9 @@
 // microphone), and shades its hits itself (reflection, float64 path length, the record [ray][bounce], the next live
 // queue and the next launch's visibility queue).  The kernel is persistent with lane refill: a query advances one wide
 // node or one leaf triangle per step, and a lane whose query has finished takes the next one from a warp-aggregated
-// atomic counter while the other lanes of its warp continue.  Results do not depend on the order: closest hits are the
-// smallest (t, triangle index), visibility is the absence of any hit in the segment.
+// atomic counter while the other lanes of its warp continue.  Between the launches of a large call in a two-level scene the
+// visibility queue is sorted by hit point.  Results do not depend on the order: closest hits are the smallest (t, triangle
+// index), visibility is the absence of any hit in the segment.
 // Compiled with -fmad=false (see st_geom.cuh).
 #include <algorithm>
 
