@@ -93,7 +93,7 @@ __global__ void k_tables(int32_t F, int32_t n_mat, int32_t n_bands, const float*
 // One CTA of the accumulation: microphone block bx % n_mb, bin block bx / n_mb, chunk by of the path list.
 // Threads past TP * NS (a block larger than the tile, as in the persistent batched launch) take part in
 // the loads, the producer and the barriers only.
-template <int KT, int KIND, int DIR, int SPLIT = 0>
+template <int KT, int KIND, int DIR, int SPLIT, bool ROWS>
 __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int bx, int by, float4* smem4) {
     static_assert((KT & (KT - 1)) == 0 && KT >= 2, "KT must be a power of two");
     constexpr int RL = row_pairs(KT), RX = row_floats(KT);
@@ -129,7 +129,7 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
         }
     }
     if (t0 < t1) {
-        if (g.mat_cached) {
+        if (ROWS) {
             const int nm = a.n_mat_tab;
             for (int e = tid; e < nm * KB; e += nthr) {
                 const int mat = e / KB, i = e - mat * KB;
@@ -148,7 +148,7 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
         load_paths<KIND>(a, PT, t0 * PT, count, pdb, pvb);
         if (t0 + 1 < t1) load_paths<KIND>(a, PT, (t0 + 1) * PT, count, pdb + PT * 12, pvb + PT);
         __syncthreads();
-        produce<KT, KIND, 0, SPLIT>(a, g, B0, pdb, pvb, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, nullptr, pb0 + t0 * PT);
+        produce<KT, KIND, 0, SPLIT, ROWS>(a, g, B0, pdb, pvb, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, nullptr, pb0 + t0 * PT);
         __syncthreads();
     }
     // software pipeline: consume tile t from buffer b while producing tile t+1 into buffer b^1
@@ -161,7 +161,7 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
         if (tile + 2 < t1) load_paths_cp<KIND>(a, PT, (tile + 2) * PT, count, pdb + b * PT * 12, pvb + b * PT);
         if (tile + 1 < t1) {
             const int nb = b ^ 1;  // path data of tile+1 sits in pd buffer nb
-            produce<KT, KIND, 0, SPLIT>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, nullptr,
+            produce<KT, KIND, 0, SPLIT, ROWS>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, nullptr,
                               pb0 + (tile + 1) * PT);
         }
         const ulonglong2* zp = C.za + s * TP + tp;
@@ -178,7 +178,8 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
             u64 orr = er, oi = ei;     // odd chain: bins 1, 3, 5, ...
             cmul2(orr, oi, w1r, w1i, fmul2(w1i, pk2(-1.0f, -1.0f)));
             const float2* xrow = reinterpret_cast<const float2*>(xp);  // two bins each
-            const float2* grow = reinterpret_cast<const float2*>(gb + (KIND == 0 ? C.goff[p] : 0));
+            const float2* grow = reinterpret_cast<const float2*>(gb + (KIND == 0 && ROWS ? C.goff[p] : 0));
+            const float2* trow = reinterpret_cast<const float2*>(C.tab) + p * KB + s;  // (not ROWS)
             const float2 ngv = up2(ng);  // -gamma^2 of the two microphones
             // diffraction with the material table read directly: the producer left the offset of the path's
             // material row in the (otherwise unused) lobe slot
@@ -188,7 +189,10 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
             u64 E2[2];  // factors of bins kk and kk + 1
 #pragma unroll
             for (int kk = 0; kk < KT; ++kk) {
-                if ((kk & 1) == 0) {
+                if (!ROWS) {
+                    const float2 t = trow[kk * NS];
+                    E2[kk & 1] = KIND == 0 ? pk2(ex2(fmaf(ngv.x, t.y, t.x)), ex2(fmaf(ngv.y, t.y, t.x))) : pk2(t.x, t.y);
+                } else if ((kk & 1) == 0) {
                     if (KIND == 1 && g.mat_direct) {
                         const ulonglong2 t = mrow[kk >> 1];
                         E2[0] = t.x;
@@ -247,18 +251,18 @@ __device__ __forceinline__ void accum_cta(const AccumArgs& a, const Geom& g, int
     }
 }
 
-template <int KT, int KIND, int DIR>
+template <int KT, int KIND, int DIR, bool ROWS>
 __global__ void __launch_bounds__(256, DIR ? 1 : 2) k_accum(const AccumArgs a, const Geom g) {
     extern __shared__ float4 smem4[];
-    accum_cta<KT, KIND, DIR>(a, g, blockIdx.x, blockIdx.y, smem4);
+    accum_cta<KT, KIND, DIR, 0, ROWS>(a, g, blockIdx.x, blockIdx.y, smem4);
 }
 
 // Persistent accumulation of a batch: each CTA takes work items -- one CTA's worth of one (job, path kind)
 // accumulation: its microphone block, bin block and chunk -- from a device counter until none is left, and
 // runs them with the single-pose CTA body.  Items are claimed in task order; no item waits for another.  One
-// launch per path kind (the tasks of that kind).  The table is declared unaliased: its fields are then read again where they
+// launch per path kind and table layout.  The task table is declared unaliased: its fields are then read again where they
 // are used instead of spilled (228 -> 164 bytes a thread; 20 poses 16.4 -> 16.0 ms).
-template <int KIND>
+template <int KIND, bool ROWS>
 __global__ void __launch_bounds__(256, 2) k_accum_queue(const AccumTask* __restrict__ tasks, int32_t n_tasks, int64_t n_items,
                                                         unsigned long long* counter) {
     extern __shared__ float4 smem4[];
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(256, 2) k_accum_queue(const AccumTask* __restr
         if (it >= n_items) break;
         const int nxy = T.g.n_mb * T.g.n_bb;
         const int local = (int)(it - T.item0);
-        accum_cta<16, KIND, 0, 1>(T.a, T.g, local % nxy, local / nxy, smem4);
+        accum_cta<16, KIND, 0, 1, ROWS>(T.a, T.g, local % nxy, local / nxy, smem4);
         __syncthreads();  // shared memory is reused by the next item
     }
 }
@@ -556,20 +560,25 @@ Geom accum_geom(const AccumArgs& a, int kind, int kt, int dir) {
     return make_geom(a.M, a.F, kt, a.n_mat_tab, tp, budget, dir ? a.n_bands_tab : 0, direct_mat, 1);
 }
 
-template <int KT, int KIND, int DIR>
-cudaError_t launch_accum(const AccumArgs& a, cudaStream_t s) {
-    const Geom g = accum_geom(a, KIND, KT, DIR);
+template <int KT, int KIND, int DIR, bool ROWS>
+cudaError_t launch_accum(const AccumArgs& a, const Geom& g, cudaStream_t s) {
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e =
-            cudaFuncSetAttribute(k_accum<KT, KIND, DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            cudaFuncSetAttribute(k_accum<KT, KIND, DIR, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     dim3 grid((unsigned)(g.n_mb * g.n_bb), (unsigned)a.n_chunks);
     note_launch();
-    k_accum<KT, KIND, DIR><<<grid, g.TP * g.NS, g.smem, s>>>(a, g);
+    k_accum<KT, KIND, DIR, ROWS><<<grid, g.TP * g.NS, g.smem, s>>>(a, g);
     return cudaGetLastError();
+}
+
+template <int KT, int KIND, int DIR>
+cudaError_t launch_accum(const AccumArgs& a, cudaStream_t s) {
+    const Geom g = accum_geom(a, KIND, KT, DIR);
+    return g.mat_cached ? launch_accum<KT, KIND, DIR, true>(a, g, s) : launch_accum<KT, KIND, DIR, false>(a, g, s);
 }
 
 // path list entries of every job (same layout as the single-pose gather; omni emitter)
@@ -743,24 +752,25 @@ cudaError_t accum_task(const AccumArgs& a, float2* out, AccumTask* t) {
     return cudaSuccess;
 }
 
-cudaError_t accumulate_queue(int kind, const AccumTask* tasks, int32_t n_tasks, int64_t n_items, size_t smem,
+cudaError_t accumulate_queue(int kind, bool rows, const AccumTask* tasks, int32_t n_tasks, int64_t n_items, size_t smem,
                              unsigned long long* counter, cudaStream_t s) {
-    static bool attr_set[2] = {false, false};
-    if (!attr_set[kind]) {
-        cudaError_t e = cudaFuncSetAttribute(kind == 0 ? k_accum_queue<0> : k_accum_queue<1>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    const auto kernel = kind == 0 ? (rows ? k_accum_queue<0, true> : k_accum_queue<0, false>)
+                                  : (rows ? k_accum_queue<1, true> : k_accum_queue<1, false>);
+    static bool attr_set[2][2] = {};
+    if (!attr_set[kind][rows]) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
-        attr_set[kind] = true;
+        attr_set[kind][rows] = true;
     }
+    if (n_tasks <= 0 || n_items <= 0) return cudaSuccess;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess || n_tasks <= 0 || n_items <= 0) return e;
+    if (e != cudaSuccess) return e;
     int dev = 0, n_sm = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int per_sm = smem > 110 * 1024 ? 1 : 2;
     const unsigned grid = (unsigned)std::min<int64_t>((int64_t)n_sm * per_sm, n_items);
     note_launch();
-    if (kind == 0) k_accum_queue<0><<<grid, 256, smem, s>>>(tasks, n_tasks, n_items, counter);
-    else k_accum_queue<1><<<grid, 256, smem, s>>>(tasks, n_tasks, n_items, counter);
+    kernel<<<grid, 256, smem, s>>>(tasks, n_tasks, n_items, counter);
     return cudaGetLastError();
 }
 

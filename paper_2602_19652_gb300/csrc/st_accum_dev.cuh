@@ -180,15 +180,16 @@ struct Geom {
 // own (6 packed FMA, 2 FMA and 2 ex2, loads).  With the bins transposed (entry kk * NS + s) every load had its address
 // computed, 16 in the term loop and 21.3 in all; with the lobe exponents read from the material table instead of copied
 // per path, two pipeline buffers of 8 paths fit two CTAs to an SM instead of 7, and the tables' half of the producer
-// shrinks: 19.7.  200k-ray clutter, 32 microphones x 512 bins: 1.145 -> 1.073 ms; 1M rays 5.60 -> 5.26; 24 x 257 with a
+// shrinks: 19.7.  Tables that shared memory does not hold stay transposed, (log2 X, g) side by side: their rows would take a
+// quarter more of it, and L1, which then serves the tables, gets less (see make_geom).  200k-ray clutter, 32 microphones x 512 bins: 1.145 -> 1.073 ms; 1M rays 5.60 -> 5.26; 24 x 257 with a
 // receiver test each 0.184 -> 0.164; the pose sweep's queue 16.1 -> 15.2 ms in all.  (Scalar instead of packed FMA costs
 // issue slots: 6.10; four bins per load in the term loop: 5.20, but the queue then spills and loses 5 %.)
 constexpr __host__ __device__ int row_floats(int KT) { return KT + 4; }
 constexpr __host__ __device__ int row_pairs(int KT) { return KT + 2; }
 
 // Shared memory: two pipeline buffers, each
-//   tab [PT][NS][row_floats] float  per (path, bin): log2 X specular, X diffraction
-//   gtab                         the same for the lobe exponent g, when the material tables are not cached (specular)
+//   tab [PT][NS][row_floats] float  per (path, bin): log2 X specular, X diffraction; or, when the material tables are not
+//                                cached, [PT][KB] float2: (log2 X, g) or (X, X), bin kb + s*KT + kk at kk*NS + s
 //   za  [PT][NS][TP] ulonglong2  phasor at bin kb + s*KT of the two mics of pair tp (re pair, im pair)
 //   wst [PT][2][TP] ulonglong2   one-bin step, two-bin step of the pair (re pair, im pair)
 //   ngp [PT][TP] u64         -gamma^2 of the pair (diffraction, mat_direct: the path's material row offset)
@@ -197,7 +198,6 @@ constexpr __host__ __device__ int row_pairs(int KT) { return KT + 2; }
 // then two path-data buffers pd [PT][12] + valid [PT], then the per-CTA material tables.
 struct Buf {
     float* tab;
-    float* gtab;
     ulonglong2* za;
     ulonglong2* wst;
     u64* ngp;
@@ -206,9 +206,9 @@ struct Buf {
     float* dband;  // [PT][MP][NB] receiver directivity band values (directional receivers only)
 };
 
-// bytes of one path in tab and gtab
+// bytes of one path in tab
 __host__ __device__ __forceinline__ size_t tab_bytes(const Geom& g) {
-    return g.mat_direct ? (size_t)0 : (size_t)g.RX * (g.mat_cached ? 4 : 8);
+    return g.mat_direct ? (size_t)0 : g.mat_cached ? (size_t)g.RX * 4 : (size_t)g.KB * 8;
 }
 
 template <int KT>
@@ -216,7 +216,6 @@ __device__ __forceinline__ Buf buf_at(float4* base, const Geom& g, int b) {
     Buf B;
     char* p = reinterpret_cast<char*>(base) + (size_t)b * g.buf_bytes;
     B.tab = reinterpret_cast<float*>(p);
-    B.gtab = B.tab + (size_t)g.PT * g.RX;
     B.za = reinterpret_cast<ulonglong2*>(p + tab_bytes(g) * g.PT);
     B.wst = B.za + (size_t)g.PT * g.NS * g.TP;
     B.ngp = reinterpret_cast<u64*>(B.wst + (size_t)g.PT * g.TP * 2);
@@ -461,13 +460,12 @@ __device__ __forceinline__ MicAnchor anchor_mic(const AccumArgs& a, const Geom& 
 }
 
 // tables and anchors of one tile (reads pd / pv, writes buffer B); ADJ: also the position-gradient
-// vectors of the adjoint (es = emitter position, diffraction only); SPLIT: see below
-template <int KT, int KIND, int ADJ = 0, int SPLIT = 0>
+// vectors of the adjoint (es = emitter position, diffraction only); SPLIT: see below; ROWS: g.mat_cached
+template <int KT, int KIND, int ADJ = 0, int SPLIT = 0, bool ROWS = true>
 __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const Buf& B, const float* pd, const int* pv,
                                         const float* mt, const float* base, int mic0, int kb, float invKB,
                                         const float* es = nullptr, int64_t pglob = 0) {
     const int PT = g.PT, NS = g.NS, TP = g.TP, KB = g.KB, MP = g.MP;
-    const bool cached = g.mat_cached > 0;
     const int tid = threadIdx.x, nthr = blockDim.x;
     // SPLIT (forward specular tiles of the batched work queue): the (path, pair) anchor items, each several
     // times a table entry's work, go to the first warps and the table entries of phase 1a to the others (when
@@ -480,15 +478,14 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
     // 1a: per (path, bin) factors (not needed when the term loop reads the material table directly).  With the material
     // tables in shared memory a thread builds four bins of a row: one chain decode, 128-bit loads and stores.
     constexpr int RX = row_floats(KT);
-    if (KIND == 0) {  // where the term loop finds the path's lobe exponents
+    if (KIND == 0 && ROWS) {  // where the term loop finds the path's lobe exponents
         for (int p = tid; p < PT; p += nthr) {
             const int matj = pv[p] ? (int)((__float_as_uint(pd[p * 12 + 8]) >> 8) & 255u) : 0;
-            const float* row = cached ? mt + a.n_mat_tab * KB + matj * g.RX : B.gtab + p * g.RX;
-            B.goff[p] = (int)(row - base);
+            B.goff[p] = (int)(mt + a.n_mat_tab * KB + matj * g.RX - base);
         }
     }
     if (KIND == 1 && g.mat_direct) {
-    } else if (cached && !a.etab) {
+    } else if (ROWS && !a.etab) {
         const int KB4 = KB >> 2;
         const float invKB4 = 4.0f * invKB;
         const bool last = kb + KB > a.F;  // bins beyond the grid contribute nothing
@@ -531,7 +528,8 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
     } else {
         for (int e = t_tab; e >= 0 && e < PT * KB; e += n_tab) {
             const int p = __float2int_rz(((float)e + 0.5f) * invKB), i = e - p * KB;
-            const int k = kb + i;
+            const int kk = ROWS ? 0 : __float2int_rz(((float)i + 0.5f) * (1.0f / (float)NS));
+            const int k = kb + (ROWS ? i : (i - kk * NS) * KT + kk);
             float lx = kNegInf, gg = 0.0f;
             if (pv[p] && k < a.F) {
                 const float* d = pd + p * 12;
@@ -539,20 +537,20 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                 const int matj = (meta >> 8) & 255;
                 if (KIND == 0) {
                     if (a.reflection_mode == 1) {
-                        lx = cached ? mt[matj * KB + i] : a.lk[(int64_t)matj * a.F + k];
+                        lx = ROWS ? mt[matj * KB + i] : a.lk[(int64_t)matj * a.F + k];
                     } else {
                         const int len = meta & 15;
                         const uint32_t c0 = __float_as_uint(d[9]), c1 = __float_as_uint(d[10]);
                         float acc = 0.0f;
                         for (int q = 0; q < len; ++q) {
                             const int mq = (q < 4 ? (c0 >> (8 * q)) : (c1 >> (8 * (q - 4)))) & 255;
-                            acc += cached ? mt[mq * KB + i] : a.lk[(int64_t)mq * a.F + k];
+                            acc += ROWS ? mt[mq * KB + i] : a.lk[(int64_t)mq * a.F + k];
                         }
                         lx = acc;
                     }
-                    if (!cached) gg = a.g2[(int64_t)matj * a.F + k];
+                    if (!ROWS) gg = a.g2[(int64_t)matj * a.F + k];
                 } else {
-                    lx = cached ? mt[matj * KB + i] : a.lid[(int64_t)matj * a.F + k];
+                    lx = ROWS ? mt[matj * KB + i] : a.lid[(int64_t)matj * a.F + k];
                 }
                 if (a.etab && d[11] >= 0.0f) {
                     const float x = d[11];
@@ -562,9 +560,9 @@ __device__ __forceinline__ void produce(const AccumArgs& a, const Geom& g, const
                     lx += de > 0.0f ? log2f(de) : kNegInf;
                 }
             }
-            const int at = (p * NS + i / KT) * RX + i % KT;
-            B.tab[at] = KIND == 0 ? lx : ex2(lx);
-            if (KIND == 0 && !cached) B.gtab[at] = gg;
+            if (KIND == 1) lx = ex2(lx);
+            if (ROWS) B.tab[(p * NS + i / KT) * RX + i % KT] = lx;
+            else reinterpret_cast<float2*>(B.tab)[p * KB + i] = make_float2(lx, KIND == 0 ? gg : lx);
         }
     }
     // 1b: per (path, mic) anchors and the phasors at the subtile starts.  Specular paths of the forward go by
@@ -652,8 +650,15 @@ inline Geom make_geom(int M, int F, int KT, int n_mat, int tp_max = 8, size_t bu
     g.n_mb = (M + g.MP - 1) / g.MP;
     g.n_bb = (F + g.KB - 1) / g.KB;
     const size_t mat_bytes = (size_t)2 * n_mat * g.KB * 4;  // two floats or one packed pair per (material, bin)
-    g.mat_cached = mat_bytes <= 24 * 1024 ? 1 : 0;
+    // Tables up to 48 KB (with a smaller budget less, with 24 KB as the least) are held in shared memory, in the adjoint up to
+    // 24: its paths need more room.  200k rays x 3: 3 microphones x 1500 bins of 4 materials (48 KB) 1.60 ms with the tables in
+    // L1, 0.94 so; 8 x 512 of 12 (48 KB) 0.84 / 0.38; but 32 x 512 of 32 (64 KB) 0.95 / 1.04.  Beyond it 6 x 2048 of 12
+    // materials takes 2.7 ms in this layout and took 3.2 in rows.
+    const size_t mat_most = balance ? std::max<size_t>(24 * 1024, std::min<size_t>(48 * 1024, budget * 9 / 20)) : 24 * 1024;
+    g.mat_cached = mat_bytes <= mat_most ? 1 : 0;
     g.mat_direct = (mat_direct && g.mat_cached) ? 1 : 0;
+    // (two CTAs to an SM with tables read from L2 through L1: 4 KB a CTA less leave L1 twice as large)
+    if (!g.mat_cached && budget <= 108 * 1024) budget = std::min<size_t>(budget, 104 * 1024);
     const size_t per_path =
         tab_bytes(g) + (size_t)g.NS * g.TP * 16 + (size_t)g.TP * 40 + 4 + (size_t)g.MP * dir_nb * 4;
     // fixed region: cached material tables (pairs; or log2 X in bin order and the lobe exponents in rows), then
@@ -684,7 +689,8 @@ struct AccumTask {
 cudaError_t accum_task(const AccumArgs& a, float2* out, AccumTask* t);
 // the persistent accumulation of the tasks of one path kind (device table, items numbered from 0); smem = the
 // largest tile's shared memory; counter: one device word, reset here
-cudaError_t accumulate_queue(int kind, const AccumTask* tasks, int32_t n_tasks, int64_t n_items, size_t smem,
+// (tasks of one path kind whose tiles hold the material tables, rows, or of one whose tiles do not)
+cudaError_t accumulate_queue(int kind, bool rows, const AccumTask* tasks, int32_t n_tasks, int64_t n_items, size_t smem,
                              unsigned long long* counter, cudaStream_t s);
 // fixed-order sums of the tasks' chunk partials into their outputs (outputs numbered from 0 over the tasks)
 cudaError_t reduce_tasks(const AccumTask* tasks, int32_t n_tasks, int64_t n_out, cudaStream_t s);

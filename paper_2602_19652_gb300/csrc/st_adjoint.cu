@@ -73,7 +73,7 @@ __device__ __forceinline__ void rs_reduce(float (&v)[8], int tp, unsigned wm) {
 // per path, folds its subtile's share of the position gradients into registers (the derivative of
 // the path length and of the lobe angle are linear in the per-subtile sums C0, C1, Cg), and its
 // share of the reflection sums V into kNV x VR registers after a reduce-scatter over the pair lanes.
-template <int KT, int KIND, int TPL, int EMIT>
+template <int KT, int KIND, int TPL, int EMIT, bool ROWS>
 __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
     k_adjoint(const AccumArgs a, const AdjointArgs j, const Geom g) {
     static_assert(KIND == 1 || KT == 8, "the reduce-scatter of the reflection sums takes 8 bins per thread");
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
 
     const float invKB = 1.0f / (float)KB;
     if (t0 < t1) {
-        if (g.mat_cached) {
+        if (ROWS) {
             const int nm = a.n_mat_tab;
             for (int e = tid; e < nm * KB; e += nthr) {
                 const int mat = e / KB, i = e - mat * KB;
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
         }
         cp_async_wait_all();
         __syncthreads();
-        produce<KT, KIND, 1>(a, g, B0, pdb, pvb, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, j.s, t0 * PT);
+        produce<KT, KIND, 1, 0, ROWS>(a, g, B0, pdb, pvb, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, j.s, t0 * PT);
         chain_counts(pdb, pvb, pcb, psg);
         __syncthreads();
     }
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
         }
         if (tile + 1 < t1) {
             const int nb = (int)((tile + 1 - t0) % 3);
-            produce<KT, KIND, 1>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, j.s,
+            produce<KT, KIND, 1, 0, ROWS>(a, g, Pn, pdb + nb * PT * 12, pvb + nb * PT, mt, reinterpret_cast<const float*>(smem4), mic0, kb, invKB, j.s,
                                  (tile + 1) * PT);
             chain_counts(pdb + nb * PT * 12, pvb + nb * PT, pcb + nb * PT, psg + nb * PT);
         }
@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
             u64 c1r = 0ull, c1i = 0ull;  // diffraction: C1 = sum_kk kk conj(G) T directly
             const float2 ngv = up2(ng);  // -gamma^2 of the two microphones (lobe sums)
             const float* xrow = C.tab + (p * NS + s) * RX;
-            const float* grow = reinterpret_cast<const float*>(smem4) + (KIND == 0 ? C.goff[p] : 0) + s * RX;
+            const float* grow = reinterpret_cast<const float*>(smem4) + (KIND == 0 && ROWS ? C.goff[p] : 0) + s * RX;
+            const float2* trow = reinterpret_cast<const float2*>(C.tab) + p * KB + s;  // (not ROWS)
             // diffraction with the material table read directly: row offset left by the producer in ngp
             const u64* mrow = reinterpret_cast<const u64*>(mt) + s * RL;
             if (KIND == 1 && g.mat_direct) mrow += (int)(uint32_t)ng;
@@ -257,6 +258,7 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
                 // P and P' by Horner's scheme from the top bin (no explicit phasor chain).
                 const u64 nw1i = fmul2(w1i, pk2(-1.0f, -1.0f));
                 auto Eat = [&](int kk) -> u64 {
+                    if (!ROWS) return reinterpret_cast<const u64*>(trow)[kk * NS];
                     return g.mat_direct ? mrow[kk] : pk2(xrow[kk], xrow[kk]);
                 };
                 u64 E = Eat(KT - 1);
@@ -283,11 +285,12 @@ __global__ void __launch_bounds__(256, (KIND == 1 || TPL >= 3) ? 2 : 1)
                 float4 x4, g4;
 #pragma unroll
                 for (int kk = 0; kk < KT; ++kk) {  // specular
-                    if ((kk & 3) == 0) {
+                    if (ROWS && (kk & 3) == 0) {
                         x4 = *reinterpret_cast<const float4*>(xrow + kk);
                         g4 = *reinterpret_cast<const float4*>(grow + kk);
                     }
-                    const float2 t = (kk & 3) == 0   ? make_float2(x4.x, g4.x)  // (log2 X, g)
+                    const float2 t = !ROWS           ? trow[kk * NS]  // (log2 X, g)
+                                     : (kk & 3) == 0 ? make_float2(x4.x, g4.x)
                                      : (kk & 3) == 1 ? make_float2(x4.y, g4.y)
                                      : (kk & 3) == 2 ? make_float2(x4.z, g4.z)
                                                      : make_float2(x4.w, g4.w);
@@ -673,12 +676,12 @@ __global__ void __launch_bounds__(128) k_pos_reduce(const float* mic_parts, int 
     }
 }
 
-template <int KT, int KIND, int TPL, int EMIT = 0>
+template <int KT, int KIND, int TPL, int EMIT, bool ROWS>
 cudaError_t launch_adjoint(const AccumArgs& a, const AdjointArgs& j, const Geom& g, cudaStream_t s) {
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_adjoint<KT, KIND, TPL, EMIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             200 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(k_adjoint<KT, KIND, TPL, EMIT, ROWS>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
@@ -686,8 +689,14 @@ cudaError_t launch_adjoint(const AccumArgs& a, const AdjointArgs& j, const Geom&
     const size_t smem =
         g.smem + (EMIT ? (size_t)3 * g.PT * 12 * 4 + 16 : 0) + (KIND == 0 ? (size_t)3 * g.PT * (16 + 4) + 16 : 0);
     note_launch();
-    k_adjoint<KT, KIND, TPL, EMIT><<<grid, g.TP * g.NS, smem, s>>>(a, j, g);
+    k_adjoint<KT, KIND, TPL, EMIT, ROWS><<<grid, g.TP * g.NS, smem, s>>>(a, j, g);
     return cudaGetLastError();
+}
+
+template <int KT, int KIND, int TPL, int EMIT = 0>
+cudaError_t launch_adjoint(const AccumArgs& a, const AdjointArgs& j, const Geom& g, cudaStream_t s) {
+    return g.mat_cached ? launch_adjoint<KT, KIND, TPL, EMIT, true>(a, j, g, s)
+                        : launch_adjoint<KT, KIND, TPL, EMIT, false>(a, j, g, s);
 }
 
 }  // namespace
@@ -720,7 +729,7 @@ acc::Geom adjoint_geom(int M, int F, int n_mat, int mat_direct, int tp_max, int 
     const size_t per_path = adjoint_per_path(g);
     const size_t per_tile = 2 * per_path + 3 * 52;
     const size_t fixed = (g.mat_cached ? g.mat_bytes : 0) + 16 + 64 + 512;
-    const size_t budget = 108 * 1024;
+    const size_t budget = (g.mat_cached ? 108 : 100) * 1024;  // (the rest of L1 for tables that are not in shared memory)
     g.PT = (int)std::max<size_t>(1, std::min<size_t>(8, budget > fixed ? (budget - fixed) / per_tile : 1));
     g.buf_bytes = (per_path * g.PT + 255) & ~size_t(255);
     g.smem = adjoint_smem(g);

@@ -153,12 +153,17 @@ struct BatchState {
     int64_t Q_total = 0;                  // per-microphone visibility queries a bounce, at most
     DevBuf narrow_partial;  // chunk partials of the jobs accumulated on their own, one slice per branch
     size_t narrow_slice = 0;  // bytes of one branch's slice
-    // persistent accumulation: one task per (job, path kind) -- the specular tasks, then the diffraction ones
-    // -- their chunk partials, the work-item counter, item counts and the largest tile's shared memory
+    // persistent accumulation: one task per (job, path kind) -- the specular tasks, then the diffraction ones, of either
+    // first those whose tiles hold the material tables -- their chunk partials, a work-item counter per launch; per launch
+    // its tasks, items and the largest tile's shared memory
     std::vector<int32_t> narrow_jobs;  // jobs accumulated on their own (one microphone pair, or receiver tables)
     DevBuf tasks, part_all, qctr;
-    int32_t n_tasks_spec = 0, n_tasks_diff = 0;
-    int64_t items_spec = 0, items_diff = 0, n_out = 0;
+    struct Queue {
+        int32_t n = 0;
+        int64_t items = 0;
+        size_t smem = 0;
+    } queue[4];                        // specular with rows, specular without, diffraction with, without
+    int64_t n_out = 0;
     // diffraction on the tensor cores (jobs with diff_mma): their tasks follow the diffraction ones in the table;
     // the compacted candidates are sorted by (job, material) and mat_off holds each such job's groups
     int32_t n_tasks_mma = 0;
@@ -166,7 +171,6 @@ struct BatchState {
     bool any_mma = false;
     bool any_table_order = false;  // some job's diffraction paths go in emitter-table row order (its table)
     DevBuf mat_off, mat_scr;
-    size_t smem_spec = 0, smem_diff = 0;
     PathList spec, diff;
     int64_t N_total = 0, R_total = 0, K_total = 0, M_total = 0, MF_total = 0;
     cudaStream_t main = nullptr;     // the batch runs here (capturable even when the context's stream is
@@ -1992,7 +1996,8 @@ AccumArgs batch_accum_args(BatchState& B, const st_job* jobs, int j, int kind, c
 cudaError_t batch_tasks(st_ctx* c, BatchState& B, const st_job* jobs, const st_sim_params& p, const st_tune& tn,
                         cudaStream_t s) {
     (void)c;
-    std::vector<AccumTask> spec, diff, mma;
+    std::vector<AccumTask> cls[5];  // those of B.queue, then the tensor-core ones
+    auto add = [&](const AccumTask& t) { cls[2 * t.a.kind + (t.g.mat_cached ? 0 : 1)].push_back(t); };
     B.narrow_jobs.clear();
     for (int j = 0; j < B.n_jobs; ++j) {
         const JobDev& jd = B.jobs[j];
@@ -2005,49 +2010,48 @@ cudaError_t batch_tasks(st_ctx* c, BatchState& B, const st_job* jobs, const st_s
         if (jd.N > 0) {
             AccumTask t{};
             accum_task(batch_accum_args(B, jobs, j, 0, p, tn), out, &t);
-            spec.push_back(t);
+            add(t);
         }
         if (jd.K > 0 && jd.diff_mma) {
             AccumTask t{};
             diffraction_mma_task(batch_accum_args(B, jobs, j, 1, p, tn), ptr<uint32_t>(B.mat_off) + (size_t)j * kMatStride,
                                  out + MF, &t);
-            mma.push_back(t);
+            cls[4].push_back(t);
         } else if (jd.K > 0) {
             AccumTask t{};
             accum_task(batch_accum_args(B, jobs, j, 1, p, tn), out + MF, &t);
-            diff.push_back(t);
+            add(t);
         }
     }
-    B.n_tasks_spec = (int32_t)spec.size();
-    B.n_tasks_diff = (int32_t)diff.size();
-    B.n_tasks_mma = (int32_t)mma.size();
-    std::vector<AccumTask> all(spec);
-    all.insert(all.end(), diff.begin(), diff.end());
-    all.insert(all.end(), mma.begin(), mma.end());
+    std::vector<AccumTask> all;
     size_t part = 0;
     int64_t out0 = 0;
-    B.items_spec = B.items_diff = B.items_mma = 0;
-    B.smem_spec = B.smem_diff = 0;
-    size_t smem_mma = 0;
-    for (size_t i = 0; i < all.size(); ++i) {
-        AccumTask& t = all[i];
-        const int cls = i < spec.size() ? 0 : (i < spec.size() + diff.size() ? 1 : 2);
-        int64_t& items = cls == 0 ? B.items_spec : (cls == 1 ? B.items_diff : B.items_mma);
-        size_t& sm = cls == 0 ? B.smem_spec : (cls == 1 ? B.smem_diff : smem_mma);
-        t.item0 = items;
-        items += (int64_t)t.g.n_mb * t.g.n_bb * t.a.n_chunks;
-        sm = std::max(sm, t.g.smem);
-        t.out0 = out0;
-        out0 += (int64_t)t.a.M * t.a.F;
-        t.a.partial = reinterpret_cast<float2*>((size_t)part);  // offset for now
-        part += (size_t)t.a.n_chunks * t.a.M * t.a.F * 8;
+    for (int q = 0; q < 5; ++q) {
+        BatchState::Queue Q;
+        Q.n = (int32_t)cls[q].size();
+        for (AccumTask& t : cls[q]) {
+            t.item0 = Q.items;
+            Q.items += (int64_t)t.g.n_mb * t.g.n_bb * t.a.n_chunks;
+            Q.smem = std::max(Q.smem, t.g.smem);
+            t.out0 = out0;
+            out0 += (int64_t)t.a.M * t.a.F;
+            t.a.partial = reinterpret_cast<float2*>((size_t)part);  // offset for now
+            part += (size_t)t.a.n_chunks * t.a.M * t.a.F * 8;
+            all.push_back(t);
+        }
+        if (q < 4) {
+            B.queue[q] = Q;
+        } else {
+            B.n_tasks_mma = Q.n;
+            B.items_mma = Q.items;
+        }
     }
     B.n_out = out0;
     cudaError_t e;
     if ((e = grow(B.part_all, std::max<size_t>(part, 256))) != cudaSuccess) return e;
     for (auto& t : all) t.a.partial = reinterpret_cast<float2*>(static_cast<char*>(B.part_all.p) + (size_t)t.a.partial);
     if ((e = grow(B.tasks, std::max<size_t>(all.size(), 1) * sizeof(AccumTask))) != cudaSuccess) return e;
-    if ((e = grow(B.qctr, 16)) != cudaSuccess) return e;
+    if ((e = grow(B.qctr, 4 * sizeof(unsigned long long))) != cudaSuccess) return e;
     if (!all.empty() &&
         (e = cudaMemcpyAsync(B.tasks.p, all.data(), all.size() * sizeof(AccumTask), cudaMemcpyHostToDevice, s)) !=
             cudaSuccess)
@@ -2182,9 +2186,9 @@ cudaError_t batch_issue(st_ctx* c, BatchState& B, const st_job* jobs, const st_s
     if (spec || B.K_total > 0)
         CB(batch_ranges(a, ptr<uint32_t>(B.sscan), cnt + 2, ptr<uint32_t>(B.sscan) + Koff, cnt + 3, s));
     if (direct) CB(batch_direct_accum(a, s));
-    {  // every job's accumulation: two persistent launches over (job, tile) items, one reduction; the jobs
-       // accumulated on their own on branches beside them (job i on branch i mod the branch count, each
-       // branch with its own slice of partial spectra), joined at the end
+    {  // every job's accumulation: persistent launches over (job, tile) items (per path kind and table layout), one
+       // reduction; the jobs accumulated on their own on branches beside them (job i on branch i mod the branch count,
+       // each branch with its own slice of partial spectra), joined at the end
         const int nbr = B.overlap && B.narrow_jobs.size() > 1 ? (int)std::min<size_t>(4, B.narrow_jobs.size()) : 0;
         if (nbr > 0) {
             CB(cudaEventRecord(B.br_fork, s));
@@ -2217,13 +2221,15 @@ cudaError_t batch_issue(st_ctx* c, BatchState& B, const st_job* jobs, const st_s
         cudaError_t eq = cudaSuccess;
         auto queue = [&]() -> cudaError_t {
             cudaError_t e;
-            if (spec) CB(accumulate_queue(0, tk, B.n_tasks_spec, B.items_spec, B.smem_spec, qc, s));
-            if (B.K_total > 0)
-                CB(accumulate_queue(1, tk + B.n_tasks_spec, B.n_tasks_diff, B.items_diff, B.smem_diff, qc + 1, s));
-            if (B.K_total > 0)
-                CB(accumulate_diffraction_mma_queue(tk + B.n_tasks_spec + B.n_tasks_diff, B.n_tasks_mma, B.items_mma, s));
-            if (spec || B.K_total > 0)
-                CB(reduce_tasks(tk, B.n_tasks_spec + B.n_tasks_diff + B.n_tasks_mma, B.n_out, s));
+            int32_t at = 0;
+            for (int q = 0; q < 4; ++q) {
+                const BatchState::Queue& Q = B.queue[q];
+                if (q < 2 ? spec : B.K_total > 0)
+                    CB(accumulate_queue(q / 2, q % 2 == 0, tk + at, Q.n, Q.items, Q.smem, qc + q, s));
+                at += Q.n;
+            }
+            if (B.K_total > 0) CB(accumulate_diffraction_mma_queue(tk + at, B.n_tasks_mma, B.items_mma, s));
+            if (spec || B.K_total > 0) CB(reduce_tasks(tk, at + B.n_tasks_mma, B.n_out, s));
             return cudaSuccess;
         };
         const cudaError_t es = solo();  // (issued first: the branches start beside the queue launches)

@@ -384,9 +384,10 @@ cudaError_t reduce_partials(const float2* partial, int32_t n_chunks, int64_t MF,
 int32_t accum_chunks(const AccumArgs& a, int64_t n_paths, bool queued = false);
 // Few frequency bins, omni receivers, three microphones or more (st_accum_few.cu).  Where the line lies: the general
 // accumulator shares a path's factors and anchors between 16 pairs and 16 subtiles and wins when it has that many
-// (specular accumulation of 104k paths, few-bin kernel / general, ms: 32 x 48 0.15 / 0.25, 32 x 96 0.22 / 0.24, 32 x 120
-// 0.29 / 0.24, 64 x 48 0.27 / 0.31, 64 x 64 0.39 / 0.28, 17 x 96 0.16 / 0.21, 17 x 128 0.22 / 0.21, 10 x 331 0.31 /
-// 0.34, 10 x 512 0.61 / 0.40, 6 x 512 0.29 / 0.39, 3 x 331 0.14 / 0.39, 3 x 1024 0.56 / 1.47).
+// (specular accumulation of 104k paths, few-bin kernel / general, ms: 32 x 14 0.08 / 0.17, 32 x 48 0.15 / 0.20, 32 x 120
+// 0.30 / 0.23, 64 x 64 0.38 / 0.27, 17 x 96 0.16 / 0.18, 17 x 128 0.22 / 0.20, 10 x 512 0.60 / 0.36, 6 x 512 0.29 /
+// 0.33, 3 x 331 0.14 / 0.22).  The line was drawn before the general tile's bins went in rows; close to it that tile
+// is now the faster one by up to a fifth (32 x 96 0.22 / 0.21, 64 x 48 0.27 / 0.26, 10 x 331 0.31 / 0.25).
 inline bool few_accum(int32_t M, int32_t F) { return M > 2 && (int64_t)M * F <= 3400 && (F <= 96 || M <= 10); }
 // Its shared memory in bytes for the caller's smem_kb (0: none): three CTAs an SM, as its registers allow, so a larger budget
 // only takes one away (10 microphones x 330 bins: 72 KB 0.50 ms a call, 108 KB 0.55, 128 KB 0.61).
