@@ -650,11 +650,13 @@ inline Geom make_geom(int M, int F, int KT, int n_mat, int tp_max = 8, size_t bu
     g.n_mb = (M + g.MP - 1) / g.MP;
     g.n_bb = (F + g.KB - 1) / g.KB;
     const size_t mat_bytes = (size_t)2 * n_mat * g.KB * 4;  // two floats or one packed pair per (material, bin)
-    // Tables up to 48 KB (with a smaller budget less, with 24 KB as the least) are held in shared memory, in the adjoint up to
-    // 24: its paths need more room.  200k rays x 3: 3 microphones x 1500 bins of 4 materials (48 KB) 1.60 ms with the tables in
-    // L1, 0.94 so; 8 x 512 of 12 (48 KB) 0.84 / 0.38; but 32 x 512 of 32 (64 KB) 0.95 / 1.04.  Beyond it 6 x 2048 of 12
-    // materials takes 2.7 ms in this layout and took 3.2 in rows.
-    const size_t mat_most = balance ? std::max<size_t>(24 * 1024, std::min<size_t>(48 * 1024, budget * 9 / 20)) : 24 * 1024;
+    // Tables up to 24 KB are held in shared memory, and up to 48 KB (less with a smaller budget) in the forward of omni receivers
+    // with at most 20 materials: the adjoint's paths and receivers' bands need the room, and many materials' tables of few
+    // bins are loaded for few paths each.  200k rays x 3: 3 microphones x 1500 bins of 4 materials (48 KB) 1.60 ms with the
+    // tables in L1, 0.93 so; 8 x 512 of 12 (48 KB) 0.85 / 0.36; but 32 x 512 of 32 (64 KB) 0.95 / 1.04, and with 60 materials,
+    // receiver tables and 3 x 90 bins 0.26 / 0.32.
+    const bool roomy = balance && dir_nb == 0 && n_mat <= 20;
+    const size_t mat_most = std::max<size_t>(24 * 1024, roomy ? std::min<size_t>(48 * 1024, budget * 9 / 20) : 0);
     g.mat_cached = mat_bytes <= mat_most ? 1 : 0;
     g.mat_direct = (mat_direct && g.mat_cached) ? 1 : 0;
     // (two CTAs to an SM with tables read from L2 through L1: 4 KB a CTA less leave L1 twice as large)
