@@ -1925,10 +1925,11 @@ void batch_release(BatchState& B) {
 // microphone pair (the narrow accumulator is several times faster for them), few bins, receiver directivity tables
 // (the tile's per-microphone band tables), and jobs of a million paths or more, which fill the GPU alone
 // with their full chunk count (in the queue they would take a fraction of it).
-// Where the queue is the better one for few bins: six microphones or more with half to all of the 512 bins that its tile
-// holds (64 poses of 10k rays x 3, on their own / in the queue, ms: 6 x 500 5.12 / 4.60, 8 x 400 5.01 / 4.61, 6 x 350 4.64 /
-// 4.53, 10 x 340 5.05 / 5.05; but 4 x 400 4.26 / 4.14 beside 4 x 800 5.34 / 5.94, 10 x 150 4.43 / 4.97, 3 x 128 3.64 / 4.04).
-static bool few_alone(int32_t M, int32_t F) { return few_accum(M, F) && !(M >= 6 && F > 256 && F <= 512); }
+// Where the queue is the better one for few bins: six to eight microphones with three quarters to all of the 512 bins that
+// its tile holds (64 and 8 poses of 10k rays x 3, on their own / in the queue, ms: 6 x 500 5.10 / 4.56 and 0.87 / 0.80, 8 x 400
+// 5.00 / 4.56 and 0.86 / 0.81; but 6 x 350 4.63 / 4.49 and 0.81 / 0.82, 10 x 340 5.04 / 5.04 and 0.87 / 0.89, 4 x 400 4.26 / 4.14
+// beside 4 x 800 5.34 / 5.94, 10 x 150 4.43 / 4.97).
+static bool few_alone(int32_t M, int32_t F) { return few_accum(M, F) && !(M >= 6 && F > 384 && F <= 512); }
 static bool big_job(const JobDev& d) { return d.N * (int64_t)d.B >= (1 << 20) || d.K >= (1 << 20); }
 static bool solo_accum(const JobDev& d) {
     return narrow_accum(d.M) || few_alone(d.M, d.F) || d.mic_tab != nullptr || big_job(d);
