@@ -2577,7 +2577,8 @@ st_status st_autotune(st_ctx* c, const st_job* J, const st_sim_params* params, s
     const st_tune saved = c->tune;
     const bool saved_overlap = c->overlap;
     c->overlap = false;  // each stage timed on its own
-    const int rpb[2] = {64, 128};  // (256 traces in blocks of 128)
+    // (the default first; 256 traces in blocks of 128)
+    const int rpb[2] = {128, 64};
     const int tiles[5][2] = {{16, 108}, {8, 108}, {16, 64}, {4, 108}, {16, 128}};
     const int kts[2] = {16, 8};
     const int depths[3] = {0, 48, 24};
@@ -2586,7 +2587,8 @@ st_status st_autotune(st_ctx* c, const st_job* J, const st_sim_params* params, s
     // one parameter at a time, each with the best of the earlier ones: the tracing block size, the accumulator
     // tile (microphone pairs and shared memory), its bins per thread (frequency tile), the traversal stack depth
     // and the lane-refill threshold (rays per warp refill); tracing phases are timed on tracing and diffraction,
-    // the others on the accumulator kernels
+    // the others on the accumulator kernels.  A candidate has to win by 1 %: (16, 108) and (16, 128) tie for a single call, but
+    // a tile of 128 KB leaves a batch's queue one CTA an SM (256 poses: 184 ms with the one, 224 with the other)
     const int n_phase[5] = {2, 5, 2, 3, 4};
     for (int phase = 0; phase < 5; ++phase) {
         const int n_cand = n_phase[phase];
@@ -2619,7 +2621,7 @@ st_status st_autotune(st_ctx* c, const st_job* J, const st_sim_params* params, s
                 const bool tracing = phase == 0 || phase >= 3;
                 if (rep > 0) acc += tracing ? st.ms_trace + st.ms_diffraction : st.ms_accum_kernel;
             }
-            if (acc < winner_ms) {
+            if (acc < 0.99f * winner_ms) {
                 winner_ms = acc;
                 winner = t;
             }
