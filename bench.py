@@ -38,16 +38,16 @@ FLOPS_PER_TERM = 10  # per (path, mic, bin) term: complex rotation (6) + real-by
 # hash of the kernel's sources it was taken on: the bench reports it only while the sources still hash to that
 # value (else null, until the kernel is captured again).  Specular k_accum: captured on 200k rays (7.95 MB read,
 # nothing written, 163,228 visible records) and scaled to the full-size launch by the visible records (816,192:
-# the path list is read once).  k_accum_diff_mma: the full-size diffraction set (21.5 MB read).
-ACCUM_TRAFFIC = {"sources_sha16": "631dcd040505b604", "specular_bytes_per_launch": 39.8e6}
+# the path list is read once).  k_accum_diff_mma: the full-size diffraction set (21.4 MB read).
+ACCUM_TRAFFIC = {"sources_sha16": "4857ae9d7d4ccadb", "specular_bytes_per_launch": 39.8e6}
 ACCUM_SOURCES = ("st_accum.cu", "st_accum_dev.cuh", "st_internal.cuh")
-DIFF_MMA_TRAFFIC = {"sources_sha16": "dea9b9d9213d8056", "bytes_per_launch": 21.5e6}
+DIFF_MMA_TRAFFIC = {"sources_sha16": "813f2a8cc2db8f5a", "bytes_per_launch": 21.4e6}
 DIFF_MMA_SOURCES = ("st_accum_mma.cu", "st_accum_dev.cuh", "st_internal.cuh")
 # k_accum_narrow on the vegetation workload (two launches a step, specular and diffraction): captured on 500k
-# rays (specular 51.43 MB read + 0.16 MB written for 871,268 visible records; diffraction 11.04 MB read for the
+# rays (specular 51.58 MB read + 0.14 MB written for 871,268 visible records; diffraction 11.05 MB read for the
 # full-size set of 222,807 kept samples), the specular launch scaled to the full-size 6,971,043 records (the
-# path list is read once: 412.8 MB), averaged over the step's two launches.
-NARROW_TRAFFIC = {"sources_sha16": "e96e031a1e996f56", "bytes_per_launch": 211.9e6}
+# path list is read once: 413.8 MB), averaged over the step's two launches.
+NARROW_TRAFFIC = {"sources_sha16": "18e725f9395ff7a2", "bytes_per_launch": 212.4e6}
 NARROW_SOURCES = ("st_accum_narrow.cu", "st_accum_dev.cuh", "st_internal.cuh")
 
 
